@@ -14,101 +14,157 @@
 
 #include "dlo_runtime.h"
 #include "dlo_kernels.h"
-#include "dlo_physics.cuh"
+#include "dlo_frames.cuh"
 
 namespace dlo {
 
 // ------------------------------------------------------------------ initial frames adjoint
-// Reverse of the frame construction of dlo_set_state (space-parallel transport, holonomy
-// spread for loops): cotangents of the initial base (t, d1) -> positions. FP64, one thread
-// per rod.
-__device__ __forceinline__ V3<double> ld(float4 a) { return V3<double>{(double)a.x, (double)a.y, (double)a.z}; }
-__device__ __forceinline__ V3<double> unit_d(V3<double> a) { return a / sqrt(dot(a, a)); }
-__device__ __forceinline__ V3<double> adapt_fwd(V3<double> w, V3<double> t) { return unit_d(w - dot(w, t) * t); }
-// reverse of u = adapt(w, t): returns lambda_w, adds lambda_t
-__device__ __forceinline__ V3<double> adapt_rev(V3<double> w, V3<double> t, V3<double> lu, V3<double>& lt) {
-    V3<double> dd = w - dot(w, t) * t;
+__device__ __forceinline__ double warp_sum_d(double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+// reverse of u = adapt(w, t), the unit projection of w normal to t: returns lambda_w, adds lambda_t
+__device__ __forceinline__ D3 adapt_rev(D3 w, D3 t, D3 lu, D3& lt) {
+    D3 dd = w - dot(w, t) * t;
     double n = sqrt(dot(dd, dd));
-    V3<double> u = dd / n;
-    V3<double> ldd = (lu - dot(lu, u) * u) / n;
+    D3 u = dd / n;
+    D3 ldd = (lu - dot(lu, u) * u) / n;
     lt += -dot(w, t) * ldd - dot(ldd, t) * w;
     return ldd - dot(ldd, t) * t;
 }
 // reverse of u = transport(a, b, d): adds lambda_a, lambda_b, returns lambda_d
-__device__ __forceinline__ V3<double> transport_rev(V3<double> A, V3<double> Bv, V3<double> d, V3<double> lu,
-                                                    V3<double>& la, V3<double>& lb) {
+__device__ __forceinline__ D3 transport_rev(D3 A, D3 Bv, D3 d, D3 lu, D3& la, D3& lb) {
     double c = dot(A, Bv);
-    V3<double> k = cross(A, Bv);
-    double kd = dot(k, d), luk = dot(lu, k), opc = 1.0 + c;
-    double lc = dot(lu, d) - kd * luk / (opc * opc);
-    V3<double> lk = cross(d, lu) + (kd / opc) * lu + (luk / opc) * d;
+    D3 k = cross(A, Bv);
+    double kd = dot(k, d), luk = dot(lu, k), q = 1.0 / (1.0 + c);
+    double lc = dot(lu, d) - kd * luk * q * q;
+    D3 lk = cross(d, lu) + (kd * q) * lu + (luk * q) * d;
     la += lc * Bv + cross(Bv, lk);
     lb += lc * A + cross(lk, A);
-    return c * lu + cross(lu, k) + (luk / opc) * k;
+    return c * lu + cross(lu, k) + (luk * q) * k;
 }
 
-__global__ void frames_adjoint_kernel(const RodInfo* rods, int B, const float4* X0, const float4* gtb0,
-                                      const float4* gd1b0, float4* gx0, V3<double>* work) {
-    const int rod = blockIdx.x * blockDim.x + threadIdx.x;
-    if (rod >= B) return;
+// Reverse of the frame construction of dlo_set_state (space-parallel transport, holonomy
+// spread for loops): cotangents of the initial base (t, d1) -> positions.  FP64, one block per
+// rod and one thread per edge.  A transported director is determined by its edge's tangent and
+// its turn about it, and a turn adds to every later director's, so the cotangent that reaches
+// the transport into edge j is W_j (t_j x d_j) with W_j the sum over the edges k >= j of their
+// cotangents' parts along t_k x d_k: a suffix sum instead of a chain, after which every edge's
+// reverse is local.  Bound by the FP64 pipe for large batches and by its latency for small
+// ones; one thread per rod walking its edges (with the frames in device memory) took 1395 us
+// for one rod of 128 vertices and 1795 us for 4096.
+__global__ void __launch_bounds__(kFrameMaxEdges) frames_adjoint_kernel(const RodInfo* rods, const float4* X0,
+                                                                       const float4* gtb0, const float4* gd1b0,
+                                                                       float4* gx0) {
+    __shared__ D3 T[kFrameMaxEdges], A[kFrameMaxEdges], D[kFrameMaxEdges];   // tangents, axes, directors
+    __shared__ Turn wsum[kFrameMaxWarps];
+    __shared__ double red[kFrameMaxWarps];
+    const int rod = blockIdx.x, j = threadIdx.x, lane = j & 31, w = j >> 5;
     const RodInfo R = rods[rod];
-    const int nv = R.nv, ne = R.ne, v0 = R.v0, e0 = R.e0;
-    const bool closed = R.flags & ROD_CLOSED;
-    V3<double>* T = work + 4 * (size_t)v0;          // tangents [ne]
-    V3<double>* Dh = T + nv;                       // uncorrected frames [ne]
-    V3<double>* Lt = Dh + nv;                      // tangent cotangents [ne]
-    V3<double>* Ldh = Lt + nv;                     // cotangents of the uncorrected frames [ne]
-    auto X = [&](int i) { return ld(X0[v0 + i]); };
-    for (int j = 0; j < ne; ++j) T[j] = unit_d(X(j + 1 == nv ? 0 : j + 1) - X(j));
-    V3<double> ax = fabs(T[0].z) < 0.9 ? V3<double>{0.0, 0.0, 1.0} : V3<double>{1.0, 0.0, 0.0};
-    Dh[0] = adapt_fwd(ax, T[0]);
-    for (int j = 1; j < ne; ++j) Dh[j] = adapt_fwd(transport_d(T[j - 1], T[j], Dh[j - 1]), T[j]);
-    double psi = 0.0;
-    V3<double> wl{0, 0, 0}, u{0, 0, 0};
-    if (closed) {
-        wl = transport_d(T[ne - 1], T[0], Dh[ne - 1]);
-        u = adapt_fwd(wl, T[0]);
-        psi = atan2(dot(cross(Dh[0], u), T[0]), dot(Dh[0], u));
+    const int nv = R.nv, ne = R.ne, v0 = R.v0, e0 = R.e0, nw = (int)blockDim.x >> 5;
+    const bool closed = R.flags & ROD_CLOSED, on = j < ne;
+    D3 t{0.0, 0.0, 1.0};
+    double il = 0.0;
+    if (on) {
+        const D3 e = ld(X0[v0 + (j + 1 == nv ? 0 : j + 1)]) - ld(X0[v0 + j]);
+        il = rsqrt(dot(e, e));
+        t = il * e;
     }
-    for (int j = 0; j < ne; ++j) Lt[j] = ld(gtb0[e0 + j]);
-    // cotangents of the uncorrected frames from the (corrected) output frames
-    double lpsi = 0.0;
-    for (int j = 0; j < ne; ++j) {
-        V3<double> l1 = ld(gd1b0[e0 + j]);
-        if (closed) {
-            double phi = -psi * (double)j / (double)ne, cph = cos(phi), sph = sin(phi);
-            Ldh[j] = cph * l1 + sph * cross(l1, T[j]);
-            Lt[j] += sph * cross(Dh[j], l1);
-            double lphi = dot(l1, -sph * Dh[j] + cph * cross(T[j], Dh[j]));
-            lpsi += -(double)j / (double)ne * lphi;
-        } else {
-            Ldh[j] = l1;
+    const D3 d = transported_director(t, false, ne, T, A, wsum);
+    const D3 td = cross(t, d);
+    if (on) D[j] = d;
+    __syncthreads();   // D is complete; A is free and takes the tangents' cotangents below
+    // cotangents of this edge's tangent (lt) and uncorrected director (ld1)
+    D3 lt{0.0, 0.0, 0.0}, ld1 = lt;
+    if (on) {
+        lt = ld(gtb0[e0 + j]);
+        ld1 = ld(gd1b0[e0 + j]);
+    }
+    const D3 a_first = A[0];
+    if (closed) {   // the frames were turned by -psi j / ne, psi the holonomy
+        const Turn z = transport_turn(T[ne - 1], D[ne - 1], T[0], a_first);
+        const double phi = -atan2(z.s, z.c) * (double)j / (double)ne;
+        double lpsi = 0.0;
+        if (on) {
+            const double cph = cos(phi), sph = sin(phi);
+            const D3 l1 = ld1;
+            ld1 = cph * l1 + sph * cross(l1, t);
+            lt += sph * cross(d, l1);
+            lpsi = -(double)j / (double)ne * dot(l1, cph * td - sph * d);
+        }
+        lpsi = warp_sum_d(lpsi);
+        if (lane == 0) red[w] = lpsi;
+        __syncthreads();
+        lpsi = 0.0;
+        for (int k = 0; k < nw; ++k) lpsi += red[k];
+        __syncthreads();
+        // psi is the angle from d_0 to u, the unit projection of the last director carried over
+        if (j == 0 || j == ne - 1) {
+            const D3 t0 = T[0], d0 = a_first;
+            const D3 wl = transport_d(T[ne - 1], t0, D[ne - 1]);
+            const D3 u = unit_d(wl - dot(wl, t0) * t0);
+            const double y = dot(cross(d0, u), t0), x = dot(d0, u), r2 = x * x + y * y;
+            const double ly = lpsi * x / r2, lx = -lpsi * y / r2;
+            D3 lt0{0.0, 0.0, 0.0}, ltl = lt0;
+            const D3 lw = adapt_rev(wl, t0, ly * cross(t0, d0) + lx * d0, lt0);
+            const D3 ldl = transport_rev(T[ne - 1], t0, D[ne - 1], lw, ltl, lt0);
+            if (j == 0) {
+                ld1 += ly * cross(u, t0) + lx * u;
+                lt += lt0 + ly * cross(d0, u);
+            } else {
+                lt += ltl;
+                ld1 += ldl;
+            }
         }
     }
-    if (closed) {
-        double y = dot(cross(Dh[0], u), T[0]), x = dot(Dh[0], u), r2 = x * x + y * y;
-        double ly = lpsi * x / r2, lx = -lpsi * y / r2;
-        V3<double> lu = ly * cross(T[0], Dh[0]) + lx * Dh[0];
-        Ldh[0] += ly * cross(u, T[0]) + lx * u;
-        Lt[0] += ly * cross(Dh[0], u);
-        V3<double> lw = adapt_rev(wl, T[0], lu, Lt[0]);
-        Ldh[ne - 1] += transport_rev(T[ne - 1], T[0], Dh[ne - 1], lw, Lt[ne - 1], Lt[0]);
+    // W_j: suffix sum of the cotangents' parts along t x d
+    double W = on ? dot(ld1, td) : 0.0;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const double p = __shfl_down_sync(0xffffffffu, W, o);
+        if (lane + o < 32) W += p;
     }
-    for (int j = ne - 1; j >= 1; --j) {
-        V3<double> w = transport_d(T[j - 1], T[j], Dh[j - 1]);
-        V3<double> lw = adapt_rev(w, T[j], Ldh[j], Lt[j]);
-        Ldh[j - 1] += transport_rev(T[j - 1], T[j], Dh[j - 1], lw, Lt[j - 1], Lt[j]);
+    if (lane == 0) red[w] = W;
+    __syncthreads();
+    for (int k = nw - 1; k > w; --k) W += red[k];
+    D3 lprev{0.0, 0.0, 0.0};   // cotangent of the previous edge's tangent
+    if (on) {
+        if (j == 0) {
+            // the first director is the projection of a fixed axis; later edges' turns reach it as W_1 t x d
+            adapt_rev(axis_of(t), t, ld1 + (W - dot(ld1, td)) * td, lt);
+        } else {
+            lt -= dot(ld1, t) * d;
+            transport_rev(T[j - 1], t, D[j - 1], W * td, lprev, lt);
+        }
     }
-    adapt_rev(ax, T[0], Ldh[0], Lt[0]);
-    for (int j = 0; j < ne; ++j) {
-        const int j1 = j + 1 == nv ? 0 : j + 1;
-        V3<double> e = X(j1) - X(j);
-        double l = sqrt(dot(e, e));
-        V3<double> t = e / l;
-        V3<double> le = (Lt[j] - dot(Lt[j], t) * t) / l;
-        float4 a0 = gx0[v0 + j], a1 = gx0[v0 + j1];
-        gx0[v0 + j] = make_float4(a0.x - (float)le.x, a0.y - (float)le.y, a0.z - (float)le.z, a0.w);
-        gx0[v0 + j1] = make_float4(a1.x + (float)le.x, a1.y + (float)le.y, a1.z + (float)le.z, a1.w);
+    __syncthreads();
+    if (on && j > 0) A[j - 1] = lprev;   // from edge j to edge j - 1
+    __syncthreads();
+    float lex = 0.f, ley = 0.f, lez = 0.f;
+    if (on) {
+        if (j + 1 < ne) lt += A[j];
+        const D3 le = il * (lt - dot(lt, t) * t);
+        lex = (float)le.x;
+        ley = (float)le.y;
+        lez = (float)le.z;
+    }
+    if (on) D[j] = D3{(double)lex, (double)ley, (double)lez};
+    __syncthreads();
+    if (j < nv) {   // vertex j ends edge j - 1 and starts edge j
+        float4 g = gx0[v0 + j];
+        if (closed && j == 0) {
+            g = make_float4(g.x - lex, g.y - ley, g.z - lez, g.w);
+            const D3 p = D[ne - 1];
+            g = make_float4(g.x + (float)p.x, g.y + (float)p.y, g.z + (float)p.z, g.w);
+        } else {
+            if (j > 0) {
+                const D3 p = D[j - 1];
+                g = make_float4(g.x + (float)p.x, g.y + (float)p.y, g.z + (float)p.z, g.w);
+            }
+            if (on) g = make_float4(g.x - lex, g.y - ley, g.z - lez, g.w);
+        }
+        gx0[v0 + j] = g;
     }
 }
 
@@ -136,9 +192,9 @@ cudaError_t launch_rev(const BwdParams& P, int nv, bool c, int grid, int warps, 
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_frames_adjoint(const RodInfo* rods, int B, const float4* X0, const float4* gtb0,
-                                  const float4* gd1b0, float4* gx0, V3<double>* work, cudaStream_t st) {
-    frames_adjoint_kernel<<<(B + 127) / 128, 128, 0, st>>>(rods, B, X0, gtb0, gd1b0, gx0, work);
+cudaError_t launch_frames_adjoint(const RodInfo* rods, int B, int nv_max, const float4* X0, const float4* gtb0,
+                                  const float4* gd1b0, float4* gx0, cudaStream_t st) {
+    frames_adjoint_kernel<<<B, nv_max, 0, st>>>(rods, X0, gtb0, gd1b0, gx0);
     return cudaGetLastError();
 }
 
@@ -235,7 +291,7 @@ dlo_status bwd_plan(dlo_ctx* c, int force, int K, BwdPlan& out, size_t rec_budge
         out.offset[k] = need;   // each class has its own region: the classes run concurrently
         need += (16 * (size_t)bk.n * (out.r3_rod[k] + out.l2_rod[k] + out.cs_rod[k]) + 255) & ~(size_t)255;
     }
-    out.fixed = (2 * 16 * (size_t)c->Et + 4 * sizeof(V3<double>) * (size_t)c->V + 1024 + 255) & ~(size_t)255;
+    out.fixed = (2 * 16 * (size_t)c->Et + 255) & ~(size_t)255;
     out.bytes = out.fixed + need;
     return DLO_OK;
 }
@@ -366,7 +422,6 @@ extern "C" dlo_status dlo_backward(dlo_ctx* c, const float* dL_dx_T, const float
     char* p = reinterpret_cast<char*>(c->bw_mem);
     float4* gtb0 = reinterpret_cast<float4*>(p);
     float4* gd1b0 = gtb0 + c->Et;
-    V3<double>* work = reinterpret_cast<V3<double>*>(gd1b0 + c->Et);
     char* region = p + plan.fixed;
     const BwdParams common = backward_common(c, force, dL_dx_T, dL_dv_T, dL_dtheta_T, dL_dactions, dL_dmaterial,
                                              dL_dx0, dL_dv0, dL_dtheta0, gtb0, gd1b0);
@@ -387,10 +442,9 @@ extern "C" dlo_status dlo_backward(dlo_ctx* c, const float* dL_dx_T, const float
         if (je != cudaSuccess) return cuda_err(c, je, "join");
     }
     if (c->rec_from_set && dL_dx0) {
-        frames_adjoint_kernel<<<(c->B + 127) / 128, 128, 0, c->stream>>>(c->d_rods, c->B, c->ck.X, gtb0, gd1b0,
-                                                                        reinterpret_cast<float4*>(dL_dx0), work);
+        cudaError_t e = launch_frames_adjoint(c->d_rods, c->B, c->buckets.back().nv_max, c->ck.X, gtb0, gd1b0,
+                                              reinterpret_cast<float4*>(dL_dx0), c->stream);
         c->launches++;
-        cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_err(c, e, "frames adjoint launch");
     }
     return check_status(c);

@@ -94,6 +94,11 @@ struct InitParams {
     const float* GP0;        // [B][2][12] initial gripper poses
     int rest_mode;           // 1: compute the rest twist from xin into rest[].z only
 };
-cudaError_t launch_init(const InitParams& P, cudaStream_t st);
+// nv_max: the largest size class of the batch (threads per block)
+cudaError_t launch_init(const InitParams& P, int nv_max, cudaStream_t st);
+// Reverse of launch_init's frame construction: from the cotangents of the base tangents and
+// directors, adds the cotangents of the positions to gx0.
+cudaError_t launch_frames_adjoint(const RodInfo* rods, int B, int nv_max, const float4* X0, const float4* gtb0,
+                                  const float4* gd1b0, float4* gx0, cudaStream_t st);
 
 }  // namespace dlo

@@ -23,10 +23,6 @@
 #include "dlo_runtime.h"
 #include "dlo_vec.cuh"
 
-namespace dlo {
-cudaError_t launch_frames_adjoint(const RodInfo* rods, int B, const float4* X0, const float4* gtb0,
-                                  const float4* gd1b0, float4* gx0, V3<double>* work, cudaStream_t st);
-}
 using namespace dlo;
 
 // 256 MiB: enough for the 4096-rod x 128-vertex workload at 50-frame checkpoints (the
@@ -87,9 +83,10 @@ extern "C" dlo_status dlo_backward_noalloc(dlo_ctx* c, const float* dL_dx_T, con
     if (st != DLO_OK) return st;
 
     // fixed part: cotangents of the initial reference frames (gtb0, gd1b0) and, when the
-    // gradient must reach x0 through the frame initialisation, its FP64 work array
+    // gradient must reach x0 through the frame initialisation, the 96 bytes per vertex that
+    // the interface's capacity rule counts
     const bool frames_adj = c->rec_from_set && dL_dx0;
-    const size_t fixed_raw = 2 * 16 * (size_t)c->Et + (frames_adj ? 4 * sizeof(V3<double>) * (size_t)c->V : 0);
+    const size_t fixed_raw = 2 * 16 * (size_t)c->Et + (frames_adj ? 96 * (size_t)c->V : 0);
     const size_t fixed = (fixed_raw + 255) & ~(size_t)255;
     const int force = c->rec_nsub > 0 ? c->rec_nsub : 0;
     BwdPlan plan;
@@ -99,7 +96,6 @@ extern "C" dlo_status dlo_backward_noalloc(dlo_ctx* c, const float* dL_dx_T, con
     const int K = c->ck_every, F = c->rec_frames;
     float4* gtb0 = reinterpret_cast<float4*>(base);
     float4* gd1b0 = gtb0 + c->Et;
-    V3<double>* work = reinterpret_cast<V3<double>*>(gd1b0 + c->Et);
     char* region = base + fixed;
     const BwdParams common = backward_common(c, force, dL_dx_T, dL_dv_T, dL_dtheta_T, dL_dactions, dL_dmaterial,
                                              dL_dx0, dL_dv0, dL_dtheta0, gtb0, gd1b0);
@@ -140,8 +136,8 @@ extern "C" dlo_status dlo_backward_noalloc(dlo_ctx* c, const float* dL_dx_T, con
         }
     }
     if (frames_adj) {
-        cudaError_t e = launch_frames_adjoint(c->d_rods, c->B, c->ck.X, gtb0, gd1b0,
-                                              reinterpret_cast<float4*>(dL_dx0), work, c->stream);
+        cudaError_t e = launch_frames_adjoint(c->d_rods, c->B, c->buckets.back().nv_max, c->ck.X, gtb0, gd1b0,
+                                              reinterpret_cast<float4*>(dL_dx0), c->stream);
         c->launches++;
         if (e != cudaSuccess) return cuda_err(c, e, "frames adjoint launch");
     }

@@ -1126,11 +1126,6 @@ __global__ void prb_out(const RodInfo* rods, long long V, long long Et, int B, P
 
 using namespace dlo;
 
-namespace dlo {
-cudaError_t launch_frames_adjoint(const RodInfo* rods, int B, const float4* X0, const float4* gtb0,
-                                  const float4* gd1b0, float4* gx0, V3<double>* work, cudaStream_t st);
-}
-
 // Checkpoint c of the ring from the state arrays S (the layout dlo_step writes).
 static cudaError_t plain_checkpoint(dlo_ctx* c, const PlainState& S, long long cidx) {
     cudaStream_t sm = c->stream;
@@ -1229,7 +1224,7 @@ extern "C" dlo_status dlo_backward_plain(dlo_ctx* c, const float* dL_dx_T, const
     const size_t rec_f4 = (size_t)nsub_max * (5 * nV + 2 * nE + (size_t)n_iter * (nE + nV) + 2 * (size_t)Pn);
     const size_t f4 = 3 * nV + 2 * nE + rec_f4 + 7 * nV + 3 * nE;
     const size_t bytes = 16 * f4 + sizeof(double) * 5 * B + sizeof(float) * (size_t)B * (12 + 12 + 36 + 72 + 24 + 24) +
-                         2 * 16 * nE + 4 * sizeof(V3<double>) * nV + 4096;
+                         2 * 16 * nE + 4096;
     if (bytes > c->bw_bytes) {
         dev_free(c, c->bw_mem);
         c->bw_mem = dev_alloc(c, bytes);
@@ -1279,9 +1274,6 @@ extern "C" dlo_status dlo_backward_plain(dlo_ctx* c, const float* dL_dx_T, const
     A.PM = A.PA + 36 * B;
     A.GPF = A.PM + 72 * B;
     float* GPW = A.GPF + 24 * B;   // the working state's gripper poses
-    m = reinterpret_cast<char*>(GPW + 24 * B);
-    m = reinterpret_cast<char*>(((uintptr_t)m + 255) & ~(uintptr_t)255);
-    V3<double>* work = reinterpret_cast<V3<double>*>(m);
     PlainState SW = S;
     SW.GP = GPW;
     cudaStream_t sm = c->stream;
@@ -1349,8 +1341,8 @@ extern "C" dlo_status dlo_backward_plain(dlo_ctx* c, const float* dL_dx_T, const
                                          reinterpret_cast<float4*>(dL_dv0), dL_dtheta0, gtb0, gd1b0, dL_dmaterial);
     c->launches++;
     if (c->rec_from_set && dL_dx0) {
-        cudaError_t e = launch_frames_adjoint(c->d_rods, B, c->ck.X, gtb0, gd1b0, reinterpret_cast<float4*>(dL_dx0),
-                                              work, sm);
+        cudaError_t e = launch_frames_adjoint(c->d_rods, B, c->buckets.back().nv_max, c->ck.X, gtb0, gd1b0,
+                                              reinterpret_cast<float4*>(dL_dx0), sm);
         c->launches++;
         if (e != cudaSuccess) return cuda_err(c, e, "frames adjoint launch");
     }

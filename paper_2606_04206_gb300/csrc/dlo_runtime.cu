@@ -187,10 +187,10 @@ dlo_status runtime_allocate(dlo_ctx* c, const std::vector<RodInfo>& rods, const 
     P.S = c->S;
     P.GP0 = c->d_gp0;
     P.rest_mode = 1;
-    st = cuda_err(c, launch_init(P, c->stream), "rest init");
+    st = cuda_err(c, launch_init(P, c->buckets.back().nv_max, c->stream), "rest init");
     if (st != DLO_OK) return st;
     P.rest_mode = 0;
-    st = cuda_err(c, launch_init(P, c->stream), "state init");
+    st = cuda_err(c, launch_init(P, c->buckets.back().nv_max, c->stream), "state init");
     c->launches += 2;
     if (st == DLO_OK && c->opt.warps_per_cta == 0) {
         // measured autotune of rods per CTA; then the rest state is set again (positions
@@ -201,7 +201,7 @@ dlo_status runtime_allocate(dlo_ctx* c, const std::vector<RodInfo>& rods, const 
                                              c->stream), "rest positions");
         if (st == DLO_OK)
             st = cuda_err(c, cudaMemsetAsync(c->d_status, 0, sizeof(unsigned) * c->B, c->stream), "status reset");
-        if (st == DLO_OK) st = cuda_err(c, launch_init(P, c->stream), "state init");
+        if (st == DLO_OK) st = cuda_err(c, launch_init(P, c->buckets.back().nv_max, c->stream), "state init");
         c->launches++;
     }
     c->from_set_state = true;

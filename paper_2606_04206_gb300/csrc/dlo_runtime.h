@@ -87,7 +87,7 @@ struct BwdPlan {
     // checkpoints) and of the carried cotangent state (CS); the class's region in the workspace
     std::vector<int> nsmax, C;
     std::vector<size_t> r3_rod, l2_rod, cs_rod, offset;
-    size_t fixed = 0;    // initial-frame cotangents and the frame-initialisation adjoint's work
+    size_t fixed = 0;    // initial-frame cotangents
     size_t bytes = 0;    // everything, for all rods at once
 };
 // the stream of size class k, and the fork / join around work issued on those streams
