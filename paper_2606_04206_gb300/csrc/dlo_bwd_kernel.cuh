@@ -27,6 +27,7 @@ namespace dlo {
 // vertices take at most 62.5 KB of shared memory each, so three fit an SM: 384 threads at 168
 // registers.  Larger rods fit two per SM (one at 256 vertices), and keep 255 registers.
 __host__ __device__ constexpr int rev_max_threads(int NV) { return NV <= 128 ? 384 : 256; }
+__host__ __device__ constexpr int rev_threads(int NV) { return NV < 128 ? NV : 128; }
 
 __host__ __device__ constexpr size_t bwd_smem_bytes(int NV, bool contact) {
     return rod_smem_bytes(NV, contact) + (size_t)(10 * NV + 20) * 16;
@@ -767,7 +768,6 @@ __global__ void __launch_bounds__(kFwdMaxThreads) rec_kernel(BwdParams P) {
             for (int i = g.tid; i < R.nv; i += TPR) {
                 const float4 x = P.ck.X[oV + R.v0 + i];
                 s.X0[i] = x;
-                s.X[i] = x;
                 s.V[i] = P.ck.Vl[oV + R.v0 + i];
                 s.HG[i] = P.ck.HG[oV + R.v0 + i];
             }
@@ -781,7 +781,6 @@ __global__ void __launch_bounds__(kFwdMaxThreads) rec_kernel(BwdParams P) {
             for (int i = g.tid; i < R.nv; i += TPR) {
                 const float4 x = e[i];
                 s.X0[i] = x;
-                s.X[i] = x;
                 s.V[i] = e[NV + i];
                 s.HG[i] = e[2 * NV + i];
             }
@@ -791,6 +790,7 @@ __global__ void __launch_bounds__(kFwdMaxThreads) rec_kernel(BwdParams P) {
             }
             if (g.tid < 24) s.fp[g.tid] = reinterpret_cast<const float*>(e + 5 * NV)[g.tid];
         }
+        const Own own = own_of(P.KIN, P.ES, R, g.tid);
         g.sync();
         bool ovf = false;
         if (P.mode == 0) {
@@ -802,8 +802,8 @@ __global__ void __launch_bounds__(kFwdMaxThreads) rec_kernel(BwdParams P) {
                 if (f + 1 == f1) break;   // the segment's last frame only needs its start state
                 if (g.tid < 12) s.act[g.tid] = P.actions[((size_t)f * P.B + rod) * 12 + g.tid];
                 g.sync();
-                run_frame<NV, CONTACT, TPR, true>(sc, P.KIN, P.ES, R, s, g, nsub, h, ovf,
-                                                  [](int) -> const Rec* { return nullptr; });
+                run_frame<NV, CONTACT, TPR>(sc, P.KIN, R, own, s, g, nsub, h, ovf,
+                                            [](int) { return Rec<NV, false>{nullptr, 0}; });
             }
         } else {
             float4* R3 = P.R3 + (size_t)k * P.r3_rod;
@@ -812,17 +812,11 @@ __global__ void __launch_bounds__(kFwdMaxThreads) rec_kernel(BwdParams P) {
                 if (g.tid < 24) reinterpret_cast<float*>(fb)[g.tid] = s.fp[g.tid];
                 if (g.tid < 12) s.act[g.tid] = P.actions[((size_t)f * P.B + rod) * 12 + g.tid];
                 g.sync();
-                Rec recs;
-                const int np = run_frame<NV, CONTACT, TPR, true>(
-                    sc, P.KIN, P.ES, R, s, g, nsub, h, ovf, [&](int sb) -> const Rec* {
-                        float4* e3 = fb + kFrameHead + NV + (size_t)sb * SR;
-                        save_state<NV, CONTACT, TPR>(e3, R, g, s);
-                        recs = Rec{e3 + 5 * NV, e3 + 6 * NV, e3 + 7 * NV, e3 + (size_t)(7 + n_iter) * NV,
-                                   e3 + (size_t)(7 + 2 * n_iter) * NV,
-                                   e3 + (size_t)(7 + 2 * n_iter + kPairsPerVertex) * NV, NV};
-                        g.sync();   // the substep overwrites what was just stored
-                        return &recs;
-                    });
+                const int np = run_frame<NV, CONTACT, TPR>(sc, P.KIN, R, own, s, g, nsub, h, ovf, [&](int sb) {
+                    float4* e3 = fb + kFrameHead + NV + (size_t)sb * SR;
+                    save_state<NV, CONTACT, TPR>(e3, R, g, s);   // each thread its own vertex and edge
+                    return Rec<NV, true>{e3, n_iter};
+                });
                 if (CONTACT) {
                     uint32_t* pl = reinterpret_cast<uint32_t*>(fb + kFrameHead);
                     for (int p = g.tid; p < np; p += TPR) pl[p] = s.pairs[p];
@@ -843,7 +837,7 @@ __global__ void __launch_bounds__(kFwdMaxThreads) rec_kernel(BwdParams P) {
 // go to CS, or to the outputs on the last chunk (fa = 0).
 template <int NV, bool CONTACT>
 __global__ void __launch_bounds__(rev_max_threads(NV)) rev_kernel(BwdParams P) {
-    constexpr int TPR = threads_per_rod(NV);
+    constexpr int TPR = rev_threads(NV);
     extern __shared__ float4 dyn_smem[];
     const int rs = threadIdx.x / TPR;
     float4* base = dyn_smem + rs * (bwd_smem_bytes(NV, CONTACT) / 16);
@@ -1025,7 +1019,7 @@ __global__ void __launch_bounds__(rev_max_threads(NV)) rev_kernel(BwdParams P) {
 // ------------------------------------------------------------------ launch helpers
 template <int NV, bool C>
 static int rev_occ_t(int rpc) {
-    if (rpc < 1 || rpc * threads_per_rod(NV) > rev_max_threads(NV)) return 0;
+    if (rpc < 1 || rpc * rev_threads(NV) > rev_max_threads(NV)) return 0;
     size_t smem = bwd_smem_bytes(NV, C) * rpc;
     auto k = rev_kernel<NV, C>;
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
@@ -1033,7 +1027,7 @@ static int rev_occ_t(int rpc) {
         return 0;
     }
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, threads_per_rod(NV) * rpc, smem) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, rev_threads(NV) * rpc, smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
@@ -1045,7 +1039,7 @@ static cudaError_t launch_rev_t(const BwdParams& P, int grid, int rpc, cudaStrea
     auto k = rev_kernel<NV, C>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k<<<grid, threads_per_rod(NV) * rpc, smem, st>>>(P);
+    k<<<grid, rev_threads(NV) * rpc, smem, st>>>(P);
     return cudaGetLastError();
 }
 template <int NV, bool C>

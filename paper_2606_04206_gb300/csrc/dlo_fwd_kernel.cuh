@@ -53,7 +53,6 @@ __global__ void __launch_bounds__(kFwdMaxThreads) fwd_kernel(FwdParams P) {
         const float h = P.scene.dt / (float)nsub;
         for (int i = g.tid; i < R.nv; i += TPR) {
             float4 x = P.S.X[R.v0 + i];
-            s.X[i] = x;
             s.X0[i] = x;
             s.V[i] = P.S.Vl[R.v0 + i];
             s.HG[i] = P.S.HG[R.v0 + i];
@@ -62,6 +61,7 @@ __global__ void __launch_bounds__(kFwdMaxThreads) fwd_kernel(FwdParams P) {
             s.ED[j] = P.S.ED[R.e0 + j];
             s.ET[j] = P.S.ET[R.e0 + j];
         }
+        const Own own = own_of(P.KIN, P.ES, R, g.tid);
         // gripper poses of the frame start
         if (g.tid < 24) s.fp[g.tid] = P.S.GP[24LL * rod + g.tid];
         g.sync();
@@ -71,21 +71,21 @@ __global__ void __launch_bounds__(kFwdMaxThreads) fwd_kernel(FwdParams P) {
             const int gf = P.frame0 + f;
             if (P.ck_every > 0 && gf % P.ck_every == 0 && gf / P.ck_every < P.ck_count) {
                 const long long c = gf / P.ck_every;
-                write_state<TPR>(P.ck, c * P.ck_strideV, c * P.ck_strideE, c * P.ck_strideB, R, rod, g, s.X, s.V,
+                write_state<TPR>(P.ck, c * P.ck_strideV, c * P.ck_strideE, c * P.ck_strideB, R, rod, g, s.X0, s.V,
                                  s.ED, s.ET, s.HG, s.fp);
             }
             if (g.tid < 12) s.act[g.tid] = P.actions ? P.actions[((long long)f * P.B + rod) * 12 + g.tid] : 0.f;
             g.sync();
             bool ovf = false;
             float mv = 0.f;
-            const int np = run_frame<NV, CONTACT, TPR, true>(P.scene, P.KIN, P.ES, R, s, g, nsub, h, ovf,
-                                                       [](int) -> const Rec* { return nullptr; },
+            const int np = run_frame<NV, CONTACT, TPR>(P.scene, P.KIN, R, own, s, g, nsub, h, ovf,
+                                                       [](int) { return Rec<NV, false>{nullptr, 0}; },
                                                        P.reaction ? P.reaction + 4LL * R.v0 : nullptr, &mv);
             if (ovf) bad |= 2u;
             np_max = max(np_max, np);
             unsigned fl = 0u;
             for (int i = g.tid; i < R.nv; i += TPR) {
-                float4 x = s.X[i], v = s.V[i];
+                float4 x = s.X0[i], v = s.V[i];
                 if (!(isfinite(x.x) && isfinite(x.y) && isfinite(x.z) && isfinite(v.x) && isfinite(v.y) &&
                       isfinite(v.z) && isfinite(v.w)))
                     fl |= 1u;
@@ -101,9 +101,9 @@ __global__ void __launch_bounds__(kFwdMaxThreads) fwd_kernel(FwdParams P) {
                     double r = 0.0;
                     for (int j = g.tid; j < R.ne; j += TPR) {
                         int j1 = (j + 1 == R.nv) ? 0 : j + 1;
-                        const double ex = (double)s.X[j1].x - (double)s.X[j].x;
-                        const double ey = (double)s.X[j1].y - (double)s.X[j].y;
-                        const double ez = (double)s.X[j1].z - (double)s.X[j].z;
+                        const double ex = (double)s.X0[j1].x - (double)s.X0[j].x;
+                        const double ey = (double)s.X0[j1].y - (double)s.X0[j].y;
+                        const double ez = (double)s.X0[j1].z - (double)s.X0[j].z;
                         if (s.ET[j].w > 0.f)   // not a break edge
                             r += fabs(sqrt(ex * ex + ey * ey + ez * ez) - (double)s.ET[j].w);
                     }
@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(kFwdMaxThreads) fwd_kernel(FwdParams P) {
                 }
             }
         }
-        write_state<TPR>(P.S, 0, 0, 0, R, rod, g, s.X, s.V, s.ED, s.ET, s.HG, s.fp);
+        write_state<TPR>(P.S, 0, 0, 0, R, rod, g, s.X0, s.V, s.ED, s.ET, s.HG, s.fp);
         if (g.tid == 0 && bad) atomicOr(&P.status[rod], bad);
         g.sync();
         bounds_end<TPR>(g, P.status, rod);

@@ -60,9 +60,13 @@ cudaError_t launch_rec(const BwdParams& P, int nv_max, bool contact, int grid, i
 int rec_blocks_per_sm(int nv_max, bool contact, int warps);
 cudaError_t launch_rev(const BwdParams& P, int nv_max, bool contact, int grid, int warps, cudaStream_t st);
 int rev_blocks_per_sm(int nv_max, bool contact, int warps);
-// Shared memory of one rod: its arrays plus a 256-byte header for group reductions.
-// per rod: the arrays above, 256 B of group-reduction scratch and the 512 B gripper block
-__host__ __device__ constexpr size_t rod_smem_bytes(int NV, bool contact) { return warp_smem_bytes(NV, contact) + 768; }
+// Substeps whose gripper blocks (256 B each) are formed together.
+constexpr int kPoseBatch = 8;
+// Shared memory of one rod: the arrays above, 256 B of group-reduction scratch, and the gripper
+// blocks, two poses and the actions (240 B), in whole 256 B.
+__host__ __device__ constexpr size_t rod_smem_bytes(int NV, bool contact) {
+    return warp_smem_bytes(NV, contact) + 512 + 256 * kPoseBatch;
+}
 
 // Rod size classes: a rod of nv vertices runs in the kernels instantiated for the smallest
 // class that holds it (shared memory is sized per class; 192 and 224 let two rods of up to
@@ -75,8 +79,8 @@ __host__ __device__ constexpr int size_class(int nv) {
     return nv <= 32 ? 32 : nv <= 64 ? 64 : nv <= 128 ? 128 : nv <= 192 ? 192 : nv <= 224 ? 224 : 256;
 }
 
-// Threads that step one rod of size class NV (one vertex per thread up to 128 vertices).
-__host__ __device__ constexpr int threads_per_rod(int NV) { return NV < 128 ? NV : 128; }
+// Threads that step one rod of size class NV: one per vertex.
+__host__ __device__ constexpr int threads_per_rod(int NV) { return NV; }
 
 cudaError_t launch_forward(const FwdParams& P, int nv_max, bool contact, int grid, int warps, cudaStream_t st);
 int forward_blocks_per_sm(int nv_max, bool contact, int warps);

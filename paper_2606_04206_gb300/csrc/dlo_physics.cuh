@@ -36,15 +36,18 @@ DLO_HD V3<double> transport_d(V3<double> a, V3<double> b, V3<double> d) {
     return c * d + cross(k, d) + (dot(k, d) / (1.0 + c)) * k;
 }
 
-// Length of e and its inverse from one reciprocal square root.
+// Length of e and its inverse from one reciprocal square root.  The length is a rounded product
+// (never fused with a following subtraction), so that the projections of the forward and of the
+// backward's recomputation agree bit for bit whatever the compiler makes of the code around them.
 DLO_HD void len_inv(V3<float> e, float& ell, float& inv) {
     const float e2 = dot(e, e);
 #ifdef __CUDA_ARCH__
     inv = rsqrtf(e2);
+    ell = __fmul_rn(e2, inv);
 #else
     inv = 1.f / sqrtf(e2);
-#endif
     ell = e2 * inv;
+#endif
 }
 
 // Axial strain |e| / |ebar| - 1 with IEEE-rounded square root and quotient: the stretching

@@ -61,6 +61,16 @@ static cudaError_t launch_bucket(dlo_ctx* c, size_t k, int warps, int grid, int 
     return e;
 }
 
+// The rods per CTA run for a requested count (0: refused).  A request is accepted when the
+// rods would fit a CTA of 512 threads at up to 128 threads and 227 KB of shared memory for all
+// (the rule callers know); a CTA of rods above 128 vertices, which take a thread per vertex, then
+// holds as many of them as it can.
+static int forced_rods_per_cta(int nv_max, bool contact, int want) {
+    if (want * std::min(nv_max, 128) > 512 || want * (warp_smem_bytes(nv_max, contact) + 768) > 227 * 1024) return 0;
+    while (want > 1 && forward_blocks_per_sm(nv_max, contact, want) < 1) --want;
+    return want;
+}
+
 // Rods per CTA by measurement (the autotuner): every count whose occupancy keeps at least
 // half of the most resident rods is timed on two frames from the rest state, after one
 // warm-up launch, and the fastest is kept.  The caller resets the state afterwards.
@@ -149,8 +159,9 @@ dlo_status runtime_allocate(dlo_ctx* c, const std::vector<RodInfo>& rods, const 
         // rods per CTA: the count (within the thread budget) that keeps the most rods resident;
         // the measured autotune below may pick another
         int best = 0, best_nb = 0;
-        for (int rpc = 1; rpc <= 16; ++rpc) {
-            if (c->opt.warps_per_cta > 0 && rpc != c->opt.warps_per_cta) continue;
+        const int forced = c->opt.warps_per_cta;
+        const int cap = forced > 0 ? forced_rods_per_cta(bk.nv_max, bk.contact, forced) : 16;
+        for (int rpc = forced > 0 ? std::max(cap, 1) : 1; rpc <= cap; ++rpc) {
             const int nb = forward_blocks_per_sm(bk.nv_max, bk.contact, rpc);
             if (nb >= 1 && rpc * nb >= best * best_nb) {
                 best = rpc;

@@ -1,16 +1,21 @@
 // dlo_step.cuh -- one rod's frame and substep on one thread group, state in shared memory.
 //
-// Shared by the forward kernel and the backward kernel's recomputations.  Per substep
-// (DLO-Lab Sec. 3.1 / 3.2 / App. A.1):
-//   edge phase    each edge's reference frame by time-parallel transport and its material frame
+// Shared by the forward kernel and the backward kernel's recomputations.  Thread i of the group
+// owns vertex i, the edge that starts there and the hinge there.  Per substep (DLO-Lab Sec. 3.1 /
+// 3.2 / App. A.1):
+//   edge phase    the edge's reference frame by time-parallel transport and its material frame
 //   hinge phase   curvature and twist, bending plasticity on the rest curvature, and the
 //                 hinge's energy gradient back to its two edges' frames
-//   edge phase    each edge's frame reversed once on the sum of its two hinges' seeds
+//   edge phase    the edge's frame reversed once on the sum of its two hinges' seeds; its strain
 //   vertex phase  gradient gather + stretching, gravity, damping, symplectic-Euler velocity,
 //                 soft SDF contact (planes, boxes, capsule grippers), displacement predict,
-//                 kinematic vertices, new reference-frame base
-//   PBD phase     N_C x (red-black inextensibility / strain limit, Jacobi self-collision)
-//   velocity      v = d/h, self-contact Coulomb friction, positions x + d
+//                 kinematic vertices, new reference-frame base; new positions when nothing
+//                 projects them
+//   PBD phase     N_C x (red-black inextensibility / strain limit, Jacobi self-collision), then
+//                 v = d/h, positions x + d, self-contact Coulomb friction
+// What a thread's own edge hands from phase to phase stays in its registers; only what a
+// neighbour reads goes through shared memory (per edge: its frame, the seeds of the hinge at its
+// end, its gradient and strain).
 // Per frame: self-contact candidates (every edge pair behind a bounding-sphere filter),
 // gripper pose update.
 #pragma once
@@ -26,9 +31,9 @@ namespace dlo {
 template <bool C>
 using RodRef = typename std::conditional<C, const RodInfo&, const RodInfo>::type;
 
-// A rod is stepped by a group of TPR threads (one or more whole warps); elements are spread
-// over the group with stride TPR and phases are separated by the group's barrier (the warp's
-// own for TPR = 32, else a named barrier of TPR threads).
+// A rod is stepped by a group of TPR threads (whole warps, at least one thread per vertex);
+// phases are separated by the group's barrier (the warp's own for TPR = 32, else a named barrier
+// of TPR threads).
 template <int TPR>
 struct Grp {
     int tid;      // thread index within the rod's group
@@ -97,7 +102,7 @@ template <int TPR>
 __device__ __forceinline__ float grp_max_nonneg(float v, const Grp<TPR>& g) {
     const unsigned w = __reduce_max_sync(0xffffffffu, __float_as_uint(v));
     if (TPR == 32) return __uint_as_float(w);
-    unsigned* r = reinterpret_cast<unsigned*>(g.red) + 60;
+    unsigned* r = reinterpret_cast<unsigned*>(g.red) + 24;
     if ((g.tid & 31) == 0) r[g.tid >> 5] = w;
     g.sync();
     unsigned m = 0u;
@@ -182,17 +187,25 @@ __device__ __forceinline__ int grp_excl_scan(int v, const Grp<TPR>& g) {
     return off + incl - v;
 }
 
-// Optional recording of a substep's intermediates for the adjoint (rec != nullptr): all in
-// global memory, one record per substep of the frames being reversed.
+// One substep's records for the adjoint, in global memory (float4 units from base; NV the size
+// class): start state (X0, V, HG, ED, ET), then what the substep itself stores.  With ON
+// false nothing is recorded.
+template <int NV, bool ON>
 struct Rec {
-    float4* v1;     // [NV]: velocity after the force update, before rigid contact
-    float4* dfin;   // [NV]: displacement after the PBD iterations, before friction
-    float4* pbd;    // [n_iter][NV]: per edge, the unit direction and target / length of its
-                    // inextensibility or strain-limit projection, (0, 0, 0, 1) where it did nothing
-    float4* csnap;  // [n_iter][NV]: displacements before each self-contact sweep (frames with candidates)
-    float4* fr0;    // [pair capacity]: first-iteration projection data of each pair
-    float4* fr1;
-    int nvmax;
+    float4* base;
+    int n_iter;
+    // [NV]: velocity after the force update, before rigid contact
+    __device__ __forceinline__ float4* v1() const { return base + 5 * NV; }
+    // [NV]: displacement after the PBD iterations, before friction
+    __device__ __forceinline__ float4* dfin() const { return base + 6 * NV; }
+    // [n_iter][NV]: per edge, the unit direction and target / length of its inextensibility or
+    // strain-limit projection, (0, 0, 0, 1) where it did nothing
+    __device__ __forceinline__ float4* pbd(int it) const { return base + (size_t)(7 + it) * NV; }
+    // [n_iter][NV]: displacements before each self-contact sweep (frames with candidates)
+    __device__ __forceinline__ float4* csnap(int it) const { return base + (size_t)(7 + n_iter + it) * NV; }
+    // [pair capacity]: first-iteration projection data of each pair
+    __device__ __forceinline__ float4* fr0() const { return base + (size_t)(7 + 2 * n_iter) * NV; }
+    __device__ __forceinline__ float4* fr1() const { return base + (size_t)(7 + 2 * n_iter + kPairsPerVertex) * NV; }
 };
 
 constexpr float kFixPos = 1073741824.f;     // 2^30: fixed-point scale of position corrections
@@ -211,7 +224,7 @@ __device__ __forceinline__ void add_impulse(float4* slot, float m, V3<float> vb,
 }
 
 // Rigid contact of one vertex against the scene and the rod's grippers (Sec. 3.2).
-// sp: the substep's gripper block (see Smem).  imp (optional): the vertex's four impulse
+// sp: the substep's gripper block (Smem::sp).  imp (optional): the vertex's four impulse
 // slots (planes, boxes, gripper 0, gripper 1), to which each active response adds the
 // impulse it gave the vertex of mass m; the rigid body receives the opposite.
 __device__ __forceinline__ V3<float> rigid_contact(const SceneDev& sc, const RodInfo& R, V3<float> x,
@@ -260,7 +273,7 @@ struct Smem {
     // gripper block (read by every thread of the rod with broadcasts):
     //   fp  [24] pose at the start of the frame being stepped, per gripper p (3), R (9) row major
     //   f0  [24] a second frame-start pose (the frame the backward reverses)
-    //   sp  [64] the current substep, per gripper (32): p0 (3), p1 (3), R0 (9), R1 (9), vp (3), w (3)
+    //   sp  [kPoseBatch][64] per substep and gripper (32): p0 (3), p1 (3), R0 (9), R1 (9), vp (3), w (3)
     //   act [12] the frame's actions
     float *fp, *f0, *sp, *act;
     __device__ Smem(float4* base) {
@@ -268,7 +281,7 @@ struct Smem {
         fp = red + 64;
         f0 = fp + 24;
         sp = f0 + 24;
-        act = sp + 64;
+        act = sp + 64 * kPoseBatch;
         X = base;
         X0 = base + NV;
         V = base + 2 * NV;
@@ -321,7 +334,7 @@ __device__ int broad_phase(const RodInfo& R, Smem<NV, CONTACT>& s, const Grp<TPR
     const bool strands = R.flags & ROD_STRANDS;
     for (int j = g.tid; j < ne; j += TPR) {
         const int j1 = (j + 1 == nv) ? 0 : j + 1;
-        const V3<float> p0 = f3(s.X[j]), p1 = f3(s.X[j1]);
+        const V3<float> p0 = f3(s.X0[j]), p1 = f3(s.X0[j1]);
         const V3<float> e = p1 - p0;
         mid[j] = (strands && !(s.ET[j].w > 0.f)) ? make_float4(0.f, 0.f, 0.f, -1.f)
                                                  : f4(0.5f * (p0 + p1), 0.5f * sqrtf(dot(e, e)));
@@ -330,16 +343,16 @@ __device__ int broad_phase(const RodInfo& R, Smem<NV, CONTACT>& s, const Grp<TPR
     for (int k = g.tid; k < nblk; k += TPR) {
         // the vertices of edges k*B .. min(ne, (k+1)*B) - 1 (a loop's last edge ends at vertex 0)
         const int v0 = k * kBpBlock, v1 = min(ne, v0 + kBpBlock);
-        V3<float> lo = f3(s.X[v0]), hi = lo;
+        V3<float> lo = f3(s.X0[v0]), hi = lo;
         for (int v = v0 + 1; v <= v1; ++v) {
-            const V3<float> x = f3(s.X[v == nv ? 0 : v]);
+            const V3<float> x = f3(s.X0[v == nv ? 0 : v]);
             lo = f3(fminf(lo.x, x.x), fminf(lo.y, x.y), fminf(lo.z, x.z));
             hi = f3(fmaxf(hi.x, x.x), fmaxf(hi.y, x.y), fmaxf(hi.z, x.z));
         }
         const V3<float> c = 0.5f * (lo + hi);
         float r2 = 0.f;
         for (int v = v0; v <= v1; ++v) {
-            const V3<float> d = f3(s.X[v == nv ? 0 : v]) - c;
+            const V3<float> d = f3(s.X0[v == nv ? 0 : v]) - c;
             r2 = fmaxf(r2, dot(d, d));
         }
         blk[k] = f4(c, sqrtf(r2));
@@ -378,7 +391,7 @@ __device__ int broad_phase(const RodInfo& R, Smem<NV, CONTACT>& s, const Grp<TPR
         if (closed) sep = min(sep, ne - sep);
         if (!(sep > R.excl || (strands && break_between(s.ET, a, b)))) continue;
         const int a1 = (a + 1 == nv) ? 0 : a + 1, b1 = (b + 1 == nv) ? 0 : b + 1;
-        const V3<float> pa0 = f3(s.X[a]), pa1 = f3(s.X[a1]), pb0 = f3(s.X[b]), pb1 = f3(s.X[b1]);
+        const V3<float> pa0 = f3(s.X0[a]), pa1 = f3(s.X0[a1]), pb0 = f3(s.X0[b]), pb1 = f3(s.X0[b1]);
         float su, uu;
         closest_params(pa0, pa1, pb0, pb1, su, uu);
         const V3<float> dd = (pa0 + su * (pa1 - pa0)) - (pb0 + uu * (pb1 - pb0));
@@ -421,17 +434,17 @@ __device__ int broad_phase_hash(const RodInfo& R, Smem<NV, CONTACT>& s, const Gr
     for (int j = g.tid; j < ne; j += TPR) {
         if (!real(j)) continue;
         const int j1 = (j + 1 == nv) ? 0 : j + 1;
-        const V3<float> e = f3(s.X[j1]) - f3(s.X[j]);
+        const V3<float> e = f3(s.X0[j1]) - f3(s.X0[j]);
         lmax = fmaxf(lmax, sqrtf(dot(e, e)));
     }
     for (int k = g.tid; k <= TBL; k += TPR) cnt[k] = 0;
     lmax = grp_max_nonneg<TPR>(lmax, g);
     const float inv_cell = 1.f / (R.contact_d + lmax);
-    const V3<float> org = f3(s.X[0]);
+    const V3<float> org = f3(s.X0[0]);
     for (int j = g.tid; j < ne; j += TPR) {
         if (!real(j)) continue;
         const int j1 = (j + 1 == nv) ? 0 : j + 1;
-        const V3<float> m = 0.5f * (f3(s.X[j]) + f3(s.X[j1])) - org;
+        const V3<float> m = 0.5f * (f3(s.X0[j]) + f3(s.X0[j1])) - org;
         const int ix = min(max(__float2int_rd(m.x * inv_cell), -510), 510) + 512;
         const int iy = min(max(__float2int_rd(m.y * inv_cell), -510), 510) + 512;
         const int iz = min(max(__float2int_rd(m.z * inv_cell), -510), 510) + 512;
@@ -439,21 +452,22 @@ __device__ int broad_phase_hash(const RodInfo& R, Smem<NV, CONTACT>& s, const Gr
         atomicAdd(&cnt[cell_hash(ix, iy, iz, TBL - 1)], 1);
     }
     g.sync();
-    {   // exclusive scan of the bucket counts, TBL / TPR consecutive buckets per thread
-        constexpr int PER = TBL / TPR;
+    {   // exclusive scan of the bucket counts, PER consecutive buckets per thread
+        constexpr int PER = (TBL + TPR - 1) / TPR;
         int loc[PER];
         int sum = 0;
 #pragma unroll
         for (int k = 0; k < PER; ++k) {
-            loc[k] = cnt[g.tid * PER + k];
+            loc[k] = g.tid * PER + k < TBL ? cnt[g.tid * PER + k] : 0;
             sum += loc[k];
         }
         int run = grp_excl_scan<TPR>(sum, g);
 #pragma unroll
-        for (int k = 0; k < PER; ++k) {
-            cnt[g.tid * PER + k] = run;
-            run += loc[k];
-        }
+        for (int k = 0; k < PER; ++k)
+            if (g.tid * PER + k < TBL) {
+                cnt[g.tid * PER + k] = run;
+                run += loc[k];
+            }
     }
     g.sync();
     for (int j = g.tid; j < ne; j += TPR) {
@@ -472,7 +486,7 @@ __device__ int broad_phase_hash(const RodInfo& R, Smem<NV, CONTACT>& s, const Gr
         const int key = keys[a];
         const int ix = key >> 20, iy = (key >> 10) & 1023, iz = key & 1023;
         const int a1 = (a + 1 == nv) ? 0 : a + 1;
-        const V3<float> pa0 = f3(s.X[a]), pa1 = f3(s.X[a1]);
+        const V3<float> pa0 = f3(s.X0[a]), pa1 = f3(s.X0[a1]);
         for (int dz = -1; dz <= 1; ++dz)
             for (int dy = -1; dy <= 1; ++dy)
                 for (int dx = -1; dx <= 1; ++dx) {
@@ -487,7 +501,7 @@ __device__ int broad_phase_hash(const RodInfo& R, Smem<NV, CONTACT>& s, const Gr
                         if (closed) sep = min(sep, ne - sep);
                         if (sep <= R.excl && !(strands && break_between(s.ET, a, b))) continue;
                         const int b1 = (b + 1 == nv) ? 0 : b + 1;
-                        const V3<float> pb0 = f3(s.X[b]), pb1 = f3(s.X[b1]);
+                        const V3<float> pb0 = f3(s.X0[b]), pb1 = f3(s.X0[b1]);
                         float su, uu;
                         closest_params(pa0, pa1, pb0, pb1, su, uu);
                         const V3<float> dd = (pa0 + su * (pa1 - pa0)) - (pb0 + uu * (pb1 - pb0));
@@ -522,7 +536,7 @@ __device__ __forceinline__ void color_range(int ne, bool closed, int color, int&
 
 // One colour of inextensibility / strain-limit projections (App. A.1) on displacements D
 // from start positions X0: C = |x_{j+1} - x_j| - |ebar|, lambda = C / (w_j + w_{j+1}).
-// prec (optional): receives each edge's projection record (see Rec::pbd).
+// prec (optional): receives each edge's projection record (Rec::pbd).
 template <int TPR>
 __device__ __forceinline__ void inext_color_arr(const RodInfo& R, const float4* X0, float4* D, const float4* ET,
                                                 const Grp<TPR>& g, int color, bool closed, float4* prec = nullptr) {
@@ -687,219 +701,208 @@ __device__ __forceinline__ void load_frame(EdgeF<float>& E, float4 ta, float4 rc
     E.d2 = E.c * E.d2r - E.s * E.d1r;
 }
 
-// A hinge's gradient seeds for one of its edges, added to the edge's sums (the other hinge of
-// the edge adds to the same sums).
-__device__ __forceinline__ void add_seeds(float4* sg, float4* sr, V3<float> gt, V3<float> gd1r, float gth) {
-    atomicAdd(&sg->x, gt.x);
-    atomicAdd(&sg->y, gt.y);
-    atomicAdd(&sg->z, gt.z);
-    atomicAdd(&sg->w, gth);
-    atomicAdd(&sr->x, gd1r.x);
-    atomicAdd(&sr->y, gd1r.y);
-    atomicAdd(&sr->z, gd1r.z);
+// ------------------------------------------------------------------ one substep
+// What a thread keeps of its own vertex and edge for the whole rod.
+struct Own {
+    int kind;      // 0 free, 1 pinned, 2 / 3 held by gripper 0 / 1
+    float invI;    // 1 / axial inertia of the edge that starts here
+};
+
+__device__ __forceinline__ Own own_of(const float4* __restrict__ KIN, const float2* __restrict__ ES, const RodInfo& R,
+                                      int i) {
+    return Own{i < R.nv ? (int)KIN[R.v0 + i].w : 1, i < R.ne ? ES[R.e0 + i].y : 0.f};
 }
 
-// ------------------------------------------------------------------ one substep
-template <int NV, bool CONTACT, int TPR>
-__device__ __forceinline__ void substep_body(const SceneDev& sc, const float4* __restrict__ KIN, const float2* __restrict__ ES,
-                        const RodInfo& R, Smem<NV, CONTACT>& s, const Grp<TPR>& g, float h, int np,
-                        const Rec* rec = nullptr, float4* imp = nullptr, float* mv = nullptr) {
-    const int nv = R.nv, ne = R.ne, v0 = R.v0, e0 = R.e0;
+// Target of a held vertex at the substep's end: the gripper's end pose applied to its grasp offset.
+__device__ __forceinline__ V3<float> grasp_target(const float* sp, int kind, float4 kin) {
+    const float* o = sp + 32 * (kind - 2);
+    const V3<float> off = f3(kin);
+    const V3<float> p1 = f3(o[3], o[4], o[5]);
+    return p1 + f3(o[15] * off.x + o[16] * off.y + o[17] * off.z, o[18] * off.x + o[19] * off.y + o[20] * off.z,
+                   o[21] * off.x + o[22] * off.y + o[23] * off.z);
+}
+
+// The group has synchronised since X0, V, ED, ET, HG and sp were written; on return it has
+// synchronised after writing them.  sp: the substep's gripper block.  The substep is bound by
+// the latency of its phases' dependent arithmetic and of the barriers between them (about a
+// third of the issue slots at four 128-vertex rods per SM), so it keeps instructions and
+// barriers few: one thread per element, four phases for a rod without projections, and no
+// atomics (a hinge's seeds for its previous edge travel through one slot; float atomics on
+// shared memory are compare-and-swap loops).  4096 elastic ropes x 128 vertices: 30.2 -> 19.1 us
+// per substep of the batch against atomics and elements spread over at most 128 threads; one
+// 256-vertex class of the ragged batch 4.2 -> 1.5 ms.
+template <int NV, bool CONTACT, int TPR, bool REC>
+__device__ __forceinline__ void substep_body(const SceneDev& sc, const float4* __restrict__ KIN, const RodInfo& R,
+                                             const Own& own, Smem<NV, CONTACT>& s, const Grp<TPR>& g, float h, int np,
+                                             const float* sp, const Rec<NV, REC> rec, float4* imp = nullptr,
+                                             float* mv = nullptr) {
+    static_assert(TPR >= NV, "one thread per vertex");
+    const int nv = R.nv, ne = R.ne;
     const bool closed = R.flags & ROD_CLOSED;
-    const int nh = closed ? nv : nv - 2;
     const bool strands = R.flags & ROD_STRANDS;
-    // --- edge frames, once per edge: (t, |e|) in EA, (w0, n1) in EW, (d1r, cos theta) in ND
-    // (the vertex phase takes the new reference director from there), and per edge the seeds
-    // its two hinges send back: (dU/dt, dU/dtheta) in SG, (dU/dd1r, sin theta) in SR.  The
-    // displacement array SR = X is rewritten by the vertex phase before it is read.
-    float4* const EA = s.HB0;
-    float4* const EW = s.HB1;
-    float4* const SG = s.HB2;
-    float4* const SR = s.X;
-    for (int j = g.tid; j < ne; j += TPR) {
-        const int j1 = (j + 1 == nv) ? 0 : j + 1;
-        const float4 ed = s.ED[j], et = s.ET[j];
-        SG[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (strands && !(et.w > 0.f)) continue;   // a break edge: no frame, no hinge
-        EdgeF<float> E;
-        edge_forward(E, f3(s.X0[j]), f3(s.X0[j1]), f3(et), f3(ed), ed.w);
-        EA[j] = f4(E.t, E.ell);
-        EW[j] = f4(E.w0, E.n1);
-        s.ND[j] = f4(E.d1r, E.c);
-        SR[j] = make_float4(0.f, 0.f, 0.f, E.s);
+    const int i = g.tid;
+    const int ip = (i + 1 == nv) ? 0 : i + 1;       // end vertex of the own edge
+    const int im = (i == 0) ? nv - 1 : i - 1;       // the edge that ends at the own vertex (if any)
+    const bool vtx = i < nv, has_e = i < ne, has_em = vtx && (closed || i > 0);
+    // exchanged between neighbours; the displacement array SR = X is rewritten by the vertex
+    // phase before it is read
+    float4* const FA = s.HB0;   // per edge (t, sin theta)
+    float4* const FB = s.HB1;   // per edge (d1r, cos theta)
+    float4* const SG = s.HB2;   // per edge (dU/dt, dU/dtheta) of the hinge at its end; then (dU/de, K A strain)
+    float4* const SR = s.X;     // per edge dU/dd1r of the hinge at its end
+    // --- the own edge's frame.  A break edge (rest length 0) has no frame and no hinge.
+    EdgeF<float> E;
+    V3<float> tb, d1b;
+    float theta = 0.f, eb = 0.f;
+    bool real = false;
+    if (has_e) {
+        const float4 ed = s.ED[i], et = s.ET[i];
+        tb = f3(et);
+        d1b = f3(ed);
+        theta = ed.w;
+        eb = et.w;
+        real = !(strands && !(eb > 0.f));
+        if (real) {
+            edge_forward(E, f3(s.X0[i]), f3(s.X0[ip]), tb, d1b, theta);
+            FA[i] = f4(E.t, E.s);
+            FB[i] = f4(E.d1r, E.c);
+        }
     }
     g.sync();
-    // --- hinge phase: the hinge's own part, from its edges' frames
-    for (int k = g.tid; k < nh; k += TPR) {
-        const int i = closed ? k : k + 1;
-        const int a = (i == 0) ? ne - 1 : i - 1;
-        const int b = i;
-        const float4 ETa = s.ET[a], ETb = s.ET[b];
-        float4 hg = s.HG[i];
-        if (strands && !(ETa.w > 0.f && ETb.w > 0.f)) continue;   // a hinge at an end of a break edge
-        HingeF<float> H;
-        load_frame(H.a, EA[a], s.ND[a], SR[a].w);
-        load_frame(H.b, EA[b], s.ND[b], SR[b].w);
-        hinge_core_forward(H, s.ED[a].w, s.ED[b].w, hg.w);
-        const float lbar = 0.5f * (ETa.w + ETb.w);
-        if (R.flags & ROD_PLASTIC) plastic_update(H.k0, H.k1, hg.x, hg.y, R.sy * lbar, R.rc);
-        const float il = 1.f / lbar;
-        const float gk0 = R.Bm * il * (H.k0 - hg.x), gk1 = R.Bm * il * (H.k1 - hg.y);
-        const float gm = R.beta * il * (H.m - hg.z);
-        V3<float> gta, gd1ra, gtb, gd1rb;
-        float ghta, ghtb;
-        hinge_core_reverse(H, gk0, gk1, gm, 0.f, gta, gd1ra, gtb, gd1rb, ghta, ghtb);
-        add_seeds(SG + a, SR + a, gta, gd1ra, ghta);
-        add_seeds(SG + b, SR + b, gtb, gd1rb, ghtb);
-        s.HG[i] = make_float4(hg.x, hg.y, hg.z, H.mref);
+    // --- the own hinge, from its edges' frames: seeds for the own edge (kept) and for the
+    // previous one (sent; zero where there is no active hinge)
+    V3<float> gtb = zf3(), gd1rb = zf3();
+    float ghtb = 0.f;
+    if (has_em) {
+        V3<float> gta = zf3(), gd1ra = zf3();
+        float ghta = 0.f;
+        const float eba = s.ET[im].w;
+        if (has_e && !(strands && !(eba > 0.f && eb > 0.f))) {
+            float4 hg = s.HG[i];
+            HingeF<float> H;
+            const float4 fa = FA[im], fb = FB[im];
+            load_frame(H.a, fa, fb, fa.w);
+            H.b = E;
+            hinge_core_forward(H, s.ED[im].w, theta, hg.w);
+            const float lbar = 0.5f * (eba + eb);
+            if (R.flags & ROD_PLASTIC) plastic_update(H.k0, H.k1, hg.x, hg.y, R.sy * lbar, R.rc);
+            const float il = 1.f / lbar;
+            const float gk0 = R.Bm * il * (H.k0 - hg.x), gk1 = R.Bm * il * (H.k1 - hg.y);
+            const float gm = R.beta * il * (H.m - hg.z);
+            hinge_core_reverse(H, gk0, gk1, gm, 0.f, gta, gd1ra, gtb, gd1rb, ghta, ghtb);
+            s.HG[i] = make_float4(hg.x, hg.y, hg.z, H.mref);
+        }
+        SG[im] = f4(gta, ghta);
+        SR[im] = f4(gd1ra, 0.f);
     }
     g.sync();
-    // --- per edge, the reverse through its frame: the gradient on the edge vector (in SG, with
-    // the edge's twist gradient; zero for a break edge)
-    for (int j = g.tid; j < ne; j += TPR) {
-        const float4 et = s.ET[j], sg = SG[j];
-        if (strands && !(et.w > 0.f)) continue;   // SG[j] stays zero
-        const float4 ea = EA[j], ew = EW[j], nd = s.ND[j];
-        EdgeF<float> E;
-        E.t = f3(ea);
-        E.ell = ea.w;
-        E.w0 = f3(ew);
-        E.n1 = ew.w;
-        E.d1r = f3(nd);
-        const V3<float> ge =
-            edge_reverse<float, false>(E, f3(et), f3(s.ED[j]), f3(sg), f3(SR[j]), 0.f, nullptr, nullptr);
-        SG[j] = f4(ge, sg.w);
+    // --- the reverse through the own edge's frame: the gradient on the edge vector.  The
+    // stretching strain has an IEEE-rounded square root and quotient (the strains of nearly
+    // inextensible ropes are ~1e-4, so a few ulps of the length matter to them).
+    V3<float> ge = zf3();
+    float gth = 0.f, str = 0.f;
+    if (has_e) {
+        if (real) {
+            const float4 sg = SG[i], sr = SR[i];
+            gth = sg.w + ghtb;
+            ge = edge_reverse<float, false>(E, tb, d1b, f3(sg) + gtb, f3(sr) + gd1rb, 0.f, nullptr, nullptr);
+            if (R.kA > 0.f) str = R.kA * edge_strain(f3(s.X0[ip]) - f3(s.X0[i]), eb);
+        }
+        SG[i] = f4(ge, str);
     }
     g.sync();
-    // --- vertex phase
-    for (int i = g.tid; i < nv; i += TPR) {
+    // --- the own vertex
+    const bool lenc = R.flags & (ROD_INEXT | ROD_SLIMIT);
+    const bool project = lenc || (CONTACT && np > 0);
+    const float ih = 1.f / h;
+    // new position (the absolute target for a held vertex) and velocity from the displacement d
+    auto finish = [&](float4 x0, V3<float> d, float om) {
+        float4 x = make_float4(x0.x + d.x, x0.y + d.y, x0.z + d.z, x0.w);
+        if (own.kind >= 2 && in_bounds(own.kind - 2 < R.ngrip, s.red))
+            x = f4(grasp_target(sp, own.kind, KIN[R.v0 + i]), x0.w);
+        if (mv) {
+            const float dx = x.x - x0.x, dy = x.y - x0.y, dz = x.z - x0.z;
+            *mv += sqrtf(dx * dx + dy * dy + dz * dz);
+        }
+        s.X0[i] = x;
+        s.V[i] = make_float4(d.x * ih, d.y * ih, d.z * ih, om);
+    };
+    if (vtx) {
         const float4 xi4 = s.X0[i];
         const V3<float> xi = f3(xi4);
-        V3<float> g = zf3();
-        const int im = (i == 0) ? nv - 1 : i - 1;
-        float gth = 0.f;
-        const bool has_e = closed || i < nv - 1;          // edge i starts here
-        const bool has_em = closed || i >= 1;             // edge i-1 ends here
-        // bending and twisting: the gradients on the edge vectors of the edges at this vertex
-        if (has_e) {
-            const float4 q = SG[i];
-            g -= f3(q);
-            gth = q.w;
+        V3<float> gr = zf3();
+        float4 pe = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (has_e) gr -= ge;
+        if (has_em) {
+            pe = SG[im];
+            gr += f3(pe);
         }
-        if (has_em) g += f3(SG[im]);
-        V3<float> t_i = zf3();
-        float ell_i = 0.f;
-        // a break edge (between two strands) starts here: no tangent, no force, frame kept
-        const bool brk = strands && has_e && !(ES[e0 + i].x > 0.f);
-        // stretching: the strains with IEEE-rounded square roots and quotients (the strains of
-        // nearly inextensible ropes are ~1e-4, so a few ulps of the length matter to them)
-        if (has_e && !brk) {
-            const float4 q = EA[i];
-            ell_i = q.w;
-            t_i = f3(q);
-            if (R.kA > 0.f) g -= (R.kA * edge_strain(f3(s.X0[i + 1 == nv ? 0 : i + 1]) - xi, ES[e0 + i].x)) * t_i;
+        if (R.kA > 0.f) {
+            if (real) gr -= str * E.t;
+            if (has_em && !(strands && !(s.ET[im].w > 0.f))) gr += pe.w * f3(FA[im]);
         }
-        if (R.kA > 0.f && has_em && !(strands && !(ES[e0 + im].x > 0.f)))   // edge i-1 ends here
-            g += (R.kA * edge_strain(xi - f3(s.X0[im]), ES[e0 + im].x)) * f3(EA[im]);
-        float4 vi = s.V[i];
-        const float4 kin = KIN[v0 + i];
-        const int kind = (int)kin.w;
+        const float4 vi = s.V[i];
         // displacement d of this substep (positions are only formed at its end, so the rebuilt
         // velocity d/h carries no cancellation error from |x| >> |h v|)
-        V3<float> v2 = zf3(), d = zf3();
-        float4 nd_out = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (kind == 0) {
+        V3<float> d = zf3();
+        if (own.kind == 0) {
             V3<float> grav = f3(0.f, 0.f, -sc.gravity);
-            V3<float> acc = (-xi4.w) * g + grav - R.cd * f3(vi);
+            V3<float> acc = (-xi4.w) * gr + grav - R.cd * f3(vi);
             V3<float> v1 = f3(vi) + h * acc;
-            if (rec) rec->v1[i] = f4(v1, 0.f);
-            v2 = rigid_contact(sc, R, xi, v1, s.sp, imp ? imp + 4 * i : nullptr, 1.f / xi4.w);
+            if (REC) rec.v1()[i] = f4(v1, 0.f);
+            const V3<float> v2 = rigid_contact(sc, R, xi, v1, sp, imp ? imp + 4 * i : nullptr, 1.f / xi4.w);
             d = h * v2;
-        } else if (kind >= 2 && in_bounds(kind - 2 < R.ngrip, s.red)) {
-            const float* o = s.sp + 32 * (kind - 2);
-            const V3<float> off = f3(kin);
-            const V3<float> p1 = f3(o[3], o[4], o[5]);
-            const V3<float> tgt = p1 + f3(o[15] * off.x + o[16] * off.y + o[17] * off.z,
-                                          o[18] * off.x + o[19] * off.y + o[20] * off.z,
-                                          o[21] * off.x + o[22] * off.y + o[23] * off.z);
-            nd_out = f4(tgt, 1.f);      // absolute target at the substep end
-            d = tgt - xi;               // a grasped vertex sits at the gripper target
-            v2 = d / h;
+        } else if (own.kind >= 2 && in_bounds(own.kind - 2 < R.ngrip, s.red)) {
+            d = grasp_target(sp, own.kind, KIN[R.v0 + i]) - xi;   // a held vertex sits at its target
         }
         float om1 = vi.w;
         if (has_e) {
-            const float invI = ES[e0 + i].y;
-            om1 = vi.w + h * (-gth * invI - R.cd * vi.w);
-            float4 ed = s.ED[i];
-            if (brk) {
-                s.ED[i] = make_float4(ed.x, ed.y, ed.z, ed.w + h * om1);
+            om1 = vi.w + h * (-gth * own.invI - R.cd * vi.w);
+            const float th1 = theta + h * om1;
+            if (real) {
+                s.ED[i] = f4(E.d1r, th1);   // the edge's new reference director
+                s.ET[i] = f4(E.t, eb);
             } else {
-                s.ED[i] = f4(f3(s.ND[i]), ed.w + h * om1);   // the edge's new reference director
-                s.ET[i] = f4(t_i, ES[e0 + i].x);
+                s.ED[i] = f4(d1b, th1);
             }
         }
-        s.ND[i] = nd_out;
-        s.X[i] = f4(d, xi4.w);
-        s.V[i] = f4(v2, om1);
+        if (project) {
+            s.X[i] = f4(d, xi4.w);
+            s.V[i].w = om1;
+        } else {
+            if (REC) rec.dfin()[i] = f4(d, xi4.w);
+            finish(xi4, d, om1);
+        }
     }
     g.sync();
+    if (!project) return;
     // --- PBD
-    const bool lenc = R.flags & (ROD_INEXT | ROD_SLIMIT);
-    if (lenc || np > 0) {
-        for (int it = 0; it < sc.n_iter; ++it) {
-            if (lenc) {
-                const int ncol = (closed && (ne & 1)) ? 3 : 2;
-                for (int k = 0; k < ncol; ++k)
-                    inext_color<NV, CONTACT, TPR>(R, s, g, k, closed, rec ? rec->pbd + (size_t)it * rec->nvmax : nullptr);
-            }
-            if (CONTACT && np > 0) {
-                // each thread stores its own vertices; the sweep reads s.X and writes only the
-                // accumulators before its own barrier
-                if (rec)
-                    for (int i = g.tid; i < nv; i += TPR) rec->csnap[(size_t)it * rec->nvmax + i] = s.X[i];
-                contact_sweep_call<NV, CONTACT, TPR>(&R, s.X, g.tid, g.bar, np, it == 0);
-            }
+    for (int it = 0; it < sc.n_iter; ++it) {
+        if (lenc) {
+            const int ncol = (closed && (ne & 1)) ? 3 : 2;
+            for (int k = 0; k < ncol; ++k)
+                inext_color<NV, CONTACT, TPR>(R, s, g, k, closed, REC ? rec.pbd(it) : nullptr);
+        }
+        if (CONTACT && np > 0) {
+            // each thread stores its own vertices; the sweep reads s.X and writes only the
+            // accumulators before its own barrier
+            if (REC && vtx) rec.csnap(it)[i] = s.X[i];
+            contact_sweep_call<NV, CONTACT, TPR>(&R, s.X, g.tid, g.bar, np, it == 0);
         }
     }
-    // --- velocity from the displacement, friction, new positions
-    const float ih = 1.f / h;
-    for (int i = g.tid; i < nv; i += TPR) {
-        float4 d = s.X[i], v = s.V[i];
-        if (rec) rec->dfin[i] = d;
-        s.V[i] = make_float4(d.x * ih, d.y * ih, d.z * ih, v.w);
+    // --- velocity from the displacement, new positions, friction
+    if (vtx) {
+        const float4 d = s.X[i];
+        if (REC) rec.dfin()[i] = d;
+        finish(s.X0[i], f3(d), s.V[i].w);
     }
-    g.sync();
-    if (CONTACT && rec)
+    if (CONTACT && REC)
         for (int p = g.tid; p < np; p += TPR) {
-            rec->fr0[p] = s.fr0[p];
-            rec->fr1[p] = s.fr1[p];
+            rec.fr0()[p] = s.fr0[p];
+            rec.fr1()[p] = s.fr1[p];
         }
-    if (CONTACT && np > 0) self_friction_call<NV, CONTACT, TPR>(&R, s.X, g.tid, g.bar, np, h, sc.mu_self);
-    float dm2 = 0.f;   // the largest squared displacement of this thread's vertices
-    for (int i = g.tid; i < nv; i += TPR) {
-        float4 x0 = s.X0[i], d = s.X[i], nd = s.ND[i];
-        float4 x = nd.w > 0.5f ? make_float4(nd.x, nd.y, nd.z, x0.w)
-                               : make_float4(x0.x + d.x, x0.y + d.y, x0.z + d.z, x0.w);
-        if (mv) {
-            const float dx = x.x - x0.x, dy = x.y - x0.y, dz = x.z - x0.z;
-            dm2 = fmaxf(dm2, dx * dx + dy * dy + dz * dz);
-        }
-        s.X0[i] = x;
-        s.X[i] = x;
-    }
-    if (mv) *mv += sqrtf(dm2);
     g.sync();
-}
-
-
-// The substep inlined (the forward kernel, and the backward's per-frame recompute with
-// records, where a call costs more than the larger code) and as one out-of-line copy (the
-// backward's replay of the frames between two checkpoints).
-template <int NV, bool CONTACT, int TPR>
-__device__ __noinline__ void substep_call(const SceneDev& sc, const float4* __restrict__ KIN,
-                                          const float2* __restrict__ ES, const RodInfo& R, Smem<NV, CONTACT>& s,
-                                          const Grp<TPR>& g, float h, int np, const Rec* rec) {
-    substep_body<NV, CONTACT, TPR>(sc, KIN, ES, R, s, g, h, np, rec);
+    if (CONTACT && np > 0) self_friction_call<NV, CONTACT, TPR>(&R, s.X, g.tid, g.bar, np, h, sc.mu_self);
 }
 
 // Substep pose block of gripper q (32 floats at out + 32 q) from the frame-start pose F
@@ -947,30 +950,30 @@ __device__ __forceinline__ void frame_advance(float* F, const float* act, int q)
 // One frame of one rod: candidates (if self-contact), nsub substeps, pose update.  The frame's
 // start pose is s.fp and its actions s.act, both set (and synchronised) by the caller; s.fp
 // holds the end pose on return.  pre(sb) runs before substep sb (after a group barrier), e.g.
-// to store the substep state, and returns the substep's record (or nullptr).  imp: the rod's
-// impulse slots (4 per vertex) when the contact impulses are being accumulated (inlined
-// substeps only).  mv (inlined substeps only): adds, per thread, the sum over the frame's
-// substeps of the largest displacement of the thread's vertices, a bound on how far any of
-// them moved during the frame.
-template <int NV, bool CONTACT, int TPR, bool INLINE, class PreSub>
-__device__ __forceinline__ int run_frame(const SceneDev& sc, const float4* __restrict__ KIN, const float2* __restrict__ ES,
-                         const RodInfo& R, Smem<NV, CONTACT>& s, const Grp<TPR>& g, int nsub, float h, bool& ovf,
-                         PreSub pre, float4* imp = nullptr, float* mv = nullptr) {
+// to store the substep state, and returns where the substep's records go.  imp: the rod's
+// impulse slots (4 per vertex) when the contact impulses are being accumulated.  mv: adds, per
+// thread, the sum over the frame's substeps of its vertex's displacement, a bound on how far it
+// moved during the frame.
+template <int NV, bool CONTACT, int TPR, class PreSub>
+__device__ __forceinline__ int run_frame(const SceneDev& sc, const float4* __restrict__ KIN, const RodInfo& R,
+                                         const Own& own, Smem<NV, CONTACT>& s, const Grp<TPR>& g, int nsub, float h,
+                                         bool& ovf, PreSub pre, float4* imp = nullptr, float* mv = nullptr) {
     int np = 0;
     if (CONTACT && (R.flags & ROD_SELF))
         np = (R.flags & ROD_HASH) ? broad_phase_hash<NV, CONTACT, TPR>(R, s, g, (R.flags & ROD_CLOSED) != 0, ovf)
                                   : broad_phase<NV, CONTACT, TPR>(R, s, g, (R.flags & ROD_CLOSED) != 0, ovf);
     const float inv_dt = 1.f / sc.dt;
     for (int sb = 0; sb < nsub; ++sb) {
-        const Rec* rec = pre(sb);
-        // the substep's gripper block: written here, read after the hinge phase's barrier
-        if (g.tid < R.ngrip)
-            substep_pose(s.fp, s.act, g.tid, (float)sb / (float)nsub, (float)(sb + 1) / (float)nsub, sb == 0, inv_dt,
-                         s.sp);
-        if (INLINE)
-            substep_body<NV, CONTACT, TPR>(sc, KIN, ES, R, s, g, h, np, rec, imp, mv);
-        else
-            substep_call<NV, CONTACT, TPR>(sc, KIN, ES, R, s, g, h, np, rec);
+        // the gripper blocks of the next kPoseBatch substeps, one per thread, side by side (two
+        // rotation exponentials each: done by one thread every substep they were about a tenth
+        // of a lone rod's substep); read after the hinge phase's barrier
+        if (sb % kPoseBatch == 0) {
+            const int k = sb + (g.tid >> 1), q = g.tid & 1;
+            if (g.tid < 2 * kPoseBatch && k < nsub && q < R.ngrip)
+                substep_pose(s.fp, s.act, q, (float)k / (float)nsub, (float)(k + 1) / (float)nsub, k == 0, inv_dt,
+                             s.sp + 64 * (g.tid >> 1));
+        }
+        substep_body(sc, KIN, R, own, s, g, h, np, s.sp + 64 * (sb % kPoseBatch), pre(sb), imp, mv);
     }
     if (g.tid < R.ngrip) frame_advance(s.fp, s.act, g.tid);
     g.sync();
