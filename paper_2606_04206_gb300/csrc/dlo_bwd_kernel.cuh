@@ -23,16 +23,6 @@
 
 namespace dlo {
 
-// Threads per CTA the reverse kernel is compiled for (its register budget).  Rods of up to 128
-// vertices take at most 62.5 KB of shared memory each, so three fit an SM: 384 threads at 168
-// registers.  Larger rods fit two per SM (one at 256 vertices), and keep 255 registers.
-__host__ __device__ constexpr int rev_max_threads(int NV) { return NV <= 128 ? 384 : 256; }
-__host__ __device__ constexpr int rev_threads(int NV) { return NV < 128 ? NV : 128; }
-
-__host__ __device__ constexpr size_t bwd_smem_bytes(int NV, bool contact) {
-    return rod_smem_bytes(NV, contact) + (size_t)(10 * NV + 20) * 16;
-}
-
 // ------------------------------------------------------------------ small helpers
 __device__ __forceinline__ void atomic_add3(float4* a, V3<float> v) {
     atomicAdd(&a->x, v.x);
@@ -117,22 +107,37 @@ __device__ __forceinline__ V3<T> prim_respond(int k, const SceneDev& sc, const R
     return contact_respond(v, sdf, n, vrig, R.radius, R.eps, sc.mu_rigid, sc.restitution, act);
 }
 
+// Shared memory of one rod of the reverse kernel: what a neighbour (or another vertex of a
+// contact pair) reads, and the frame's gripper data.
 template <int NV, bool CONTACT>
-struct AdjArrays {
-    float4 *LX, *LD, *LV, *LE, *LT, *LK, *LP0, *LG, *V1, *DF;
-    float* PM;   // per gripper (36): the substep's M0, M1, c0 J_l(c0 dphi)^T, c1 J_l(c1 dphi)^T (row major)
-    __device__ AdjArrays(float4* a) {
-        LX = a;
-        LD = a + NV;
-        LV = a + 2 * NV;
-        LE = a + 3 * NV;
-        LT = a + 4 * NV;
-        LK = a + 5 * NV;
-        LP0 = a + 6 * NV;
-        LG = a + 7 * NV;
-        V1 = a + 8 * NV;
-        DF = a + 9 * NV;
-        PM = reinterpret_cast<float*>(a + 10 * NV);
+struct RevSmem {
+    float4 *LD;                 // displacement cotangents, then the force cotangents, then dL/d(edge vectors)
+    float4 *F0, *F1, *F2, *F3;  // per edge: its dual frame, replaced by the seeds of the hinge at its end
+    float2* GM;                 // [5][NV]: the threads' material sums, each an unevaluated sum of two floats
+    uint32_t* pairs;
+    float *red, *f0, *act;      // reduction scratch, the frame's start pose (24) and actions (12)
+    float *sp, *PM;             // per substep of a batch: gripper blocks (64) and pose maps (72)
+    double *PR, *PC;            // per warp, its sums of the 24 pose terms; the carried pose cotangents (12)
+    float* GA;                  // the frame's action cotangents carried from the next frame's pose (12)
+    static constexpr size_t kHeader = 64 + 24 + 16 + 64 * kPoseBatch + 72 * kPoseBatch + 2 * (8 * 24 + 12) + 12 + 4;
+    static constexpr size_t kBytes = 16 * (size_t)(5 * NV) + 8 * (size_t)(5 * NV) +
+                                     (CONTACT ? 4 * (size_t)(kPairsPerVertex * NV) : 0) + 4 * kHeader;
+    __device__ explicit RevSmem(float4* b) {
+        LD = b;
+        F0 = b + NV;
+        F1 = b + 2 * NV;
+        F2 = b + 3 * NV;
+        F3 = b + 4 * NV;
+        GM = reinterpret_cast<float2*>(b + 5 * NV);
+        PR = reinterpret_cast<double*>(GM + 5 * NV);
+        PC = PR + 8 * 24;
+        red = reinterpret_cast<float*>(PC + 12);
+        f0 = red + 64;
+        act = f0 + 24;
+        sp = act + 16;
+        PM = sp + 64 * kPoseBatch;
+        GA = PM + 72 * kPoseBatch;
+        pairs = reinterpret_cast<uint32_t*>(GA + 16);
     }
 };
 
@@ -149,560 +154,551 @@ __device__ __forceinline__ void save_state(float4* dst, const RodInfo& R, const 
         dst[4 * NV + j] = s.ET[j];
     }
 }
-template <int NV, bool C, int TPR>
-__device__ __forceinline__ void load_state(const float4* src, const RodInfo& R, const Grp<TPR>& g, Smem<NV, C>& s) {
-    for (int i = g.tid; i < R.nv; i += TPR) {
-        float4 x = src[i];
-        s.X0[i] = x;
-        s.X[i] = x;
-        s.V[i] = src[NV + i];
-        s.HG[i] = src[2 * NV + i];
-    }
-    for (int j = g.tid; j < R.ne; j += TPR) {
-        s.ED[j] = src[3 * NV + j];
-        s.ET[j] = src[4 * NV + j];
-    }
-    g.sync();
-}
-
-// Per-g.tid pose cotangents of one substep (two grippers x 3).
-struct PoseAdj {
-    float ps0[6], phs0[6], ps1[6], phs1[6], vp[6], w[6];
-    __device__ void zero() {
-#pragma unroll
-        for (int k = 0; k < 6; ++k) ps0[k] = phs0[k] = ps1[k] = phs1[k] = vp[k] = w[k] = 0.f;
-    }
-};
-// gripper q in {0, 1}; both halves are addressed with constant indices so that the per-thread
-// arrays stay in registers
-__device__ __forceinline__ void add3(float* a, int q, V3<float> v) {
-    if (q == 0) {
-        a[0] += v.x;
-        a[1] += v.y;
-        a[2] += v.z;
-    } else {
-        a[3] += v.x;
-        a[4] += v.y;
-        a[5] += v.z;
-    }
-}
-__device__ __forceinline__ V3<float> get3(const float* a, int q) {
-    return q == 0 ? f3(a[0], a[1], a[2]) : f3(a[3], a[4], a[5]);
-}
 // row-major 3x3 at o times v
 __device__ __forceinline__ V3<float> mul_rm(const float* o, V3<float> v) {
     return f3(o[0] * v.x + o[1] * v.y + o[2] * v.z, o[3] * v.x + o[4] * v.y + o[5] * v.z,
               o[6] * v.x + o[7] * v.y + o[8] * v.z);
 }
+__device__ __forceinline__ V3<float> mul_rm_t(const float* o, V3<float> v) {
+    return f3(o[0] * v.x + o[3] * v.y + o[6] * v.z, o[1] * v.x + o[4] * v.y + o[7] * v.z,
+              o[2] * v.x + o[5] * v.y + o[8] * v.z);
+}
 
-// The dual-number frames of a rod's edges (7 float4 per edge) and the seeds the hinges send
-// back to each edge (3 float4 per edge, accumulated with shared-memory atomics), kept in ten
-// per-edge arrays that the substep's reverse no longer uses when it reaches its hinges.
-struct EdgeDual {
-    float4 *tv, *td, *wv, *wd, *rv, *rd, *cs;   // t | ell, w0 | n1, d1r | c (values, derivatives); s
-    float4 *s0, *s1, *s2;                       // seeds: gt.v | gd1r.x.v, gt.d | gd1r.x.d, gd1r.yz (v, d)
-    __device__ __forceinline__ void store(int j, const EdgeF<dualf>& E) const {
-        tv[j] = make_float4(E.t.x.v, E.t.y.v, E.t.z.v, E.ell.v);
-        td[j] = make_float4(E.t.x.d, E.t.y.d, E.t.z.d, E.ell.d);
-        wv[j] = make_float4(E.w0.x.v, E.w0.y.v, E.w0.z.v, E.n1.v);
-        wd[j] = make_float4(E.w0.x.d, E.w0.y.d, E.w0.z.d, E.n1.d);
-        rv[j] = make_float4(E.d1r.x.v, E.d1r.y.v, E.d1r.z.v, E.c.v);
-        rd[j] = make_float4(E.d1r.x.d, E.d1r.y.d, E.d1r.z.d, E.c.d);
-        cs[j] = make_float4(E.s.v, E.s.d, 0.f, 0.f);
-    }
-    // what the hinge needs: t, d1r, d2r = t x d1r, the material frame (d1, d2) and (c, s)
-    __device__ __forceinline__ void load_frame(int j, EdgeF<dualf>& E) const {
-        const float4 a = tv[j], b = td[j], c = rv[j], d = rd[j], e = cs[j];
-        E.t = mk3(mkd(a.x, b.x), mkd(a.y, b.y), mkd(a.z, b.z));
-        E.d1r = mk3(mkd(c.x, d.x), mkd(c.y, d.y), mkd(c.z, d.z));
-        E.c = mkd(c.w, d.w);
-        E.s = mkd(e.x, e.y);
-        E.d2r = cross(E.t, E.d1r);
-        E.d1 = E.c * E.d1r + E.s * E.d2r;
-        E.d2 = E.c * E.d2r - E.s * E.d1r;
-    }
-    // what edge_reverse needs: t, w0, d1r, n1, ell
-    __device__ __forceinline__ void load_rev(int j, EdgeF<dualf>& E) const {
-        const float4 a = tv[j], b = td[j], c = wv[j], d = wd[j], e = rv[j], f = rd[j];
-        E.t = mk3(mkd(a.x, b.x), mkd(a.y, b.y), mkd(a.z, b.z));
-        E.ell = mkd(a.w, b.w);
-        E.w0 = mk3(mkd(c.x, d.x), mkd(c.y, d.y), mkd(c.z, d.z));
-        E.n1 = mkd(c.w, d.w);
-        E.d1r = mk3(mkd(e.x, f.x), mkd(e.y, f.y), mkd(e.z, f.z));
-    }
-    __device__ __forceinline__ void zero_seeds(int j) const {
-        s0[j] = s1[j] = s2[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    __device__ __forceinline__ void add_seeds(int j, V3<dualf> gt, V3<dualf> gr) const {
-        atomicAdd(&s0[j].x, gt.x.v);
-        atomicAdd(&s0[j].y, gt.y.v);
-        atomicAdd(&s0[j].z, gt.z.v);
-        atomicAdd(&s0[j].w, gr.x.v);
-        atomicAdd(&s1[j].x, gt.x.d);
-        atomicAdd(&s1[j].y, gt.y.d);
-        atomicAdd(&s1[j].z, gt.z.d);
-        atomicAdd(&s1[j].w, gr.x.d);
-        atomicAdd(&s2[j].x, gr.y.v);
-        atomicAdd(&s2[j].y, gr.z.v);
-        atomicAdd(&s2[j].z, gr.y.d);
-        atomicAdd(&s2[j].w, gr.z.d);
-    }
-    __device__ __forceinline__ void load_seeds(int j, V3<dualf>& gt, V3<dualf>& gr) const {
-        const float4 a = s0[j], b = s1[j], c = s2[j];
-        gt = mk3(mkd(a.x, b.x), mkd(a.y, b.y), mkd(a.z, b.z));
-        gr = mk3(mkd(a.w, b.w), mkd(c.x, c.z), mkd(c.y, c.w));
-    }
+// Pose cotangents of one substep and gripper (positions and rotations at the substep's start
+// and end, rigid velocities) -> the frame-start pose and the frame's actions.  acc: the thread's
+// 24 pose terms (positions 2 x 3, rotations 2 x 3, actions 2 x 6).  Only the threads of held
+// vertices and of vertices touching a gripper come here, so acc lives in local memory.
+static __device__ __noinline__ void fold_pose(float* acc, int q, const float* pm, float c0, float c1, float idt, V3<float> ps0,
+                                       V3<float> ph0, V3<float> ps1, V3<float> ph1, V3<float> vp, V3<float> w) {
+    auto add = [](float* o, V3<float> v) {
+        o[0] += v.x;
+        o[1] += v.y;
+        o[2] += v.z;
+    };
+    pm += 36 * q;
+    add(acc + 3 * q, ps0 + ps1);
+    add(acc + 6 + 3 * q, mul_rm_t(pm, ph0) + mul_rm_t(pm + 9, ph1));
+    add(acc + 12 + 6 * q, c0 * ps0 + c1 * ps1 + idt * vp);
+    add(acc + 15 + 6 * q, mul_rm(pm + 18, ph0) + mul_rm(pm + 27, ph1) + idt * w);
+}
+
+struct RevGrip {
+    V3<float> lx, lam;
 };
 
-// The values of a dual-number edge frame.
-__device__ __forceinline__ EdgeF<float> edge_vals(const EdgeF<dualf>& D) {
-    EdgeF<float> E;
-    E.t = vals(D.t);
-    E.w0 = vals(D.w0);
-    E.d1r = vals(D.d1r);
-    E.d2r = vals(D.d2r);
-    E.d1 = vals(D.d1);
-    E.d2 = vals(D.d2);
-    E.ell = D.ell.v;
-    E.n1 = D.n1.v;
-    E.c = D.c.v;
-    E.s = D.s.v;
-    return E;
+// d2r and the material directors of a frame from its tangent, first director and (cos, sin),
+// formed where the hinge needs them: as opaque values, or the compiler would carry an edge's own
+// 18 numbers across the barrier instead of forming them again (twice the spills).
+__device__ __forceinline__ void opaque(dualf& a) { asm volatile("" : "+f"(a.v), "+f"(a.d)); }
+__device__ __forceinline__ void material_frame(EdgeF<dualf>& E) {
+    opaque(E.t.x);
+    opaque(E.t.y);
+    opaque(E.t.z);
+    opaque(E.d1r.x);
+    opaque(E.d1r.y);
+    opaque(E.d1r.z);
+    opaque(E.c);
+    opaque(E.s);
+    E.d2r = cross(E.t, E.d1r);
+    E.d1 = E.c * E.d1r + E.s * E.d2r;
+    E.d2 = E.c * E.d2r - E.s * E.d1r;
+}
+
+// Reverse of an active gripper contact: the cotangents of the vertex position (to add) and of
+// the velocity before the contact; the pose cotangents go to acc.  Out of line: few vertices
+// touch a gripper, and inlined its registers would be every vertex's.
+static __device__ __noinline__ RevGrip gripper_reverse(const BwdParams& P, const RodInfo* Rp, const float* sp, const float* pm,
+                                                float* acc, int q, float c0, float c1, V3<float> x, V3<float> v,
+                                                V3<float> lam) {
+    const SceneDev& sc = P.scene;
+    const RodInfo& R = *Rp;
+    const float* o = sp + 32 * q;
+    const V3<float> gp = f3(o[0], o[1], o[2]), gax = f3(o[8], o[11], o[14]), vp = f3(o[24], o[25], o[26]),
+                    w = f3(o[27], o[28], o[29]);
+    RevGrip r;
+    V3<float> lp, lphi, lvp, lw, ntmp;
+    if (sdf_capsule(x, gp - sc.grip_hl * gax, gp + sc.grip_hl * gax, sc.grip_r, ntmp) > -sc.grip_r) {
+        capsule_contact_rev(x, v, gp, gax, sc.grip_hl, sc.grip_r, vp, w, R.radius, R.eps, sc.mu_rigid, sc.restitution,
+                            lam, r.lx, r.lam, lp, lphi, lvp, lw);
+    } else {   // the degenerate on-axis contact, by dual numbers, one input direction at a time
+        const int k = sc.n_planes + sc.n_boxes + q;
+        float lin[18];
+#pragma unroll 1
+        for (int d = 0; d < 18; ++d) {
+            V3<float> e = zf3();
+            (d % 3 == 0 ? e.x : d % 3 == 1 ? e.y : e.z) = 1.f;
+            const int g = d / 3;
+            bool on;
+            const V3<dualf> out = prim_respond<dualf>(
+                k, sc, R, lift(x, g == 0 ? e : zf3()), lift(v, g == 1 ? e : zf3()), lift(gp, g == 2 ? e : zf3()),
+                lift(gax, g == 3 ? cross(e, gax) : zf3()), lift(vp, g == 4 ? e : zf3()), lift(w, g == 5 ? e : zf3()), on);
+            lin[d] = dot(ders(out), lam);
+        }
+        r.lx = f3(lin[0], lin[1], lin[2]);
+        r.lam = f3(lin[3], lin[4], lin[5]);
+        lp = f3(lin[6], lin[7], lin[8]);
+        lphi = f3(lin[9], lin[10], lin[11]);
+        lvp = f3(lin[12], lin[13], lin[14]);
+        lw = f3(lin[15], lin[16], lin[17]);
+    }
+    fold_pose(acc, q, pm, c0, c1, 1.f / sc.dt, lp, lphi, zf3(), zf3(), lvp, lw);
+    return r;
+}
+
+// The k-th rigid primitive (planes, boxes, grippers) acting on a vertex velocity.
+__device__ __forceinline__ V3<float> respond_at(int k, const SceneDev& sc, const RodInfo& R, const float* sp, V3<float> x,
+                                                V3<float> v, bool& on) {
+    const int q = k - sc.n_planes - sc.n_boxes;
+    V3<float> gp = zf3(), gax = zf3(), vp = zf3(), w = zf3();
+    if (q >= 0) {
+        const float* o = sp + 32 * q;
+        gp = f3(o[0], o[1], o[2]);
+        gax = f3(o[8], o[11], o[14]);
+        vp = f3(o[24], o[25], o[26]);
+        w = f3(o[27], o[28], o[29]);
+    }
+    return prim_respond<float>(k, sc, R, x, v, gp, gax, vp, w, on);
+}
+
+// Reverse of the rigid contact of one vertex: from the cotangent lam of the velocity after it,
+// that of the velocity v1 before it; adds the position's to lx.
+__device__ __forceinline__ V3<float> rigid_reverse(const BwdParams& P, const RodInfo& R, const RodInfo* Rp, const float* sp,
+                                                   const float* pm, float* acc, float c0, float c1, V3<float> x,
+                                                   V3<float> v1, V3<float> lam, V3<float>& lx, bool& touched) {
+    const SceneDev& sc = P.scene;
+    const int nprim = sc.n_planes + sc.n_boxes + R.ngrip;
+    unsigned mask = 0;
+    V3<float> v = v1, vb = v1;   // vb: the velocity before the last active primitive
+#pragma unroll 1
+    for (int k = 0; k < nprim; ++k) {
+        bool on;
+        const V3<float> nxt = respond_at(k, sc, R, sp, x, v, on);
+        if (on) {
+            mask |= 1u << k;
+            vb = v;
+        }
+        v = nxt;
+    }
+    while (mask) {
+        const int k = 31 - __clz(mask), q = k - sc.n_planes - sc.n_boxes;
+        mask ^= 1u << k;
+        if (q >= 0) {
+            const RevGrip r = gripper_reverse(P, Rp, sp, pm, acc, q, c0, c1, x, vb, lam);
+            lx += r.lx;
+            lam = r.lam;
+            touched = true;
+        } else if (k < sc.n_planes) {   // sdf = n.x - o, constant n
+            const V3<float> n = f3(sc.planes[k]);
+            V3<float> lv, ln, lvr;
+            float lsdf;
+            contact_respond_rev(vb, dot(x, n) - sc.planes[k].w, n, zf3(), R.radius, R.eps, sc.mu_rigid, sc.restitution,
+                                lam, lv, lsdf, ln, lvr);
+            lx += lsdf * n;
+            lam = lv;
+        } else {
+            const int bi = k - sc.n_planes;
+            V3<float> lv;
+            lx += box_contact_rev(x, vb, f3(sc.box_c[bi]), f3(sc.box_h[bi]), R.radius, R.eps, sc.mu_rigid,
+                                  sc.restitution, lam, lv);
+            lam = lv;
+        }
+        if (mask) {   // several at once (rare): the velocity before the one below, again from v1
+            const int top = 31 - __clz(mask);
+            vb = v1;
+            for (int j = 0; j < top; ++j) {
+                bool on;
+                if ((mask >> j) & 1u) vb = respond_at(j, sc, R, sp, x, vb, on);
+            }
+        }
+    }
+    return lam;
+}
+
+// Adds v to the unevaluated sum s.x + s.y (Knuth's exact two-term sum): what FP64 addition gave
+// these strongly cancelling sums, on the FP32 pipe (an FP64 addition and its conversion take 16
+// cycles of the SM each).
+__device__ __forceinline__ void add_comp(float2* s, float v) {
+    float2 a = *s;
+    const float t = __fadd_rn(a.x, v), b = __fsub_rn(t, a.x);
+    const float e = __fadd_rn(__fsub_rn(a.x, __fsub_rn(t, b)), __fsub_rn(v, b));
+    *s = make_float2(t, __fadd_rn(a.y, e));
+}
+
+// A rod's cotangents as a thread holds them for its own vertex, edge and hinge.
+struct Cot {
+    V3<float> x, v, d1, t;     // position, velocity, base director, base tangent
+    float om, th, k0, k1;      // twist rate, twist angle, rest curvature
+};
+
+// Threads that reverse a rod's length projections: thread t takes the edges 2t and 2t + 1.
+__host__ __device__ constexpr int pbd_threads(int NV) { return NV <= 64 ? 32 : (NV / 2 + 31) / 32 * 32; }
+constexpr int kPbdBar = 2;   // their named barrier (the rod's own is 1)
+
+template <int NV>
+__device__ __forceinline__ void pbd_sync() {
+    if (pbd_threads(NV) == 32)
+        __syncwarp();
+    else
+        asm volatile("bar.sync %0, %1;" ::"r"(kPbdBar), "r"(pbd_threads(NV)) : "memory");
+}
+
+// The two edges of a projecting thread and their running sums of cotangents.
+struct PbdRev {
+    bool e0, e1, ring;         // edge 2t, edge 2t + 1 are projected; edge 2t is an odd loop's last (its own colour)
+    int i0, i2;                // vertices 2t and the end of edge 2t + 1
+    float a0, b0, a1, b1;      // w_a / (w_a + w_b), w_b / (w_a + w_b) of both
+    V3<float> s0, s1;          // sums over the iterations
+};
+
+// One projection reversed, from its record q (unit direction t, ratio r = target / length): it
+// moved its ends by -+ w lambda t, lambda = (l - target) / (w_a + w_b).  A record that did
+// nothing, (0, 0, 0, 1), gives zero.
+__device__ __forceinline__ V3<float> project_rev(float4 q, float a, float b, V3<float> la, V3<float> lb) {
+    const V3<float> t = f3(q);
+    const V3<float> mu = a * la - b * lb;
+    return mu - q.w * (mu - dot(mu, t) * t);
 }
 
 // ------------------------------------------------------------------ reverse of one substep
-// On entry the shared state holds S_n (the substep's start), the recorded intermediates and,
-// for a self-contact rod, the frame's pair list and the projection data of the first
-// iteration; the cotangent arrays hold the cotangents of S_{n+1}.  On exit they hold those
-// of S_n.  PBD: the substep's projection records ([n_iter][NV], see Rec::pbd); CSN: its
-// displacements before each contact sweep ([n_iter][NV]).  gm accumulates (kA, Bm, beta,
-// sigma_y, c_d) cotangents, lpf/lphif the frame-start pose cotangents and ga the frame's
-// action cotangents (all per g.tid).
-template <int NV, bool CONTACT, int TPR>
-__device__ __noinline__ void reverse_substep(const BwdParams& P, const RodInfo& R, Smem<NV, CONTACT>& s,
-                                AdjArrays<NV, CONTACT>& a, const float4* PBD, const float4* CSN, const Grp<TPR>& g,
-                                float h, float c0, float c1, int np,
-                                double* gm, float* lpf, float* lphif, float* ga) {
+// rec: the substep's records.  c holds the cotangents of S_{n+1} on entry and of S_n on exit.
+// sp, pm: the substep's gripper block and pose maps; acc: the thread's pose terms.
+// Bound by latency: dependent arithmetic of few warps (registers), barriers and record loads.
+// Each thread keeps its vertex's, edge's and hinge's data in registers from phase to phase; a
+// thread's local memory holds only the pose terms, which few threads touch.
+template <int NV, bool CONTACT>
+__device__ __forceinline__ void reverse_substep(const BwdParams& P, const RodInfo& R, const RodInfo* Rp, const Own& own,
+                                                float4 kin, float eb, float eba, RevSmem<NV, CONTACT>& s,
+                                                const Grp<NV>& g, const Rec<NV, true> rec, float h, float c0, float c1,
+                                                int np, const float* sp, const float* pm, Cot& c, float* acc,
+                                                bool& touched) {
     const SceneDev& sc = P.scene;
-    const int nv = R.nv, ne = R.ne, v0 = R.v0, e0 = R.e0;
+    const int nv = R.nv, ne = R.ne, i = g.tid;
     const bool closed = R.flags & ROD_CLOSED;
-    const int nh = closed ? nv : nv - 2;
     const float ih = 1.f / h;
     const bool lenc = R.flags & (ROD_INEXT | ROD_SLIMIT);
-    const float rsum = 2.f * R.radius;
-    PoseAdj pa;
-    pa.zero();
-    // this substep's material terms, in registers (gm is the caller's memory), added to gm at
-    // the end
-    double gl[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    for (int i = g.tid; i < nv; i += TPR) a.LP0[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    // ---- B1: positions at the substep end
-    for (int i = g.tid; i < nv; i += TPR) {
-        const float4 kin = P.KIN[v0 + i];
-        const int kind = (int)kin.w;
-        float4 lx = a.LX[i];
-        if (kind >= 2 && in_bounds(kind - 2 < R.ngrip, s.red)) {
-            const int q = kind - 2;
-            V3<float> y1 = mul_rm(s.sp + 32 * q + 15, f3(kin));
-            add3(pa.ps1, q, f3(lx));
-            add3(pa.phs1, q, cross(y1, f3(lx)));
-            a.LX[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-            a.LD[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        } else {
-            a.LD[i] = make_float4(lx.x, lx.y, lx.z, 0.f);
-        }
+    const bool project = lenc || (CONTACT && np > 0);
+    const bool vtx = i < nv, has_e = i < ne, has_em = vtx && (closed || i > 0);
+    const bool strands = R.flags & ROD_STRANDS;
+    const bool real = has_e && !(strands && !(eb > 0.f));
+    const int ip = (i + 1 == nv) ? 0 : i + 1, im = (i == 0) ? nv - 1 : i - 1;
+    const float4* S = rec.base;
+    float4 x4 = make_float4(0.f, 0.f, 0.f, 0.f), v4 = x4, xb = x4, hg = x4, ed = x4, et = x4, v1 = x4;
+    float tha = 0.f;
+    if (vtx) {
+        x4 = S[i];
+        v4 = S[NV + i];
+        v1 = rec.v1()[i];
     }
-    g.sync();
-    // ---- B2: self-contact friction
-    if (CONTACT && np > 0) {
-        // displacements at the first contact sweep (after the colours of iteration 0)
-        const float4* T0 = CSN;
-        float4* LTMP = s.HB0;
-        for (int i = g.tid; i < nv; i += TPR) LTMP[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (has_e) {
+        xb = S[ip];
+        ed = S[3 * NV + i];
+        et = S[4 * NV + i];
+    }
+    if (has_em) {
+        hg = S[2 * NV + i];
+        tha = S[3 * NV + im].w;
+    }
+    g.sync();   // LD of the substep after this one has been read; its frame's shared data is written
+    // ---- positions at the substep end, and the velocity rebuilt from the displacement
+    const bool held = own.kind >= 2;
+    V3<float> ld = held ? zf3() : c.x, dx = zf3(), lp0 = zf3();
+    if (CONTACT && np > 0) {   // self-contact friction
+        const float4* T0 = rec.csnap(0);   // displacements at the first contact sweep
+        const float4 *DF = rec.dfin(), *FR1 = rec.fr1();
+        if (vtx) {
+            s.F1[i] = f4(c.v, 0.f);
+            s.F2[i] = s.F3[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
         g.sync();
-        for (int p = g.tid; p < np; p += TPR) {
-            if (!(s.fr1[p].w > 0.f)) continue;
-            uint32_t pr = s.pairs[p];
+        for (int p = g.tid; p < np; p += NV) {
+            if (!(FR1[p].w > 0.f)) continue;
+            const uint32_t pr = s.pairs[p];
             const int a0 = pr & 0xffff, q0 = pr >> 16;
             if (!in_bounds(a0 < nv && q0 < nv, s.red)) continue;
             const int idx[4] = {a0, (a0 + 1 == nv) ? 0 : a0 + 1, q0, (q0 + 1 == nv) ? 0 : q0 + 1};
-            const V3<float> o = f3(s.X0[a0]);
+            const V3<float> o = f3(S[a0]);
             V3<float> Pf[4], Vf[4], lo[4];
             float w[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                Pf[k] = (k == 0) ? f3(T0[idx[0]]) : (f3(s.X0[idx[k]]) - o) + f3(T0[idx[k]]);
-                Vf[k] = ih * f3(a.DF[idx[k]]);
-                w[k] = s.X0[idx[k]].w;
-                lo[k] = f3(a.LV[idx[k]]);
+                const float4 xk = S[idx[k]];
+                Pf[k] = (k == 0) ? f3(T0[idx[0]]) : (f3(xk) - o) + f3(T0[idx[k]]);
+                Vf[k] = ih * f3(DF[idx[k]]);
+                w[k] = xk.w;
+                lo[k] = f3(s.F1[idx[k]]);
             }
             V3<float> pb[4], vb[4];
-            if (fric_pair_vjp(Pf, Vf, w, rsum, sc.mu_self, h, lo, pb, vb))
+            if (fric_pair_vjp(Pf, Vf, w, 2.f * R.radius, sc.mu_self, h, lo, pb, vb))
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    atomic_add3(&a.LP0[idx[k]], pb[k]);
-                    atomic_add3(&LTMP[idx[k]], vb[k]);
+                    atomic_add3(&s.F2[idx[k]], pb[k]);
+                    atomic_add3(&s.F3[idx[k]], vb[k]);
                 }
         }
         g.sync();
-        for (int i = g.tid; i < nv; i += TPR) {
-            float4 l = a.LV[i], t = LTMP[i];
-            a.LV[i] = make_float4(l.x + t.x, l.y + t.y, l.z + t.z, l.w);
+        if (vtx) {
+            lp0 = f3(s.F2[i]);
+            c.v += f3(s.F3[i]);
         }
-        g.sync();
     }
-    // ---- B3: velocity rebuilt from the displacement
-    for (int i = g.tid; i < nv; i += TPR) {
-        const float4 kin = P.KIN[v0 + i];
-        const int kind = (int)kin.w;
-        (void)kin;
-        (void)kind;
-        float4 l = a.LV[i];
-        V3<float> lv = ih * f3(l);
-        float4 d = a.LD[i];
-        a.LD[i] = make_float4(d.x + lv.x, d.y + lv.y, d.z + lv.z, 0.f);
-        a.LV[i] = make_float4(0.f, 0.f, 0.f, l.w);
-    }
-    g.sync();
-    // ---- B4: PBD iterations in reverse
-    if (lenc || (CONTACT && np > 0)) {
+    ld += ih * c.v;
+    // ---- projections in reverse
+    if (project) {
+        constexpr int PT = pbd_threads(NV);
         const int ncol = lenc ? ((closed && (ne & 1)) ? 3 : 2) : 0;
+        const bool proj = lenc && i < PT;
+        PbdRev b{};
+        float4 q0 = make_float4(0.f, 0.f, 0.f, 1.f), q1 = q0;
+        if (proj) {
+            const int j = 2 * i;
+            b.e0 = j < ne;
+            b.e1 = j + 1 < ne;
+            b.ring = ncol == 3 && j == ne - 1;
+            b.i0 = min(j, nv - 1);
+            b.i2 = j + 2 >= nv ? 0 : j + 2;
+            const float4* W = S;
+            const float w0 = b.e0 ? W[j].w : 0.f, w1 = b.e0 ? W[j + 1 == nv ? 0 : j + 1].w : 0.f,
+                        w2 = b.e1 ? W[b.i2].w : 0.f;
+            b.a0 = w0 + w1 > 0.f ? w0 / (w0 + w1) : 0.f;
+            b.b0 = w0 + w1 > 0.f ? w1 / (w0 + w1) : 0.f;
+            b.a1 = w1 + w2 > 0.f ? w1 / (w1 + w2) : 0.f;
+            b.b1 = w1 + w2 > 0.f ? w2 / (w1 + w2) : 0.f;
+            b.s0 = b.s1 = zf3();
+            const float4* Q = rec.pbd(sc.n_iter - 1);
+            if (b.e0) q0 = Q[j];
+            if (b.e1) q1 = Q[j + 1];
+        }
+        if (vtx) s.LD[i] = f4(ld, 0.f);
+        g.sync();
         for (int it = sc.n_iter - 1; it >= 0; --it) {
             if (CONTACT && np > 0) {
-                const float4* Dc = CSN + (size_t)it * NV;   // displacements before the contact sweep
-                float4* LTMP = a.LG;
-                for (int i = g.tid; i < nv; i += TPR) LTMP[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                const float4* Dc = rec.csnap(it);   // displacements before the contact sweep
+                if (vtx) s.F3[i] = make_float4(0.f, 0.f, 0.f, 0.f);
                 g.sync();
-                for (int p = g.tid; p < np; p += TPR) {
-                    uint32_t pr = s.pairs[p];
-                    const int a0 = pr & 0xffff, q0 = pr >> 16;
-                    if (!in_bounds(a0 < nv && q0 < nv, s.red)) continue;
-                    const int idx[4] = {a0, (a0 + 1 == nv) ? 0 : a0 + 1, q0, (q0 + 1 == nv) ? 0 : q0 + 1};
-                    const V3<float> o = f3(s.X0[a0]);
+                for (int p = g.tid; p < np; p += NV) {
+                    const uint32_t pr = s.pairs[p];
+                    const int a0 = pr & 0xffff, c0_ = pr >> 16;
+                    if (!in_bounds(a0 < nv && c0_ < nv, s.red)) continue;
+                    const int idx[4] = {a0, (a0 + 1 == nv) ? 0 : a0 + 1, c0_, (c0_ + 1 == nv) ? 0 : c0_ + 1};
+                    const V3<float> o = f3(S[a0]);
                     V3<float> Pf[4], lo[4];
                     float w[4];
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
-                        Pf[k] = (k == 0) ? f3(Dc[idx[0]]) : (f3(s.X0[idx[k]]) - o) + f3(Dc[idx[k]]);
-                        w[k] = s.X0[idx[k]].w;
-                        lo[k] = f3(a.LD[idx[k]]);
+                        const float4 xk = S[idx[k]];
+                        Pf[k] = (k == 0) ? f3(Dc[idx[0]]) : (f3(xk) - o) + f3(Dc[idx[k]]);
+                        w[k] = xk.w;
+                        lo[k] = f3(s.LD[idx[k]]);
                     }
                     V3<float> pb[4];
-                    if (pair_correction_vjp(Pf, w, rsum, lo, pb))
+                    if (pair_correction_vjp(Pf, w, 2.f * R.radius, lo, pb))
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) atomic_add3(&LTMP[idx[k]], pb[k]);
+                        for (int k = 0; k < 4; ++k) atomic_add3(&s.F3[idx[k]], pb[k]);
                 }
                 g.sync();
-                for (int i = g.tid; i < nv; i += TPR) {
-                    float4 t = LTMP[i];
-                    if (it == 0) {
-                        float4 q = a.LP0[i];
-                        t = make_float4(t.x + q.x, t.y + q.y, t.z + q.z, 0.f);
+                if (vtx) {
+                    V3<float> t = f3(s.F3[i]);
+                    if (it == 0) t += lp0;
+                    s.LD[i] = f4(f3(s.LD[i]) + t, 0.f);
+                    dx += t;
+                }
+                g.sync();
+            }
+            if (proj) {
+                // the records of the iteration before, fetched while this one is reversed
+                const float4 r0 = q0, r1 = q1;
+                if (it > 0) {
+                    const float4* Q = rec.pbd(it - 1);
+                    if (b.e0) q0 = Q[2 * i];
+                    if (b.e1) q1 = Q[2 * i + 1];
+                }
+                if (ncol == 3) {
+                    if (b.ring) {
+                        const V3<float> la = f3(s.LD[b.i0]), lb = f3(s.LD[0]);
+                        const V3<float> le = project_rev(r0, b.a0, b.b0, la, lb);
+                        s.LD[b.i0] = f4(la - le, 0.f);
+                        s.LD[0] = f4(lb + le, 0.f);
+                        b.s0 += le;
                     }
-                    float4 ld = a.LD[i], lx = a.LX[i];
-                    a.LD[i] = make_float4(ld.x + t.x, ld.y + t.y, ld.z + t.z, 0.f);
-                    a.LX[i] = make_float4(lx.x + t.x, lx.y + t.y, lx.z + t.z, 0.f);
+                    pbd_sync<NV>();
                 }
-                g.sync();
+                // vertex 2t + 1 belongs to this thread's two edges alone
+                V3<float> lm = b.e0 && !b.ring ? f3(s.LD[2 * i + 1]) : zf3();
+                if (b.e1) {
+                    const V3<float> lb = f3(s.LD[b.i2]);
+                    const V3<float> le = project_rev(r1, b.a1, b.b1, lm, lb);
+                    lm = lm - le;
+                    s.LD[b.i2] = f4(lb + le, 0.f);
+                    b.s1 += le;
+                }
+                pbd_sync<NV>();
+                if (b.e0 && !b.ring) {
+                    const V3<float> la = f3(s.LD[b.i0]);
+                    const V3<float> le = project_rev(r0, b.a0, b.b0, la, lm);
+                    s.LD[b.i0] = f4(la - le, 0.f);
+                    s.LD[2 * i + 1] = f4(lm + le, 0.f);
+                    b.s0 += le;
+                }
+                pbd_sync<NV>();
             }
-            // colours in reverse, from each edge's record (unit direction t, ratio r = target /
-            // length): the projection moved its ends by -+ w lambda t, lambda = (l - target) / ws
-            const float4* Q = PBD + (size_t)it * NV;
-            for (int k = ncol - 1; k >= 0; --k) {
-                int first, last;
-                color_range(ne, closed, k, first, last);
-                for (int j = first + 2 * g.tid; j < last; j += 2 * TPR) {
-                    const int j1 = (j + 1 == nv) ? 0 : j + 1;
-                    const float4 q = Q[j];
-                    if (q.x == 0.f && q.y == 0.f && q.z == 0.f) continue;   // the projection did nothing
-                    const float wa = s.X0[j].w, wb = s.X0[j1].w, ws = wa + wb;
-                    const V3<float> t = f3(q);
-                    V3<float> la = f3(a.LD[j]), lb = f3(a.LD[j1]);
-                    V3<float> mu = (wa / ws) * la - (wb / ws) * lb;
-                    V3<float> le = mu - q.w * (mu - dot(mu, t) * t);
-                    a.LD[j] = f4(la - le, 0.f);
-                    a.LD[j1] = f4(lb + le, 0.f);
-                    a.LX[j] = f4(f3(a.LX[j]) - le, 0.f);
-                    a.LX[j1] = f4(f3(a.LX[j1]) + le, 0.f);
-                }
-                g.sync();
+            if (CONTACT && np > 0) g.sync();
+        }
+        if (proj) {   // F0: each edge's summed cotangent
+            if (b.e0) s.F0[2 * i] = f4(b.s0, 0.f);
+            if (b.e1) s.F0[2 * i + 1] = f4(b.s1, 0.f);
+        }
+        g.sync();
+        if (vtx) {
+            ld = f3(s.LD[i]);
+            if (lenc) {
+                if (has_e) dx -= f3(s.F0[i]);
+                if (has_em) dx += f3(s.F0[im]);
             }
         }
     }
-    // ---- B5: vertex phase (rigid contact, symplectic Euler, gravity, damping, twist rate)
-    for (int i = g.tid; i < nv; i += TPR) {
-        const float4 kin = P.KIN[v0 + i];
-        const int kind = (int)kin.w;
-        const float4 x4 = s.X0[i];
-        const float4 vn = s.V[i];
-        V3<float> ld0 = f3(a.LD[i]);
-        float4 lvn = make_float4(0.f, 0.f, 0.f, 0.f), lg = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (kind == 0) {
-            V3<float> lam = h * ld0;
-            // forward sequence of the rigid primitives from the recorded pre-contact velocity
-            const int nprim = sc.n_planes + sc.n_boxes + R.ngrip;
-            V3<float> vs[kMaxPlanes + kMaxBoxes + 2];
-            vs[0] = f3(a.V1[i]);
-            const V3<float> x = f3(x4);
-            unsigned onmask = 0;
-            for (int k = 0; k < nprim; ++k) {
-                const int q = k - sc.n_planes - sc.n_boxes;
-                V3<float> gp = zf3(), gax = zf3(), vp = zf3(), w = zf3();
-                if (q >= 0) {
-                    const float* o = s.sp + 32 * q;
-                    gp = f3(o[0], o[1], o[2]);
-                    gax = f3(o[8], o[11], o[14]);
-                    vp = f3(o[24], o[25], o[26]);
-                    w = f3(o[27], o[28], o[29]);
-                }
-                bool on;
-                V3<float> nxt = prim_respond<float>(k, sc, R, x, vs[k], gp, gax, vp, w, on);
-                if (on) onmask |= 1u << k;
-                if (k + 1 < kMaxPlanes + kMaxBoxes + 2) vs[k + 1] = nxt;
-            }
-            V3<float> lx_acc = zf3();
-            for (int k = nprim - 1; k >= 0; --k) {
-                if (!((onmask >> k) & 1u)) continue;
-                const int q = k - sc.n_planes - sc.n_boxes;
-                V3<float> gp = zf3(), gax = zf3(), vp = zf3(), w = zf3();
-                if (q >= 0) {
-                    const float* o = s.sp + 32 * q;
-                    gp = f3(o[0], o[1], o[2]);
-                    gax = f3(o[8], o[11], o[14]);
-                    vp = f3(o[24], o[25], o[26]);
-                    w = f3(o[27], o[28], o[29]);
-                }
-                V3<float> ntmp;
-                if (q >= 0 && sdf_capsule(x, gp - sc.grip_hl * gax, gp + sc.grip_hl * gax, sc.grip_r, ntmp) > -sc.grip_r) {
-                    // capsule gripper: closed-form reverse (the degenerate on-axis case keeps dual numbers)
-                    V3<float> lxk, lvk, lpk, lphik, lvpk, lwk;
-                    capsule_contact_rev(x, vs[k], gp, gax, sc.grip_hl, sc.grip_r, vp, w, R.radius, R.eps,
-                                        sc.mu_rigid, sc.restitution, lam, lxk, lvk, lpk, lphik, lvpk, lwk);
-                    lx_acc += lxk;
-                    lam = lvk;
-                    add3(pa.ps0, q, lpk);
-                    add3(pa.phs0, q, lphik);
-                    add3(pa.vp, q, lvpk);
-                    add3(pa.w, q, lwk);
-                    continue;
-                }
-                if (k < sc.n_planes) {   // plane: closed-form reverse (sdf = n.x - o, constant n)
-                    const V3<float> n = f3(sc.planes[k]);
-                    V3<float> lv, ln, lvr;
-                    float lsdf;
-                    contact_respond_rev(vs[k], dot(x, n) - sc.planes[k].w, n, zf3(), R.radius, R.eps, sc.mu_rigid,
-                                        sc.restitution, lam, lv, lsdf, ln, lvr);
-                    lx_acc += lsdf * n;
-                    lam = lv;
-                    continue;
-                }
-                if (q < 0) {   // box: closed-form reverse
-                    const int bi = k - sc.n_planes;
-                    V3<float> lv;
-                    lx_acc += box_contact_rev(x, vs[k], f3(sc.box_c[bi]), f3(sc.box_h[bi]), R.radius, R.eps,
-                                              sc.mu_rigid, sc.restitution, lam, lv);
-                    lam = lv;
-                    continue;
-                }
-                const int nin = 18;   // the degenerate on-axis gripper contact keeps dual numbers
-                float lin[18];
-#pragma unroll 1
-                for (int d = 0; d < nin; ++d) {
-                    V3<float> e = zf3();
-                    (d % 3 == 0 ? e.x : d % 3 == 1 ? e.y : e.z) = 1.f;
-                    const int g = d / 3;
-                    V3<dualf> xd = lift(x, g == 0 ? e : zf3()), vd = lift(vs[k], g == 1 ? e : zf3());
-                    V3<dualf> gpd = lift(gp, g == 2 ? e : zf3()), gaxd = lift(gax, g == 3 ? cross(e, gax) : zf3());
-                    V3<dualf> vpd = lift(vp, g == 4 ? e : zf3()), wd = lift(w, g == 5 ? e : zf3());
-                    bool on2;
-                    V3<dualf> out = prim_respond<dualf>(k, sc, R, xd, vd, gpd, gaxd, vpd, wd, on2);
-                    lin[d] = dot(ders(out), lam);
-                }
-                lx_acc += f3(lin[0], lin[1], lin[2]);
-                lam = f3(lin[3], lin[4], lin[5]);
-                add3(pa.ps0, q, f3(lin[6], lin[7], lin[8]));
-                add3(pa.phs0, q, f3(lin[9], lin[10], lin[11]));
-                add3(pa.vp, q, f3(lin[12], lin[13], lin[14]));
-                add3(pa.w, q, f3(lin[15], lin[16], lin[17]));
-            }
+    // ---- vertex phase (rigid contact, symplectic Euler, gravity, damping, twist rate)
+    float4 lg = make_float4(0.f, 0.f, 0.f, 0.f);
+    float m_cd = 0.f;
+    if (vtx) {
+        V3<float> lx = held ? dx : c.x + dx, lv = zf3();
+        if (own.kind == 0) {
+            V3<float> lam = h * ld;
+            lam = rigid_reverse(P, R, Rp, sp, pm, acc, c0, c1, f3(x4), f3(v1), lam, lx, touched);
             // v1 = v + h (-w g + gravity - c_d v)
-            const float wi = x4.w;
-            lvn = f4((1.f - h * R.cd) * lam, 0.f);
-            lg = f4((-h * wi) * lam, 0.f);
-            gl[4] += (double)(-h * dot(f3(vn), lam));
-            a.LX[i] = f4(f3(a.LX[i]) + lx_acc, 0.f);
-        } else if (kind >= 2 && in_bounds(kind - 2 < R.ngrip, s.red)) {
-            // d = target(pose at the substep end) - x0
-            const int q = kind - 2;
-            add3(pa.ps1, q, ld0);
-            add3(pa.phs1, q, cross(mul_rm(s.sp + 32 * q + 15, f3(kin)), ld0));
-            a.LX[i] = f4(f3(a.LX[i]) - ld0, 0.f);
+            lv = (1.f - h * R.cd) * lam;
+            const V3<float> l = (-h * x4.w) * lam;
+            lg = f4(l, 0.f);
+            m_cd = -h * dot(f3(v4), lam);
+        } else if (held && in_bounds(own.kind - 2 < R.ngrip, s.red)) {
+            // x = target and d = target - x0, the target moving with the gripper's end pose
+            const int q = own.kind - 2;
+            const V3<float> y1 = mul_rm(sp + 32 * q + 15, f3(kin)), l = c.x + ld;
+            fold_pose(acc, q, pm, c0, c1, 1.f / sc.dt, zf3(), zf3(), l, cross(y1, l), zf3(), zf3());
+            touched = true;
+            lx -= ld;
         }
-        const bool has_e = closed || i < nv - 1;
+        c.x = lx;
+        c.v = lv;
         if (has_e) {
-            const float lw1 = a.LV[i].w + h * a.LE[i].w;     // d theta_{n+1} / d omega_1 = h
-            const float invI = P.ES[e0 + i].y;
-            lvn.w = (1.f - h * R.cd) * lw1;
-            lg.w = -h * invI * lw1;
-            gl[4] += (double)(-h * vn.w * lw1);
+            const float lw1 = c.om + h * c.th;     // d theta_{n+1} / d omega_1 = h
+            c.om = (1.f - h * R.cd) * lw1;
+            lg.w = -h * own.invI * lw1;
+            m_cd -= h * v4.w * lw1;
+        } else {
+            c.om = 0.f;
         }
-        a.LV[i] = lvn;
-        a.LG[i] = lg;
+        s.LD[i] = lg;
     }
     g.sync();
-    // ---- pose cotangents of this substep -> frame-start pose and the frame's actions (pa is
-    // complete after B5; folding it here ends its registers' life before B8 and B7).  Only
-    // grasped vertices and vertices touching a gripper have any; the maps are a.PM's.
-    const float idt = 1.f / sc.dt;
-    for (int q = 0; q < R.ngrip; ++q) {
-        const V3<float> ps0 = get3(pa.ps0, q), ps1 = get3(pa.ps1, q), vp = get3(pa.vp, q);
-        const V3<float> ph0 = get3(pa.phs0, q), ph1 = get3(pa.phs1, q), w = get3(pa.w, q);
-        const bool nz = ps0.x != 0.f || ps0.y != 0.f || ps0.z != 0.f || ps1.x != 0.f || ps1.y != 0.f ||
-                        ps1.z != 0.f || vp.x != 0.f || vp.y != 0.f || vp.z != 0.f || ph0.x != 0.f ||
-                        ph0.y != 0.f || ph0.z != 0.f || ph1.x != 0.f || ph1.y != 0.f || ph1.z != 0.f ||
-                        w.x != 0.f || w.y != 0.f || w.z != 0.f;
-        if (!nz) continue;
-        const float* pm = a.PM + 36 * q;
-        add3(lpf, q, ps0 + ps1);
-        const V3<float> gdp = c0 * ps0 + c1 * ps1 + idt * vp;
-        const V3<float> gdr = mul_rm(pm + 18, ph0) + mul_rm(pm + 27, ph1) + idt * w;
-        ga[6 * q] += gdp.x;
-        ga[6 * q + 1] += gdp.y;
-        ga[6 * q + 2] += gdp.z;
-        ga[6 * q + 3] += gdr.x;
-        ga[6 * q + 4] += gdr.y;
-        ga[6 * q + 5] += gdr.z;
-        const V3<float> m0 = f3(pm[0] * ph0.x + pm[3] * ph0.y + pm[6] * ph0.z,
-                                pm[1] * ph0.x + pm[4] * ph0.y + pm[7] * ph0.z,
-                                pm[2] * ph0.x + pm[5] * ph0.y + pm[8] * ph0.z);
-        const V3<float> m1 = f3(pm[9] * ph1.x + pm[12] * ph1.y + pm[15] * ph1.z,
-                                pm[10] * ph1.x + pm[13] * ph1.y + pm[16] * ph1.z,
-                                pm[11] * ph1.x + pm[14] * ph1.y + pm[17] * ph1.z);
-        add3(lphif, q, m0 + m1);
-    }
-    // ---- B8: per edge, the reverse of the new reference-frame base and the stretching second
-    // order; and the edge's frame as dual numbers in the direction of the force cotangents LG,
-    // once per edge, for the hinge phase (B7).  Arrays dead after B5 hold the dual frames
-    // (EdgeDual) and the seeds the two hinges of an edge send back to it (zeroed here).
-    const bool strands = R.flags & ROD_STRANDS;
-    const EdgeDual ES{a.LD, a.LP0, a.V1, a.DF, s.X, s.V, s.HB0, s.HB1, s.HB2, s.ND};
-    // Each thread keeps its edges' position cotangents (this phase's and B7's) in registers and
-    // adds them up per vertex in a fixed order at the end: no floating-point atomics, so the
-    // reverse of a substep without contact candidates is bitwise reproducible.
-    constexpr int EPT = (NV + TPR - 1) / TPR;   // edges per thread
-    V3<float> le_keep[EPT];
-#pragma unroll
-    for (int m = 0; m < EPT; ++m) {
-        const int j = g.tid + m * TPR;
-        le_keep[m] = zf3();
-        if (j >= ne) continue;
-        const int j1 = (j + 1 == nv) ? 0 : j + 1;
-        const float4 ed = s.ED[j], et = s.ET[j];
-        ES.zero_seeds(j);
-        if (strands && !(et.w > 0.f)) continue;   // a break edge kept its base frame: identity reverse
-        const float4 lga = a.LG[j], lgb = a.LG[j1];
-        EdgeF<dualf> Ed;
-        edge_forward(Ed, lift(f3(s.X0[j]), f3(lga)), lift(f3(s.X0[j1]), f3(lgb)), lift(f3(et)), lift(f3(ed)),
-                     mkd(ed.w, lga.w));
-        ES.store(j, Ed);
-        const EdgeF<float> E = edge_vals(Ed);
-        V3<float> gtb, gd1b;
-        V3<float> le = edge_reverse<float, true>(E, f3(et), f3(ed), f3(a.LT[j]), f3(a.LE[j]), 0.f, &gtb, &gd1b);
+    // ---- the own edge's frame as dual numbers in the direction of the force cotangents, the
+    // reverse of its stretching
+    EdgeF<dualf> E;
+    V3<float> tot = zf3();
+    float m_K = 0.f;
+    if (real) {
+        const float4 lgb = s.LD[ip];
+        edge_forward(E, lift(f3(x4), f3(lg)), lift(f3(xb), f3(lgb)), lift(f3(et)), lift(f3(ed)), mkd(ed.w, lg.w));
+        s.F0[i] = make_float4(E.t.x.v, E.t.y.v, E.t.z.v, E.c.v);
+        s.F1[i] = make_float4(E.t.x.d, E.t.y.d, E.t.z.d, E.c.d);
+        s.F2[i] = make_float4(E.d1r.x.v, E.d1r.y.v, E.d1r.z.v, E.s.v);
+        s.F3[i] = make_float4(E.d1r.x.d, E.d1r.y.d, E.d1r.z.d, E.s.d);
         if (R.kA > 0.f) {
-            const V3<float> les = f3(lgb) - f3(lga);
-            const float eb = P.ES[e0 + j].x;
-            const float tl = dot(E.t, les);
-            const float st = edge_strain(f3(s.X0[j1]) - f3(s.X0[j]), eb);
-            le += R.kA * ((tl / eb) * E.t + st / E.ell * (les - tl * E.t));
-            gl[0] += (double)(st * tl);
+            const V3<float> les = f3(lgb) - f3(lg), t = vals(E.t);
+            const float tl = dot(t, les);
+            const float st = edge_strain(f3(xb) - f3(x4), eb);
+            tot = R.kA * ((tl / eb) * t + st / E.ell.v * (les - tl * t));
+            m_K = st * tl;
         }
-        le_keep[m] = le;
-        a.LT[j] = f4(gtb, 0.f);
-        a.LE[j] = f4(gd1b, a.LE[j].w);
     }
+    const float lga_w = has_em ? s.LD[im].w : 0.f;   // the previous edge's twist-angle direction
     g.sync();
-    // ---- B7: hinges: force second order (dual numbers), plasticity, its first-order reverse.
-    // The hinge's own part runs here; the reverse through its edges' frames runs per edge below
-    // on the sum of the seeds of both hinges of the edge (the reverse is linear in them).
-    for (int k = g.tid; k < nh; k += TPR) {
-        const int i = closed ? k : k + 1;
-        const int ea = (i == 0) ? ne - 1 : i - 1, eb = i;
-        const float4 ETa = s.ET[ea], ETb = s.ET[eb], hg = s.HG[i];
-        if (strands && !(ETa.w > 0.f && ETb.w > 0.f)) continue;   // inactive: at an end of a break edge
-        const float lbar = 0.5f * (ETa.w + ETb.w), il = 1.f / lbar;
-        // second order of the elastic force: tangents = cotangents of the gradient
-        HingeF<dualf> Hd;
-        ES.load_frame(ea, Hd.a);
-        ES.load_frame(eb, Hd.b);
-        hinge_core_forward(Hd, mkd(s.ED[ea].w, a.LG[ea].w), mkd(s.ED[eb].w, a.LG[eb].w), mkd(hg.w));
-        const float hk0 = Hd.k0.v, hk1 = Hd.k1.v;   // the hinge's material curvature (for plasticity)
-        float kb0 = hg.x, kb1 = hg.y;
-        const bool plastic = R.flags & ROD_PLASTIC;
-        const bool yielded = plastic && plastic_update(hk0, hk1, kb0, kb1, R.sy * lbar, R.rc);
-        dualf e0d = Hd.k0 - kb0, e1d = Hd.k1 - kb1, emd = Hd.m - hg.z;
-        dualf gk0 = (R.Bm * il) * e0d, gk1 = (R.Bm * il) * e1d, gmt = (R.beta * il) * emd;
-        // each term in float, added to the FP64 sums (the cancellation is across terms)
-        gl[1] += (double)(il * (e0d.v * e0d.d + e1d.v * e1d.d));
-        gl[2] += (double)(il * emd.v * emd.d);
-        // rest curvature: cotangent of the one used (-d gk / d .) plus the carried one
-        float lk0 = a.LK[i].x - gk0.d, lk1 = a.LK[i].y - gk1.d;
-        if (yielded) {
-            const float el0 = hk0 - hg.x, el1 = hk1 - hg.y;
-            const float n = sqrtf(el0 * el0 + el1 * el1), thr = R.sy * lbar;
-            const float g = R.rc * (n - thr) / n;
-            const float kk = R.rc * thr / (n * n * n) * (el0 * lk0 + el1 * lk1);
-            const float le0 = g * lk0 + kk * el0, le1 = g * lk1 + kk * el1;     // cotangent of kappa_el
-            gl[3] += (double)(-R.rc * lbar * (el0 * lk0 + el1 * lk1) / n);
-            // The first-order reverse of kappa from seeds (le0, le1) is needed too.  The hinge
-            // reverse is linear in its seeds, so adding them to the derivative part of the
-            // dual seeds makes the reverse below return J^T le on top of the Hessian term.
-            gk0.d += le0;
-            gk1.d += le1;
-            lk0 -= le0;
-            lk1 -= le1;
+    // ---- the own hinge: force second order, plasticity and its first-order reverse.  Seeds for
+    // the own edge are kept, those for the previous edge replace its frame (read here alone).
+    V3<dualf> gt = zero3<dualf>(), gr = zero3<dualf>();
+    float gth = 0.f, m_E = 0.f, m_G = 0.f, m_sy = 0.f;
+    if (has_em) {
+        V3<dualf> gta = zero3<dualf>(), gra = zero3<dualf>();
+        float gtha = 0.f;
+        if (has_e && !(strands && !(eba > 0.f && eb > 0.f))) {
+            const float lbar = 0.5f * (eba + eb), il = 1.f / lbar;
+            HingeF<dualf> H;
+            {
+                const float4 a = s.F0[im], d = s.F1[im], e = s.F2[im], f = s.F3[im];
+                H.a.t = mk3(mkd(a.x, d.x), mkd(a.y, d.y), mkd(a.z, d.z));
+                H.a.d1r = mk3(mkd(e.x, f.x), mkd(e.y, f.y), mkd(e.z, f.z));
+                H.a.c = mkd(a.w, d.w);
+                H.a.s = mkd(e.w, f.w);
+            }
+            H.b = E;
+            material_frame(H.a);
+            material_frame(H.b);
+            hinge_core_forward(H, mkd(tha, lga_w), mkd(ed.w, lg.w), mkd(hg.w));
+            const float hk0 = H.k0.v, hk1 = H.k1.v;   // the hinge's material curvature (for plasticity)
+            float kb0 = hg.x, kb1 = hg.y;
+            const bool yielded = (R.flags & ROD_PLASTIC) && plastic_update(hk0, hk1, kb0, kb1, R.sy * lbar, R.rc);
+            const dualf e0d = H.k0 - kb0, e1d = H.k1 - kb1, emd = H.m - hg.z;
+            dualf gk0 = (R.Bm * il) * e0d, gk1 = (R.Bm * il) * e1d;
+            const dualf gmt = (R.beta * il) * emd;
+            m_E = il * (e0d.v * e0d.d + e1d.v * e1d.d);
+            m_G = il * emd.v * emd.d;
+            // rest curvature: cotangent of the one used (-d gk / d .) plus the carried one
+            float lk0 = c.k0 - gk0.d, lk1 = c.k1 - gk1.d;
+            if (yielded) {
+                const float el0 = hk0 - hg.x, el1 = hk1 - hg.y;
+                const float n = sqrtf(el0 * el0 + el1 * el1), thr = R.sy * lbar;
+                const float gg = R.rc * (n - thr) / n;
+                const float kk = R.rc * thr / (n * n * n) * (el0 * lk0 + el1 * lk1);
+                const float le0 = gg * lk0 + kk * el0, le1 = gg * lk1 + kk * el1;     // cotangent of kappa_el
+                m_sy = -R.rc * lbar * (el0 * lk0 + el1 * lk1) / n;
+                // The first-order reverse of kappa from seeds (le0, le1) is needed too.  The hinge
+                // reverse is linear in its seeds, so adding them to the derivative part of the
+                // dual seeds makes the reverse below return J^T le on top of the Hessian term.
+                gk0.d += le0;
+                gk1.d += le1;
+                lk0 -= le0;
+                lk1 -= le1;
+            }
+            dualf ga_, gb_;
+            hinge_core_reverse(H, gk0, gk1, gmt, mkd(0.f), gta, gra, gt, gr, ga_, gb_);
+            gtha = ga_.d;
+            gth = gb_.d;
+            c.k0 = lk0;
+            c.k1 = lk1;
         }
-        V3<dualf> gta, gd1ra, gtb, gd1rb;
-        dualf ghta, ghtb;
-        hinge_core_reverse(Hd, gk0, gk1, gmt, mkd(0.f), gta, gd1ra, gtb, gd1rb, ghta, ghtb);
-        ES.add_seeds(ea, gta, gd1ra);
-        ES.add_seeds(eb, gtb, gd1rb);
-        atomicAdd(&ES.cs[ea].z, ghta.d);   // two terms per edge, added to zero: order-free
-        atomicAdd(&ES.cs[eb].z, ghtb.d);
-        a.LK[i] = make_float4(lk0, lk1, 0.f, 0.f);
+        s.F0[im] = make_float4(gta.x.v, gta.y.v, gta.z.v, gra.x.v);
+        s.F1[im] = make_float4(gta.x.d, gta.y.d, gta.z.d, gra.x.d);
+        s.F2[im] = make_float4(gra.y.v, gra.z.v, gra.y.d, gra.z.d);
+        s.F3[im].x = gtha;
     }
     g.sync();
-    // ---- B7, per edge: the reverse through the edge's frame (vertices and base frame); the
-    // edge's total position cotangent goes to s0 (its own slot, after its seeds are read)
-#pragma unroll
-    for (int m = 0; m < EPT; ++m) {
-        const int j = g.tid + m * TPR;
-        if (j >= ne) continue;
-        const float4 et = s.ET[j];
-        V3<float> tot = le_keep[m];
-        if (!(strands && !(et.w > 0.f))) {
-            V3<dualf> gt, gd1r;
-            ES.load_seeds(j, gt, gd1r);
-            EdgeF<dualf> Ed;
-            ES.load_rev(j, Ed);
-            V3<dualf> gtbd, gd1bd;
-            tot += ders(edge_reverse<dualf, true>(Ed, lift(f3(et)), lift(f3(s.ED[j])), gt, gd1r, mkd(0.f), &gtbd,
-                                                  &gd1bd));
-            const float4 lt = a.LT[j], le = a.LE[j];
-            a.LT[j] = f4(f3(lt) + ders(gtbd), 0.f);
-            a.LE[j] = f4(f3(le) + ders(gd1bd), le.w + ES.cs[j].z);
+    // ---- the reverse through the own edge's frame on the sum of its hinges' seeds; the
+    // cotangents of the frame it hands on (new base tangent and director) join the derivative
+    // parts (the reverse is linear in its seeds, as above)
+    if (has_e) {
+        if (real) {
+            const float4 a = s.F0[i], d = s.F1[i], e = s.F2[i];
+            gt += mk3(mkd(a.x, d.x + c.t.x), mkd(a.y, d.y + c.t.y), mkd(a.z, d.z + c.t.z));
+            gr += mk3(mkd(a.w, d.w + c.d1.x), mkd(e.x, e.z + c.d1.y), mkd(e.y, e.w + c.d1.z));
+            c.th += gth + s.F3[i].x;
+            V3<dualf> gtb, gdb;
+            tot += ders(edge_reverse<dualf, true>(E, lift(f3(et)), lift(f3(ed)), gt, gr, mkd(0.f), &gtb, &gdb));
+            c.t = ders(gtb);
+            c.d1 = ders(gdb);
         }
-        ES.s0[j] = f4(tot, 0.f);
+        s.LD[i] = f4(tot, 0.f);
+    }
+    if (P.gmat && vtx) {
+        add_comp(s.GM + i, m_K);
+        add_comp(s.GM + NV + i, m_E);
+        add_comp(s.GM + 2 * NV + i, m_G);
+        add_comp(s.GM + 3 * NV + i, m_sy);
+        add_comp(s.GM + 4 * NV + i, m_cd);
     }
     g.sync();
-    for (int i = g.tid; i < nv; i += TPR) {
-        V3<float> l = f3(a.LX[i]);
-        if (closed || i < nv - 1) l -= f3(ES.s0[i]);                   // edge i starts here
-        if (closed || i > 0) l += f3(ES.s0[i == 0 ? ne - 1 : i - 1]);  // edge i-1 ends here
-        a.LX[i] = f4(l, 0.f);
+    if (vtx) {
+        if (has_e) c.x -= tot;                  // edge i starts here
+        if (has_em) c.x += f3(s.LD[im]);        // edge i-1 ends here
     }
-#pragma unroll
-    for (int c = 0; c < 5; ++c) gm[c] += gl[c];
-    g.sync();
 }
 
 // ------------------------------------------------------------------ record layout
@@ -727,6 +723,12 @@ __host__ __device__ constexpr size_t seg_state(int NV) { return (size_t)5 * NV +
 // cotangent state carried from one chunk's reverse to the next: LX, LV, LE, LT, LK, then the
 // material sums (5 doubles) and the frame-start pose cotangents (12 floats)
 __host__ __device__ constexpr size_t cot_state(int NV) { return (size_t)5 * NV + 6; }
+
+// CTAs per SM the reverse kernel is compiled for.  Up to 128 vertices 384 threads per SM (168
+// registers): with 512 (128 registers) 120 registers spill and 4096 ropes x 128 take 12.1 instead
+// of 11.6 ms.  Above, two CTAs: with one (255 registers, no spills) 1024 bands x 200 in contact
+// take 5.8 instead of 4.8 ms.
+__host__ __device__ constexpr int rev_min_ctas(int NV) { return NV <= 128 ? 384 / NV : 2; }
 
 // ------------------------------------------------------------------ the recompute kernel
 // Persistent, forward-like (a group of threads per rod, state in shared memory, several rods
@@ -830,25 +832,23 @@ __global__ void __launch_bounds__(kFwdMaxThreads) rec_kernel(BwdParams P) {
 }
 
 // ------------------------------------------------------------------ the reverse kernel
-// Persistent, one group of threads per rod: for frames fb-1 .. fa, last first, and each
-// frame's substeps, last first, load the substep's records and apply the reverse of every
-// phase (reverse_substep).  The cotangents of the rod's state at frame fb come from dL/d(final
-// state) on the first chunk (fb = F), else from the previous chunk's launch (CS); those at fa
-// go to CS, or to the outputs on the last chunk (fa = 0).
+// Persistent, one CTA of one thread per vertex for each rod: for frames fb-1 .. fa, last first,
+// and each frame's substeps, last first, applies the reverse of every phase (reverse_substep)
+// from the substep's records.  The cotangents of the rod's state at frame fb come from
+// dL/d(final state) on the first chunk (fb = F), else from the previous chunk's launch (CS);
+// those at fa go to CS, or to the outputs on the last chunk (fa = 0).
 template <int NV, bool CONTACT>
-__global__ void __launch_bounds__(rev_max_threads(NV)) rev_kernel(BwdParams P) {
-    constexpr int TPR = rev_threads(NV);
+__global__ void __launch_bounds__(NV, rev_min_ctas(NV)) rev_kernel(BwdParams P) {
+    constexpr int TPR = NV;
     extern __shared__ float4 dyn_smem[];
-    const int rs = threadIdx.x / TPR;
-    float4* base = dyn_smem + rs * (bwd_smem_bytes(NV, CONTACT) / 16);
-    Smem<NV, CONTACT> s(base);
-    AdjArrays<NV, CONTACT> a(base + rod_smem_bytes(NV, CONTACT) / 16);
-    const Grp<TPR> g{(int)(threadIdx.x % TPR), 1 + rs, s.red};
+    RevSmem<NV, CONTACT> s(dyn_smem);
+    const Grp<TPR> g{(int)threadIdx.x, 1, s.red};
+    const int i = g.tid;
     const SceneDev& sc = P.scene;
     const int n_iter = sc.n_iter;
     const size_t SR = sub_rec(NV, n_iter), FR = frame_rec(NV, n_iter, P.nsub_max);
     for (;;) {
-        const int k = grp_bcast0<TPR>(g.tid == 0 ? atomicAdd(P.counter, 1) : 0, g);
+        const int k = grp_bcast0<TPR>(i == 0 ? atomicAdd(P.counter, 1) : 0, g);
         if (k >= P.n_items) break;
         const int rod = P.order[P.item0 + k];
         bounds_begin<TPR>(g);
@@ -857,128 +857,149 @@ __global__ void __launch_bounds__(rev_max_threads(NV)) rev_kernel(BwdParams P) {
             bounds_end<TPR>(g, P.status, (rod >= 0 && rod < P.B) ? rod : 0);
             continue;
         }
-        const RodInfo R = P.rods[rod];
+        const RodInfo* Rp = P.rods + rod;
+        const RodInfo R = *Rp;
         const int nsub = P.force_nsub > 0 ? P.force_nsub : R.nsub;
         const float h = sc.dt / (float)nsub;
+        const bool vtx = i < R.nv, has_e = i < R.ne, closed = R.flags & ROD_CLOSED;
+        const Own own = own_of(P.KIN, P.ES, R, i);
+        const float4 kin = own.kind >= 2 ? P.KIN[R.v0 + i] : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float eb = has_e ? P.ES[R.e0 + i].x : 0.f;   // rest lengths of the own and the previous edge
+        const float eba = vtx && (closed || i > 0) ? P.ES[R.e0 + (i == 0 ? R.ne - 1 : i - 1)].x : 0.f;
         float4* CS = P.CS + (size_t)k * P.cs_rod;
-        double gm[5] = {0.0, 0.0, 0.0, 0.0, 0.0};   // FP64: these sums cancel strongly
-        float lpf[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, lphif[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        Cot c{zf3(), zf3(), zf3(), zf3(), 0.f, 0.f, 0.f, 0.f};
         if (P.first_chunk) {
-            for (int i = g.tid; i < R.nv; i += TPR) {
-                float4 dx = P.dLdx ? P.dLdx[R.v0 + i] : make_float4(0.f, 0.f, 0.f, 0.f);
-                float4 dv = P.dLdv ? P.dLdv[R.v0 + i] : make_float4(0.f, 0.f, 0.f, 0.f);
-                if (!(R.flags & ROD_CLOSED) && i == R.nv - 1) dv.w = 0.f;
-                a.LX[i] = make_float4(dx.x, dx.y, dx.z, 0.f);
-                a.LV[i] = dv;
-                a.LK[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (vtx) {
+                const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+                const float4 dx = P.dLdx ? P.dLdx[R.v0 + i] : z, dv = P.dLdv ? P.dLdv[R.v0 + i] : z;
+                c.x = f3(dx);
+                c.v = f3(dv);
+                c.om = !closed && i == R.nv - 1 ? 0.f : dv.w;
             }
-            for (int j = g.tid; j < R.ne; j += TPR) {
-                a.LE[j] = make_float4(0.f, 0.f, 0.f, P.dLdth ? P.dLdth[R.e0 + j] : 0.f);
-                a.LT[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (has_e && P.dLdth) c.th = P.dLdth[R.e0 + i];
+        } else {
+            if (vtx) {
+                const float4 lv = CS[NV + i], lk = CS[4 * NV + i];
+                c.x = f3(CS[i]);
+                c.v = f3(lv);
+                c.om = lv.w;
+                c.k0 = lk.x;
+                c.k1 = lk.y;
             }
-        } else {   // the sums are carried by thread 0 of the group
-            for (int i = g.tid; i < R.nv; i += TPR) {
-                a.LX[i] = CS[i];
-                a.LV[i] = CS[NV + i];
-                a.LK[i] = CS[4 * NV + i];
-            }
-            for (int j = g.tid; j < R.ne; j += TPR) {
-                a.LE[j] = CS[2 * NV + j];
-                a.LT[j] = CS[3 * NV + j];
-            }
-            if (g.tid == 0) {
-                const double* d = reinterpret_cast<const double*>(CS + 5 * NV);
-                const float* q = reinterpret_cast<const float*>(CS + 5 * NV + 3);
-#pragma unroll
-                for (int c = 0; c < 5; ++c) gm[c] = d[c];
-#pragma unroll
-                for (int c = 0; c < 6; ++c) {
-                    lpf[c] = q[c];
-                    lphif[c] = q[6 + c];
-                }
+            if (has_e) {
+                const float4 le = CS[2 * NV + i];
+                c.d1 = f3(le);
+                c.th = le.w;
+                c.t = f3(CS[3 * NV + i]);
             }
         }
-        float ga[12];
+        // carried sums: the pose cotangents of frame fb's start, positions (2 x 3) then rotations
+        if (i < 12) s.PC[i] = P.first_chunk ? 0.0 : (double)reinterpret_cast<const float*>(CS + 5 * NV + 3)[i];
+        for (int m = 0; m < 5; ++m) s.GM[m * NV + i] = make_float2(0.f, 0.f);
+        float acc[24];   // the frame's pose terms of this thread (see fold_pose)
+        bool touched = true;
         for (int f = P.fb - 1; f >= P.fa; --f) {
             const float4* fb = P.R3 + (size_t)k * P.r3_rod + (size_t)(f - P.fa) * FR;
-            g.sync();   // the previous frame's reverse has finished reading s.act, s.f0 and the pairs
-            if (g.tid < 12) s.act[g.tid] = P.actions[((size_t)f * P.B + rod) * 12 + g.tid];
-            if (g.tid < 24) s.f0[g.tid] = reinterpret_cast<const float*>(fb)[g.tid];
+            g.sync();   // the previous frame's reverse has finished reading the frame's shared data
+            if (i < 12) s.act[i] = P.actions[((size_t)f * P.B + rod) * 12 + i];
+            if (i < 24) s.f0[i] = reinterpret_cast<const float*>(fb)[i];
             int np = 0;
             if (CONTACT) {
                 np = reinterpret_cast<const int*>(fb)[24];
                 if (!in_bounds(np >= 0 && np <= R.pair_cap, s.red)) np = 0;
                 const uint32_t* pl = reinterpret_cast<const uint32_t*>(fb + kFrameHead);
-                for (int p = g.tid; p < np; p += TPR) s.pairs[p] = pl[p];
+                for (int p = i; p < np; p += TPR) s.pairs[p] = pl[p];
+            }
+            if (touched) {
+#pragma unroll 1
+                for (int m = 0; m < 24; ++m) acc[m] = 0.f;
+                touched = false;
             }
             g.sync();
-            // carry the pose cotangent of frame f+1's start into this frame's actions
+            // the pose cotangent of frame f+1's start through the frame's motion: into its actions
+            // and its own start pose
+            if (i < R.ngrip) {
+                const V3<float> dphi = f3(s.act[6 * i + 3], s.act[6 * i + 4], s.act[6 * i + 5]);
+                double* lr = s.PC + 6 + 3 * i;
+                const V3<float> l = f3((float)lr[0], (float)lr[1], (float)lr[2]);
+                const V3<float> jr = jl_t(dphi, l), nr = mulT(expmap(dphi), l);
 #pragma unroll
-            for (int c = 0; c < 12; ++c) ga[c] = 0.f;
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                if (q >= R.ngrip) break;
-                const V3<float> dphi = f3(s.act[6 * q + 3], s.act[6 * q + 4], s.act[6 * q + 5]);
-                const V3<float> lp = get3(lpf, q), lr = get3(lphif, q);
-                ga[6 * q] = lp.x;
-                ga[6 * q + 1] = lp.y;
-                ga[6 * q + 2] = lp.z;
-                const V3<float> jr = jl_t(dphi, lr);
-                ga[6 * q + 3] = jr.x;
-                ga[6 * q + 4] = jr.y;
-                ga[6 * q + 5] = jr.z;
-                const V3<float> nr = mulT(expmap(dphi), lr);
-                lphif[3 * q] = nr.x;
-                lphif[3 * q + 1] = nr.y;
-                lphif[3 * q + 2] = nr.z;
+                for (int m = 0; m < 3; ++m) s.GA[6 * i + m] = (float)s.PC[3 * i + m];
+                s.GA[6 * i + 3] = jr.x;
+                s.GA[6 * i + 4] = jr.y;
+                s.GA[6 * i + 5] = jr.z;
+                lr[0] = nr.x;
+                lr[1] = nr.y;
+                lr[2] = nr.z;
             }
+#pragma unroll 1
             for (int sb = nsub - 1; sb >= 0; --sb) {
-                const float c0 = (float)sb / (float)nsub, c1 = (float)(sb + 1) / (float)nsub;
-                // the substep's gripper block (read after the barrier below)
-                if (g.tid < R.ngrip) substep_pose(s.f0, s.act, g.tid, c0, c1, sb == 0, 1.f / sc.dt, s.sp);
-                // the reverse's pose maps, on other threads (another warp where there is one)
-                constexpr int PT = TPR > 32 ? 32 : 2;
-                if (g.tid >= PT && g.tid < PT + 4 * R.ngrip) pose_rev_mat(s.act, g.tid - PT, c0, c1, a.PM);
-                // the substep's start state and recorded intermediates
-                const float4* e3 = fb + kFrameHead + NV + (size_t)sb * SR;
-                load_state<NV, CONTACT, TPR>(e3, R, g, s);
-                for (int i = g.tid; i < R.nv; i += TPR) {
-                    a.V1[i] = e3[5 * NV + i];
-                    a.DF[i] = e3[6 * NV + i];
-                }
-                if (CONTACT)
-                    for (int p = g.tid; p < np; p += TPR) {
-                        s.fr0[p] = e3[(7 + 2 * n_iter) * NV + p];
-                        s.fr1[p] = e3[(7 + 2 * n_iter + kPairsPerVertex) * NV + p];
+                const int slot = sb % kPoseBatch;
+                if (slot == kPoseBatch - 1 || sb == nsub - 1) {
+                    // gripper blocks and pose maps of this and the earlier substeps of the batch,
+                    // one per thread, side by side (read after the substep's first barrier)
+                    if (sb != nsub - 1) g.sync();
+                    for (int m = i; m < 10 * (slot + 1); m += TPR) {
+                        const int u = m / 10, w = m % 10, sk = sb - slot + u;
+                        const float k0 = (float)sk / (float)nsub, k1 = (float)(sk + 1) / (float)nsub;
+                        if (w < 2) {
+                            if (w < R.ngrip)
+                                substep_pose(s.f0, s.act, w, k0, k1, sk == 0, 1.f / sc.dt, s.sp + 64 * u);
+                        } else if (w - 2 < 4 * R.ngrip) {
+                            pose_rev_mat(s.act, w - 2, k0, k1, s.PM + 72 * u);
+                        }
                     }
-                g.sync();
-                reverse_substep<NV, CONTACT, TPR>(P, R, s, a, e3 + 7 * NV, e3 + (size_t)(7 + n_iter) * NV, g, h, c0,
-                                                  c1, np, gm, lpf, lphif, ga);
-            }
-            if (P.gact) {
-#pragma unroll
-                for (int c = 0; c < 12; ++c) {
-                    if (c >= 6 * R.ngrip) break;
-                    const float v = (float)grp_sum<TPR>((double)ga[c], g);
-                    if (g.tid == 0) P.gact[((size_t)f * P.B + rod) * 12 + c] = v;
                 }
-                if (g.tid == 0)
-                    for (int c = 6 * R.ngrip; c < 12; ++c) P.gact[((size_t)f * P.B + rod) * 12 + c] = 0.f;
+                const Rec<NV, true> rec{const_cast<float4*>(fb) + kFrameHead + NV + (size_t)sb * SR, n_iter};
+                reverse_substep<NV, CONTACT>(P, R, Rp, own, kin, eb, eba, s, g, rec, h, (float)sb / (float)nsub,
+                                             (float)(sb + 1) / (float)nsub, np, s.sp + 64 * slot, s.PM + 72 * slot, c,
+                                             acc, touched);
+            }
+            // the threads' pose terms: each warp's sums (zero where no thread has any), then over warps
+            {
+                const int lane = i & 31, w = i >> 5;
+                const bool any = __any_sync(0xffffffffu, touched);
+#pragma unroll 1
+                for (int m = 0; m < 24; ++m) {
+                    double v = 0.0;
+                    if (any) v = warp_sum(touched ? (double)acc[m] : 0.0);
+                    if (lane == 0) s.PR[24 * w + m] = v;
+                }
+                g.sync();
+                if (i < 24) {
+                    double v = 0.0;
+#pragma unroll
+                    for (int q = 0; q < TPR / 32; ++q) v += s.PR[24 * q + i];
+                    if (i < 12) {
+                        if (i % 6 < 3 * R.ngrip) s.PC[i] += v;
+                    } else if (P.gact) {
+                        const int m = i - 12;
+                        P.gact[((size_t)f * P.B + rod) * 12 + m] = m < 6 * R.ngrip ? (float)((double)s.GA[m] + v) : 0.f;
+                    }
+                }
             }
         }
-#pragma unroll
-        for (int c = 0; c < 5; ++c) gm[c] = grp_sum<TPR>(gm[c], g);
+        double gm[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+        if (P.gmat)
+#pragma unroll 1
+            for (int m = 0; m < 5; ++m) {
+                const float2 a = s.GM[m * NV + i];
+                gm[m] = grp_sum<TPR>((double)a.x + (double)a.y, g);
+                if (!P.first_chunk) gm[m] += reinterpret_cast<const double*>(CS + 5 * NV)[m];
+            }
+        g.sync();
+        const float4 lx = f4(c.x, 0.f), lv = f4(c.v, c.om);
         if (P.last_chunk) {   // outputs: the cotangents of the initial state and the material
-            for (int i = g.tid; i < R.nv; i += TPR) {
-                if (P.gx0) P.gx0[R.v0 + i] = a.LX[i];
-                if (P.gv0) P.gv0[R.v0 + i] = a.LV[i];
+            if (vtx) {
+                if (P.gx0) P.gx0[R.v0 + i] = lx;
+                if (P.gv0) P.gv0[R.v0 + i] = lv;
             }
-            for (int j = g.tid; j < R.ne; j += TPR) {
-                if (P.gth0) P.gth0[R.e0 + j] = a.LE[j].w;
-                P.gtb0[R.e0 + j] = a.LT[j];
-                P.gd1b0[R.e0 + j] = make_float4(a.LE[j].x, a.LE[j].y, a.LE[j].z, 0.f);
+            if (has_e) {
+                if (P.gth0) P.gth0[R.e0 + i] = c.th;
+                P.gtb0[R.e0 + i] = f4(c.t, 0.f);
+                P.gd1b0[R.e0 + i] = f4(c.d1, 0.f);
             }
-            if (g.tid == 0 && P.gmat) {
+            if (i == 0 && P.gmat) {
                 const double r = R.radius, A = 3.14159265358979323846 * r * r, r2 = r * r;
                 P.gmat[5 * rod + 0] = R.kA > 0.f ? (float)(gm[0] * A) : 0.f;   // K_stretch
                 P.gmat[5 * rod + 1] = (float)(gm[1] * A * r2 / 4.0);            // E_bend
@@ -986,30 +1007,22 @@ __global__ void __launch_bounds__(rev_max_threads(NV)) rev_kernel(BwdParams P) {
                 P.gmat[5 * rod + 3] = (float)gm[3];                             // yield curvature
                 P.gmat[5 * rod + 4] = (float)gm[4];                             // damping
             }
-        } else {   // carry to the next chunk: arrays, and the group sums of gm, lpf, lphif
-            for (int i = g.tid; i < R.nv; i += TPR) {
-                CS[i] = a.LX[i];
-                CS[NV + i] = a.LV[i];
-                CS[4 * NV + i] = a.LK[i];
+        } else {   // carry to the next chunk: cotangents, material and pose sums
+            if (vtx) {
+                CS[i] = lx;
+                CS[NV + i] = lv;
+                CS[4 * NV + i] = make_float4(c.k0, c.k1, 0.f, 0.f);
             }
-            for (int j = g.tid; j < R.ne; j += TPR) {
-                CS[2 * NV + j] = a.LE[j];
-                CS[3 * NV + j] = a.LT[j];
+            if (has_e) {
+                CS[2 * NV + i] = f4(c.d1, c.th);
+                CS[3 * NV + i] = f4(c.t, 0.f);
             }
-            float q[12];
-#pragma unroll
-            for (int c = 0; c < 6; ++c) {
-                q[c] = (float)grp_sum<TPR>((double)lpf[c], g);
-                q[6 + c] = (float)grp_sum<TPR>((double)lphif[c], g);
-            }
-            if (g.tid == 0) {
+            if (i == 0 && P.gmat) {
                 double* d = reinterpret_cast<double*>(CS + 5 * NV);
-                float* qq = reinterpret_cast<float*>(CS + 5 * NV + 3);
 #pragma unroll
-                for (int c = 0; c < 5; ++c) d[c] = gm[c];
-#pragma unroll
-                for (int c = 0; c < 12; ++c) qq[c] = q[c];
+                for (int m = 0; m < 5; ++m) d[m] = gm[m];
             }
+            if (i < 12) reinterpret_cast<float*>(CS + 5 * NV + 3)[i] = (float)s.PC[i];
         }
         g.sync();
         bounds_end<TPR>(g, P.status, rod);
@@ -1018,28 +1031,28 @@ __global__ void __launch_bounds__(rev_max_threads(NV)) rev_kernel(BwdParams P) {
 
 // ------------------------------------------------------------------ launch helpers
 template <int NV, bool C>
-static int rev_occ_t(int rpc) {
-    if (rpc < 1 || rpc * rev_threads(NV) > rev_max_threads(NV)) return 0;
-    size_t smem = bwd_smem_bytes(NV, C) * rpc;
+static int rev_occ_t(int rpc) {   // one rod per CTA
+    if (rpc != 1) return 0;
+    const size_t smem = RevSmem<NV, C>::kBytes;
     auto k = rev_kernel<NV, C>;
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, rev_threads(NV) * rpc, smem) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, NV, smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
     return nb;
 }
 template <int NV, bool C>
-static cudaError_t launch_rev_t(const BwdParams& P, int grid, int rpc, cudaStream_t st) {
-    size_t smem = bwd_smem_bytes(NV, C) * rpc;
+static cudaError_t launch_rev_t(const BwdParams& P, int grid, int, cudaStream_t st) {
+    const size_t smem = RevSmem<NV, C>::kBytes;
     auto k = rev_kernel<NV, C>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k<<<grid, rev_threads(NV) * rpc, smem, st>>>(P);
+    k<<<grid, NV, smem, st>>>(P);
     return cudaGetLastError();
 }
 template <int NV, bool C>

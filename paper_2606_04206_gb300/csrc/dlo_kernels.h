@@ -6,14 +6,14 @@
 
 namespace dlo {
 
-// Shared memory of one rod group (one rod of at most NV vertices) in the persistent kernels:
-// ten float4 arrays of NV (positions, start positions, velocities, base frames + twist,
-// base tangents + rest lengths, hinge state, three per-hinge gradient slots, new reference
-// frames) and, with self-contact, 4 NV pair slots (two float4 of projection data each,
-// one packed index pair) plus an int4 fixed-point accumulator per vertex.
+// Shared memory of one rod (of at most NV vertices) in the forward and recompute kernels: nine
+// float4 arrays of NV (displacements, positions, velocities, base frames + twist, base tangents +
+// rest lengths, hinge state, three exchanged between neighbours) and, with self-contact, 4 NV
+// pair slots (two float4 of projection data each, one packed index pair) plus an int4 fixed-point
+// accumulator per vertex.
 constexpr int kPairsPerVertex = 4;
 __host__ __device__ constexpr size_t warp_smem_bytes(int NV, bool contact) {
-    return (size_t)(10 * NV) * 16 +
+    return (size_t)(9 * NV) * 16 +
            (contact ? ((size_t)(2 * kPairsPerVertex * NV) * 16 + (size_t)NV * 16 + (size_t)(kPairsPerVertex * NV) * 4)
                     : 0);
 }

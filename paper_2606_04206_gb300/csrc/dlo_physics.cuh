@@ -117,11 +117,27 @@ struct HingeF {
     T cc, y, xq, mref, m, k0, k1;
 };
 
+// a x b with the roundings of its values fixed: each component one rounded product and one fused
+// multiply-add.  A hinge on its yield surface branches on the last bits of its curvature, and the
+// compiler may fuse either product, differently in the forward and in the backward's
+// recomputation, unless it is told which.
+DLO_HD float cross_comp(float p, float q, float r, float s) {   // p q - r s
+#ifdef __CUDA_ARCH__
+    return __fmaf_rn(p, q, -__fmul_rn(r, s));
+#else
+    return p * q - r * s;
+#endif
+}
+DLO_HD V3<float> cross_fixed(V3<float> a, V3<float> b) {
+    return {cross_comp(a.y, b.z, a.z, b.y), cross_comp(a.z, b.x, a.x, b.z), cross_comp(a.x, b.y, a.y, b.x)};
+}
+DLO_HD V3<dualf> cross_fixed(V3<dualf> a, V3<dualf> b) { return lift(cross_fixed(vals(a), vals(b)), ders(cross(a, b))); }
+
 // The hinge's own part, from its two edges' frames (H.a, H.b: t, d1r, d2r, d1, d2 set).
 template <class T>
 DLO_HD void hinge_core_forward(HingeF<T>& H, T tha, T thb, T mprev) {
     H.cc = 1.f + dot(H.a.t, H.b.t);
-    H.X = cross(H.a.t, H.b.t);
+    H.X = cross_fixed(H.a.t, H.b.t);
     H.kb = (2.f / H.cc) * H.X;
     H.k0 = 0.5f * dot(H.kb, H.a.d2 + H.b.d2);
     H.k1 = 0.5f * dot(H.kb, H.a.d1 + H.b.d1);
@@ -213,13 +229,25 @@ DLO_HD void hinge_reverse(const HingeF<T>& H, V3<T> tba, V3<T> d1ba, V3<T> tbb, 
 
 // ------------------------------------------------------------------ plasticity (App. A.1)
 // kappa_el = kappa - kbar; if |kappa_el| > sigma_y lbar: kbar += r_c (|k_el| - y)/|k_el| k_el.
+// The roundings are fixed (see cross_fixed): the rest curvature decides the next substep's yield.
+DLO_HD float sub_rounded(float a, float b) {   // never fused with the product b may be
+#ifdef __CUDA_ARCH__
+    return __fsub_rn(a, b);
+#else
+    return a - b;
+#endif
+}
 DLO_HD bool plastic_update(float k0, float k1, float& kb0, float& kb1, float thr, float rc) {
     float e0 = k0 - kb0, e1 = k1 - kb1;
+#ifdef __CUDA_ARCH__
+    float n2 = __fmaf_rn(e0, e0, __fmul_rn(e1, e1));
+#else
     float n2 = e0 * e0 + e1 * e1;
+#endif
     if (!(n2 > 0.f)) return false;
     float n = sqrtf(n2);
     if (!(n > thr)) return false;
-    float g = rc * (n - thr) / n;
+    float g = rc * sub_rounded(n, thr) / n;
     kb0 = kb0 + g * e0;
     kb1 = kb1 + g * e1;
     return true;

@@ -66,7 +66,7 @@ static cudaError_t launch_bucket(dlo_ctx* c, size_t k, int warps, int grid, int 
 // (the rule callers know); a CTA of rods above 128 vertices, which take a thread per vertex, then
 // holds as many of them as it can.
 static int forced_rods_per_cta(int nv_max, bool contact, int want) {
-    if (want * std::min(nv_max, 128) > 512 || want * (warp_smem_bytes(nv_max, contact) + 768) > 227 * 1024) return 0;
+    if (want * std::min(nv_max, 128) > 512 || want * (warp_smem_bytes(nv_max, contact) + 16 * nv_max + 768) > 227 * 1024) return 0;
     while (want > 1 && forward_blocks_per_sm(nv_max, contact, want) < 1) --want;
     return want;
 }

@@ -265,7 +265,7 @@ __device__ __forceinline__ V3<float> rigid_contact(const SceneDev& sc, const Rod
 
 template <int NV, bool CONTACT>
 struct Smem {
-    float4 *X, *X0, *V, *ED, *ET, *HG, *HB0, *HB1, *HB2, *ND;
+    float4 *X, *X0, *V, *ED, *ET, *HG, *HB0, *HB1, *HB2;
     float4 *fr0, *fr1;
     int4* acc;
     uint32_t* pairs;
@@ -291,8 +291,7 @@ struct Smem {
         HB0 = base + 6 * NV;
         HB1 = base + 7 * NV;
         HB2 = base + 8 * NV;
-        ND = base + 9 * NV;
-        fr0 = base + 10 * NV;
+        fr0 = base + 9 * NV;
         fr1 = fr0 + kPairsPerVertex * NV;
         acc = reinterpret_cast<int4*>(fr1 + kPairsPerVertex * NV);
         pairs = reinterpret_cast<uint32_t*>(acc + NV);
