@@ -233,13 +233,15 @@ size_t frame_rec_h(int NV, int n_iter, int nsub) {
     return (size_t)(8 + NV) + (size_t)nsub * (size_t)(7 + 2 * n_iter + 2 * kPairsPerVertex) * NV;
 }
 
-// rods per CTA and CTAs per SM that keep the most rods resident
+// Rods per CTA and CTAs per SM that keep the most rods resident, with the fewest rods per CTA
+// (a batch smaller than the device then spreads over all SMs: 304 rods of 128 vertices in CTAs of
+// four filled half of them).
 void best_shape(int nv, bool contact, bool rec, int& w, int& nb) {
     w = 0;
     nb = 0;
     for (int rpc = 1; rpc <= 16; ++rpc) {
         const int b = rec ? rec_blocks_per_sm(nv, contact, rpc) : rev_blocks_per_sm(nv, contact, rpc);
-        if (b >= 1 && rpc * b >= w * nb) {
+        if (b >= 1 && rpc * b > w * nb) {
             w = rpc;
             nb = b;
         }

@@ -114,13 +114,15 @@ struct RevSmem {
     float4 *LD;                 // displacement cotangents, then the force cotangents, then dL/d(edge vectors)
     float4 *F0, *F1, *F2, *F3;  // per edge: its dual frame, replaced by the seeds of the hinge at its end
     float2* GM;                 // [5][NV]: the threads' material sums, each an unevaluated sum of two floats
+    float* PA;                  // [24][NV]: the threads' pose terms of the frame: positions (2 x 3),
+                                // rotations (2 x 3), actions (2 x 6)
     uint32_t* pairs;
     float *red, *f0, *act;      // reduction scratch, the frame's start pose (24) and actions (12)
     float *sp, *PM;             // per substep of a batch: gripper blocks (64) and pose maps (72)
-    double *PR, *PC;            // per warp, its sums of the 24 pose terms; the carried pose cotangents (12)
+    double* PC;                 // the carried pose cotangents (12)
     float* GA;                  // the frame's action cotangents carried from the next frame's pose (12)
-    static constexpr size_t kHeader = 64 + 24 + 16 + 64 * kPoseBatch + 72 * kPoseBatch + 2 * (8 * 24 + 12) + 12 + 4;
-    static constexpr size_t kBytes = 16 * (size_t)(5 * NV) + 8 * (size_t)(5 * NV) +
+    static constexpr size_t kHeader = 64 + 24 + 16 + 64 * kPoseBatch + 72 * kPoseBatch + 2 * 12 + 16;
+    static constexpr size_t kBytes = 16 * (size_t)(5 * NV) + 8 * (size_t)(5 * NV) + 4 * (size_t)(24 * NV) +
                                      (CONTACT ? 4 * (size_t)(kPairsPerVertex * NV) : 0) + 4 * kHeader;
     __device__ explicit RevSmem(float4* b) {
         LD = b;
@@ -129,8 +131,8 @@ struct RevSmem {
         F2 = b + 3 * NV;
         F3 = b + 4 * NV;
         GM = reinterpret_cast<float2*>(b + 5 * NV);
-        PR = reinterpret_cast<double*>(GM + 5 * NV);
-        PC = PR + 8 * 24;
+        PA = reinterpret_cast<float*>(GM + 5 * NV);
+        PC = reinterpret_cast<double*>(PA + 24 * NV);
         red = reinterpret_cast<float*>(PC + 12);
         f0 = red + 64;
         act = f0 + 24;
@@ -166,20 +168,21 @@ __device__ __forceinline__ V3<float> mul_rm_t(const float* o, V3<float> v) {
 
 // Pose cotangents of one substep and gripper (positions and rotations at the substep's start
 // and end, rigid velocities) -> the frame-start pose and the frame's actions.  acc: the thread's
-// 24 pose terms (positions 2 x 3, rotations 2 x 3, actions 2 x 6).  Only the threads of held
-// vertices and of vertices touching a gripper come here, so acc lives in local memory.
-static __device__ __noinline__ void fold_pose(float* acc, int q, const float* pm, float c0, float c1, float idt, V3<float> ps0,
-                                       V3<float> ph0, V3<float> ps1, V3<float> ph1, V3<float> vp, V3<float> w) {
-    auto add = [](float* o, V3<float> v) {
-        o[0] += v.x;
-        o[1] += v.y;
-        o[2] += v.z;
-    };
+// pose terms (RevSmem::PA), stride apart.  Only the threads of held vertices and of vertices
+// touching a gripper have any.
+__device__ __forceinline__ void add_pose(float* acc, int stride, int m, V3<float> v) {
+    acc[m * stride] += v.x;
+    acc[(m + 1) * stride] += v.y;
+    acc[(m + 2) * stride] += v.z;
+}
+__device__ __forceinline__ void fold_pose(float* acc, int stride, int q, const float* pm, float c0, float c1, float idt,
+                                          V3<float> ps0, V3<float> ph0, V3<float> ps1, V3<float> ph1, V3<float> vp,
+                                          V3<float> w) {
     pm += 36 * q;
-    add(acc + 3 * q, ps0 + ps1);
-    add(acc + 6 + 3 * q, mul_rm_t(pm, ph0) + mul_rm_t(pm + 9, ph1));
-    add(acc + 12 + 6 * q, c0 * ps0 + c1 * ps1 + idt * vp);
-    add(acc + 15 + 6 * q, mul_rm(pm + 18, ph0) + mul_rm(pm + 27, ph1) + idt * w);
+    add_pose(acc, stride, 3 * q, ps0 + ps1);
+    add_pose(acc, stride, 6 + 3 * q, mul_rm_t(pm, ph0) + mul_rm_t(pm + 9, ph1));
+    add_pose(acc, stride, 12 + 6 * q, c0 * ps0 + c1 * ps1 + idt * vp);
+    add_pose(acc, stride, 15 + 6 * q, mul_rm(pm + 18, ph0) + mul_rm(pm + 27, ph1) + idt * w);
 }
 
 struct RevGrip {
@@ -207,8 +210,8 @@ __device__ __forceinline__ void material_frame(EdgeF<dualf>& E) {
 // Reverse of an active gripper contact: the cotangents of the vertex position (to add) and of
 // the velocity before the contact; the pose cotangents go to acc.  Out of line: few vertices
 // touch a gripper, and inlined its registers would be every vertex's.
-static __device__ __noinline__ RevGrip gripper_reverse(const BwdParams& P, const RodInfo* Rp, const float* sp, const float* pm,
-                                                float* acc, int q, float c0, float c1, V3<float> x, V3<float> v,
+static __device__ __noinline__ RevGrip gripper_reverse(const BwdParams& P, const RodInfo* Rp, const float* sp,
+                                                       const float* pm, float* acc, int stride, int q, float c0, float c1, V3<float> x, V3<float> v,
                                                 V3<float> lam) {
     const SceneDev& sc = P.scene;
     const RodInfo& R = *Rp;
@@ -241,7 +244,7 @@ static __device__ __noinline__ RevGrip gripper_reverse(const BwdParams& P, const
         lvp = f3(lin[12], lin[13], lin[14]);
         lw = f3(lin[15], lin[16], lin[17]);
     }
-    fold_pose(acc, q, pm, c0, c1, 1.f / sc.dt, lp, lphi, zf3(), zf3(), lvp, lw);
+    fold_pose(acc, stride, q, pm, c0, c1, 1.f / sc.dt, lp, lphi, zf3(), zf3(), lvp, lw);
     return r;
 }
 
@@ -253,6 +256,10 @@ __device__ __forceinline__ V3<float> respond_at(int k, const SceneDev& sc, const
     if (q >= 0) {
         const float* o = sp + 32 * q;
         gp = f3(o[0], o[1], o[2]);
+        if (grip_far(x, gp, o)) {
+            on = false;
+            return v;
+        }
         gax = f3(o[8], o[11], o[14]);
         vp = f3(o[24], o[25], o[26]);
         w = f3(o[27], o[28], o[29]);
@@ -263,8 +270,8 @@ __device__ __forceinline__ V3<float> respond_at(int k, const SceneDev& sc, const
 // Reverse of the rigid contact of one vertex: from the cotangent lam of the velocity after it,
 // that of the velocity v1 before it; adds the position's to lx.
 __device__ __forceinline__ V3<float> rigid_reverse(const BwdParams& P, const RodInfo& R, const RodInfo* Rp, const float* sp,
-                                                   const float* pm, float* acc, float c0, float c1, V3<float> x,
-                                                   V3<float> v1, V3<float> lam, V3<float>& lx, bool& touched) {
+                                                   const float* pm, float* acc, int stride, float c0, float c1,
+                                                   V3<float> x, V3<float> v1, V3<float> lam, V3<float>& lx, bool& touched) {
     const SceneDev& sc = P.scene;
     const int nprim = sc.n_planes + sc.n_boxes + R.ngrip;
     unsigned mask = 0;
@@ -283,7 +290,7 @@ __device__ __forceinline__ V3<float> rigid_reverse(const BwdParams& P, const Rod
         const int k = 31 - __clz(mask), q = k - sc.n_planes - sc.n_boxes;
         mask ^= 1u << k;
         if (q >= 0) {
-            const RevGrip r = gripper_reverse(P, Rp, sp, pm, acc, q, c0, c1, x, vb, lam);
+            const RevGrip r = gripper_reverse(P, Rp, sp, pm, acc, stride, q, c0, c1, x, vb, lam);
             lx += r.lx;
             lam = r.lam;
             touched = true;
@@ -361,15 +368,15 @@ __device__ __forceinline__ V3<float> project_rev(float4 q, float a, float b, V3<
 
 // ------------------------------------------------------------------ reverse of one substep
 // rec: the substep's records.  c holds the cotangents of S_{n+1} on entry and of S_n on exit.
-// sp, pm: the substep's gripper block and pose maps; acc: the thread's pose terms.
+// sp, pm: the substep's gripper block and pose maps.  touched: set when the thread adds to its
+// pose terms.
 // Bound by latency: dependent arithmetic of few warps (registers), barriers and record loads.
-// Each thread keeps its vertex's, edge's and hinge's data in registers from phase to phase; a
-// thread's local memory holds only the pose terms, which few threads touch.
+// Each thread keeps its vertex's, edge's and hinge's data in registers from phase to phase.
 template <int NV, bool CONTACT>
 __device__ __forceinline__ void reverse_substep(const BwdParams& P, const RodInfo& R, const RodInfo* Rp, const Own& own,
                                                 float4 kin, float eb, float eba, RevSmem<NV, CONTACT>& s,
                                                 const Grp<NV>& g, const Rec<NV, true> rec, float h, float c0, float c1,
-                                                int np, const float* sp, const float* pm, Cot& c, float* acc,
+                                                int np, const float* sp, const float* pm, Cot& c,
                                                 bool& touched) {
     const SceneDev& sc = P.scene;
     const int nv = R.nv, ne = R.ne, i = g.tid;
@@ -563,7 +570,7 @@ __device__ __forceinline__ void reverse_substep(const BwdParams& P, const RodInf
         V3<float> lx = held ? dx : c.x + dx, lv = zf3();
         if (own.kind == 0) {
             V3<float> lam = h * ld;
-            lam = rigid_reverse(P, R, Rp, sp, pm, acc, c0, c1, f3(x4), f3(v1), lam, lx, touched);
+            lam = rigid_reverse(P, R, Rp, sp, pm, s.PA + i, NV, c0, c1, f3(x4), f3(v1), lam, lx, touched);
             // v1 = v + h (-w g + gravity - c_d v)
             lv = (1.f - h * R.cd) * lam;
             const V3<float> l = (-h * x4.w) * lam;
@@ -573,7 +580,7 @@ __device__ __forceinline__ void reverse_substep(const BwdParams& P, const RodInf
             // x = target and d = target - x0, the target moving with the gripper's end pose
             const int q = own.kind - 2;
             const V3<float> y1 = mul_rm(sp + 32 * q + 15, f3(kin)), l = c.x + ld;
-            fold_pose(acc, q, pm, c0, c1, 1.f / sc.dt, zf3(), zf3(), l, cross(y1, l), zf3(), zf3());
+            fold_pose(s.PA + i, NV, q, pm, c0, c1, 1.f / sc.dt, zf3(), zf3(), l, cross(y1, l), zf3(), zf3());
             touched = true;
             lx -= ld;
         }
@@ -896,7 +903,6 @@ __global__ void __launch_bounds__(NV, rev_min_ctas(NV)) rev_kernel(BwdParams P) 
         // carried sums: the pose cotangents of frame fb's start, positions (2 x 3) then rotations
         if (i < 12) s.PC[i] = P.first_chunk ? 0.0 : (double)reinterpret_cast<const float*>(CS + 5 * NV + 3)[i];
         for (int m = 0; m < 5; ++m) s.GM[m * NV + i] = make_float2(0.f, 0.f);
-        float acc[24];   // the frame's pose terms of this thread (see fold_pose)
         bool touched = true;
         for (int f = P.fb - 1; f >= P.fa; --f) {
             const float4* fb = P.R3 + (size_t)k * P.r3_rod + (size_t)(f - P.fa) * FR;
@@ -912,7 +918,7 @@ __global__ void __launch_bounds__(NV, rev_min_ctas(NV)) rev_kernel(BwdParams P) 
             }
             if (touched) {
 #pragma unroll 1
-                for (int m = 0; m < 24; ++m) acc[m] = 0.f;
+                for (int m = 0; m < 24; ++m) s.PA[m * NV + i] = 0.f;
                 touched = false;
             }
             g.sync();
@@ -944,7 +950,7 @@ __global__ void __launch_bounds__(NV, rev_min_ctas(NV)) rev_kernel(BwdParams P) 
                         const float k0 = (float)sk / (float)nsub, k1 = (float)(sk + 1) / (float)nsub;
                         if (w < 2) {
                             if (w < R.ngrip)
-                                substep_pose(s.f0, s.act, w, k0, k1, sk == 0, 1.f / sc.dt, s.sp + 64 * u);
+                                substep_pose(sc, R, s.f0, s.act, w, k0, k1, sk == 0, 1.f / sc.dt, s.sp + 64 * u);
                         } else if (w - 2 < 4 * R.ngrip) {
                             pose_rev_mat(s.act, w - 2, k0, k1, s.PM + 72 * u);
                         }
@@ -953,32 +959,27 @@ __global__ void __launch_bounds__(NV, rev_min_ctas(NV)) rev_kernel(BwdParams P) 
                 const Rec<NV, true> rec{const_cast<float4*>(fb) + kFrameHead + NV + (size_t)sb * SR, n_iter};
                 reverse_substep<NV, CONTACT>(P, R, Rp, own, kin, eb, eba, s, g, rec, h, (float)sb / (float)nsub,
                                              (float)(sb + 1) / (float)nsub, np, s.sp + 64 * slot, s.PM + 72 * slot, c,
-                                             acc, touched);
+                                             touched);
             }
-            // the threads' pose terms: each warp's sums (zero where no thread has any), then over warps
-            {
-                const int lane = i & 31, w = i >> 5;
-                const bool any = __any_sync(0xffffffffu, touched);
-#pragma unroll 1
-                for (int m = 0; m < 24; ++m) {
-                    double v = 0.0;
-                    if (any) v = warp_sum(touched ? (double)acc[m] : 0.0);
-                    if (lane == 0) s.PR[24 * w + m] = v;
-                }
-                g.sync();
-                if (i < 24) {
-                    double v = 0.0;
-#pragma unroll
-                    for (int q = 0; q < TPR / 32; ++q) v += s.PR[24 * q + i];
-                    if (i < 12) {
-                        if (i % 6 < 3 * R.ngrip) s.PC[i] += v;
-                    } else if (P.gact) {
-                        const int m = i - 12;
-                        P.gact[((size_t)f * P.B + rod) * 12 + m] = m < 6 * R.ngrip ? (float)((double)s.GA[m] + v) : 0.f;
-                    }
+            // the frame's pose terms: one thread per term adds those of the threads that have any, in
+            // order (a tree of FP64 shuffles over every term took a third of the rollout's reverse)
+            unsigned* hit = reinterpret_cast<unsigned*>(s.red);
+            const unsigned warp_hit = __ballot_sync(0xffffffffu, touched);
+            if ((i & 31) == 0) hit[i >> 5] = warp_hit;
+            g.sync();
+            if (i < 24) {
+                double v = 0.0;
+                for (int w = 0; w < TPR / 32; ++w)
+                    for (unsigned m = hit[w]; m; m &= m - 1) v += (double)s.PA[i * NV + 32 * w + __ffs(m) - 1];
+                if (i < 12) {
+                    if (i % 6 < 3 * R.ngrip) s.PC[i] += v;
+                } else if (P.gact) {
+                    const int m = i - 12;
+                    P.gact[((size_t)f * P.B + rod) * 12 + m] = m < 6 * R.ngrip ? (float)((double)s.GA[m] + v) : 0.f;
                 }
             }
         }
+        g.sync();   // the last frame's pose terms have been added
         double gm[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
         if (P.gmat)
 #pragma unroll 1

@@ -51,7 +51,7 @@ __global__ void pl_pose(SceneDev sc, const RodInfo* rods, int B, const float* GP
     const int n = nsub_of(R, force);
     if (s >= n) return;
     for (int q = 0; q < R.ngrip; ++q)
-        substep_pose(GP + 24LL * b, act + 12LL * b, q, (float)s / (float)n, (float)(s + 1) / (float)n, s == 0,
+        substep_pose(sc, R, GP + 24LL * b, act + 12LL * b, q, (float)s / (float)n, (float)(s + 1) / (float)n, s == 0,
                      1.f / sc.dt, POSE + 64LL * b);
 }
 
@@ -654,7 +654,7 @@ __global__ void prb_sub_begin(SceneDev sc, const RodInfo* rods, int B, const flo
     if (s >= n) return;
     const float c0 = (float)s / (float)n, c1 = (float)(s + 1) / (float)n;
     for (int q = 0; q < R.ngrip; ++q) {
-        substep_pose(A.GPF + 24LL * b, act + 12LL * b, q, c0, c1, s == 0, 1.f / sc.dt, POSE + 64LL * b);
+        substep_pose(sc, R, A.GPF + 24LL * b, act + 12LL * b, q, c0, c1, s == 0, 1.f / sc.dt, POSE + 64LL * b);
         for (int m = 0; m < 4; ++m) pose_rev_mat(act + 12LL * b, 4 * q + m, c0, c1, A.PM + 72LL * b);
     }
 }

@@ -223,6 +223,19 @@ __device__ __forceinline__ void add_impulse(float4* slot, float m, V3<float> vb,
     *slot = make_float4(a.x + m * (va.x - vb.x), a.y + m * (va.y - vb.y), a.z + m * (va.z - vb.z), 0.f);
 }
 
+// Squared distance from a gripper's centre beyond which no vertex can touch it: the capsule's
+// half length plus the contact's reach, a little enlarged.  Nearly every vertex is rejected by
+// this one test (the capsule's own takes a projection on its axis and a quotient).
+__device__ __forceinline__ float grip_bound(const SceneDev& sc, const RodInfo& R, const float* o) {
+    const V3<float> ax = f3(o[8], o[11], o[14]);
+    const float b = sc.grip_hl * sqrtf(dot(ax, ax)) + 1.001f * (sc.grip_r + R.radius + kContactReach * R.eps);
+    return 1.0001f * b * b;
+}
+__device__ __forceinline__ bool grip_far(V3<float> x, V3<float> p, const float* o) {
+    const V3<float> d = x - p;
+    return dot(d, d) > o[30];
+}
+
 // Rigid contact of one vertex against the scene and the rod's grippers (Sec. 3.2).
 // sp: the substep's gripper block (Smem::sp).  imp (optional): the vertex's four impulse
 // slots (planes, boxes, gripper 0, gripper 1), to which each active response adds the
@@ -248,6 +261,7 @@ __device__ __forceinline__ V3<float> rigid_contact(const SceneDev& sc, const Rod
     for (int g = 0; g < R.ngrip; ++g) {
         const float* o = sp + 32 * g;
         V3<float> p = f3(o[0], o[1], o[2]);
+        if (grip_far(x, p, o)) continue;
         V3<float> ax = f3(o[8], o[11], o[14]);   // column 2 of R0: the capsule axis
         V3<float> a = p - sc.grip_hl * ax, b = p + sc.grip_hl * ax, n;
         if (capsule_far(x, a, b, sc.grip_r + R.radius + kContactReach * R.eps)) continue;
@@ -273,7 +287,8 @@ struct Smem {
     // gripper block (read by every thread of the rod with broadcasts):
     //   fp  [24] pose at the start of the frame being stepped, per gripper p (3), R (9) row major
     //   f0  [24] a second frame-start pose (the frame the backward reverses)
-    //   sp  [kPoseBatch][64] per substep and gripper (32): p0 (3), p1 (3), R0 (9), R1 (9), vp (3), w (3)
+    //   sp  [kPoseBatch][64] per substep and gripper (32): p0 (3), p1 (3), R0 (9), R1 (9), vp (3), w (3),
+    //       grip_bound (1)
     //   act [12] the frame's actions
     float *fp, *f0, *sp, *act;
     __device__ Smem(float4* base) {
@@ -908,8 +923,8 @@ __device__ __forceinline__ void substep_body(const SceneDev& sc, const float4* _
 // (per gripper p (3), R (9) row major) and the frame's actions: positions and rotations at
 // the substep's start (c0) and end (c1) of the frame, p + c dp and exp(c dphi) R (the start
 // rotation of the first substep is the frame's own), and the rigid velocities dp/dt, dphi/dt.
-__device__ __forceinline__ void substep_pose(const float* F, const float* act, int q, float c0, float c1, bool first,
-                                             float inv_dt, float* out) {
+__device__ __forceinline__ void substep_pose(const SceneDev& sc, const RodInfo& R, const float* F, const float* act,
+                                             int q, float c0, float c1, bool first, float inv_dt, float* out) {
     const float* f = F + 12 * q;
     const float* a = act + 6 * q;
     M3 RF;
@@ -930,6 +945,7 @@ __device__ __forceinline__ void substep_pose(const float* F, const float* act, i
         o[6 + k] = R0.m[k];
         o[15 + k] = R1.m[k];
     }
+    o[30] = grip_bound(sc, R, o);
 }
 
 // Frame end for gripper q: p += dp, R = exp(dphi) R.
@@ -969,8 +985,8 @@ __device__ __forceinline__ int run_frame(const SceneDev& sc, const float4* __res
         if (sb % kPoseBatch == 0) {
             const int k = sb + (g.tid >> 1), q = g.tid & 1;
             if (g.tid < 2 * kPoseBatch && k < nsub && q < R.ngrip)
-                substep_pose(s.fp, s.act, q, (float)k / (float)nsub, (float)(k + 1) / (float)nsub, k == 0, inv_dt,
-                             s.sp + 64 * (g.tid >> 1));
+                substep_pose(sc, R, s.fp, s.act, q, (float)k / (float)nsub, (float)(k + 1) / (float)nsub, k == 0,
+                             inv_dt, s.sp + 64 * (g.tid >> 1));
         }
         substep_body(sc, KIN, R, own, s, g, h, np, s.sp + 64 * (sb % kPoseBatch), pre(sb), imp, mv);
     }
