@@ -337,18 +337,6 @@ struct Cot {
     float om, th, k0, k1;      // twist rate, twist angle, rest curvature
 };
 
-// Threads that reverse a rod's length projections: thread t takes the edges 2t and 2t + 1.
-__host__ __device__ constexpr int pbd_threads(int NV) { return NV <= 64 ? 32 : (NV / 2 + 31) / 32 * 32; }
-constexpr int kPbdBar = 2;   // their named barrier (the rod's own is 1)
-
-template <int NV>
-__device__ __forceinline__ void pbd_sync() {
-    if (pbd_threads(NV) == 32)
-        __syncwarp();
-    else
-        asm volatile("bar.sync %0, %1;" ::"r"(kPbdBar), "r"(pbd_threads(NV)) : "memory");
-}
-
 // The two edges of a projecting thread and their running sums of cotangents.
 struct PbdRev {
     bool e0, e1, ring;         // edge 2t, edge 2t + 1 are projected; edge 2t is an odd loop's last (its own colour)
@@ -527,7 +515,7 @@ __device__ __forceinline__ void reverse_substep(const BwdParams& P, const RodInf
                         s.LD[0] = f4(lb + le, 0.f);
                         b.s0 += le;
                     }
-                    pbd_sync<NV>();
+                    pbd_sync<NV>(g.bar);
                 }
                 // vertex 2t + 1 belongs to this thread's two edges alone
                 V3<float> lm = b.e0 && !b.ring ? f3(s.LD[2 * i + 1]) : zf3();
@@ -538,7 +526,7 @@ __device__ __forceinline__ void reverse_substep(const BwdParams& P, const RodInf
                     s.LD[b.i2] = f4(lb + le, 0.f);
                     b.s1 += le;
                 }
-                pbd_sync<NV>();
+                pbd_sync<NV>(g.bar);
                 if (b.e0 && !b.ring) {
                     const V3<float> la = f3(s.LD[b.i0]);
                     const V3<float> le = project_rev(r0, b.a0, b.b0, la, lm);
@@ -546,7 +534,7 @@ __device__ __forceinline__ void reverse_substep(const BwdParams& P, const RodInf
                     s.LD[2 * i + 1] = f4(lm + le, 0.f);
                     b.s0 += le;
                 }
-                pbd_sync<NV>();
+                pbd_sync<NV>(g.bar);
             }
             if (CONTACT && np > 0) g.sync();
         }
@@ -738,12 +726,11 @@ __host__ __device__ constexpr size_t cot_state(int NV) { return (size_t)5 * NV +
 __host__ __device__ constexpr int rev_min_ctas(int NV) { return NV <= 128 ? 384 / NV : 2; }
 
 // ------------------------------------------------------------------ the recompute kernel
-// Persistent, forward-like (a group of threads per rod, state in shared memory, several rods
-// per CTA).  mode 0: from the checkpoint of the segment that holds frame fa, store the start
-// state of each of the segment's frames (L2).  mode 1: from the start state of frame fa (a
-// checkpoint, or the segment's stored state), run frames fa .. fb-1 storing every substep's
-// records (R3).
-template <int NV, bool CONTACT>
+// Persistent, forward-like (a group of threads per rod, state in shared memory).  RECORD false:
+// from the checkpoint of the segment that holds frame fa, store the start state of each of the
+// segment's frames (L2).  RECORD true: from the start state of frame fa (a checkpoint, or the
+// segment's stored state), run frames fa .. fb-1 storing every substep's records (R3).
+template <int NV, bool CONTACT, bool RECORD>
 __global__ void __launch_bounds__(kFwdMaxThreads) rec_kernel(BwdParams P) {
     constexpr int TPR = threads_per_rod(NV);
     extern __shared__ float4 dyn_smem[];
@@ -772,7 +759,7 @@ __global__ void __launch_bounds__(kFwdMaxThreads) rec_kernel(BwdParams P) {
         const float h = sc.dt / (float)nsub;
         const int seg = P.fa / P.ck_every, f0 = seg * P.ck_every;
         float4* L2 = P.L2 + (size_t)k * P.l2_rod;
-        if (P.mode == 0 || P.fa == f0) {   // the segment's checkpoint
+        if (!RECORD || P.fa == f0) {   // the segment's checkpoint
             const long long oV = seg * P.ck_strideV, oE = seg * P.ck_strideE;
             for (int i = g.tid; i < R.nv; i += TPR) {
                 const float4 x = P.ck.X[oV + R.v0 + i];
@@ -802,7 +789,7 @@ __global__ void __launch_bounds__(kFwdMaxThreads) rec_kernel(BwdParams P) {
         const Own own = own_of(P.KIN, P.ES, R, g.tid);
         g.sync();
         bool ovf = false;
-        if (P.mode == 0) {
+        if constexpr (!RECORD) {
             const int f1 = min(f0 + P.ck_every, P.frames);
             for (int f = f0; f < f1; ++f) {
                 float4* e = L2 + (size_t)(f - f0) * seg_state(NV);
@@ -1060,7 +1047,7 @@ template <int NV, bool C>
 static int rec_occ_t(int rpc) {
     if (rpc < 1 || rpc * threads_per_rod(NV) > kFwdMaxThreads) return 0;
     size_t smem = rod_smem_bytes(NV, C) * rpc;
-    auto k = rec_kernel<NV, C>;
+    auto k = rec_kernel<NV, C, true>;
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;
@@ -1075,7 +1062,7 @@ static int rec_occ_t(int rpc) {
 template <int NV, bool C>
 static cudaError_t launch_rec_t(const BwdParams& P, int grid, int rpc, cudaStream_t st) {
     size_t smem = rod_smem_bytes(NV, C) * rpc;
-    auto k = rec_kernel<NV, C>;
+    auto k = P.mode ? rec_kernel<NV, C, true> : rec_kernel<NV, C, false>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     k<<<grid, threads_per_rod(NV) * rpc, smem, st>>>(P);

@@ -40,6 +40,18 @@ struct PlainWs {
     long long P;      // pair slots
 };
 
+// Edges first, first+2, ... < last of one colour of the red-black inextensibility sweep.
+__device__ __forceinline__ void color_range(int ne, bool closed, int color, int& first, int& last) {
+    const bool three = closed && (ne & 1);
+    if (color == 2) {
+        first = ne - 1;
+        last = ne;
+    } else {
+        first = color;
+        last = (color == 0 && three) ? ne - 1 : ne;
+    }
+}
+
 __device__ __forceinline__ int nsub_of(const RodInfo& R, int force) { return force > 0 ? force : R.nsub; }
 
 // gripper block of substep s (positions, rotations and rigid velocities, Sec. 3.2)

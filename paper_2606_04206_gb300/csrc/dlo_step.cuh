@@ -536,64 +536,44 @@ __device__ int broad_phase_hash(const RodInfo& R, Smem<NV, CONTACT>& s, const Gr
 }
 
 // ------------------------------------------------------------------ PBD pieces
-// Edges first, first+2, ... < last of one colour of the red-black inextensibility sweep.
-__device__ __forceinline__ void color_range(int ne, bool closed, int color, int& first, int& last) {
-    const bool three = closed && (ne & 1);
-    if (color == 2) {
-        first = ne - 1;
-        last = ne;
-    } else {
-        first = color;
-        last = (color == 0 && three) ? ne - 1 : ne;
-    }
+// Length projections (inextensibility, strain limit): edges of even index, then of odd index
+// (an odd loop's last edge after both), N_C times.  Thread t of the first pbd_threads takes the
+// edges 2t and 2t + 1: vertex 2t + 1 belongs to no other edge and stays in its registers, as do the
+// edges' start vectors, targets and weights; only the even vertices go through shared memory,
+// one load and one store per colour, between barriers of the projecting warps alone.  (Every
+// thread meeting at a barrier per colour and reading both ends' positions, displacements and
+// the rest length took about 480 cycles per colour.)
+__host__ __device__ constexpr int pbd_threads(int NV) { return NV <= 64 ? 32 : (NV / 2 + 31) / 32 * 32; }
+
+// Barrier of a rod's projecting threads (bar: the rod's own barrier, 1..4 where this one is named).
+template <int NV>
+__device__ __forceinline__ void pbd_sync(int bar) {
+    if (pbd_threads(NV) == 32)
+        __syncwarp();
+    else
+        asm volatile("bar.sync %0, %1;" ::"r"(bar + 7), "r"(pbd_threads(NV)) : "memory");
 }
 
-// One colour of inextensibility / strain-limit projections (App. A.1) on displacements D
-// from start positions X0: C = |x_{j+1} - x_j| - |ebar|, lambda = C / (w_j + w_{j+1}).
-// prec (optional): receives each edge's projection record (Rec::pbd).
-template <int TPR>
-__device__ __forceinline__ void inext_color_arr(const RodInfo& R, const float4* X0, float4* D, const float4* ET,
-                                                const Grp<TPR>& g, int color, bool closed, float4* prec = nullptr) {
-    const int ne = R.ne, nv = R.nv;
-    int first, last;
-    color_range(ne, closed, color, first, last);
-    const bool inext = R.flags & ROD_INEXT;
-    for (int j = first + 2 * g.tid; j < last; j += 2 * TPR) {
-        int j1 = (j + 1 == nv) ? 0 : j + 1;
-        float4 A = D[j], B = D[j1];              // displacements (w = inverse mass)
-        V3<float> e = (f3(X0[j1]) - f3(X0[j])) + (f3(B) - f3(A));
-        float ell, ie;
-        len_inv(e, ell, ie);
-        float eb = ET[j].w;
-        float target;
-        bool active;
-        if (inext) {
-            target = eb;
-            active = true;
-        } else {
-            float hi = (1.f + R.slim) * eb, lo = (1.f - R.slim) * eb;
-            active = (ell > hi) || (ell < lo);
-            target = ell > hi ? hi : lo;
-        }
-        float ws = A.w + B.w;
-        if (!active || !(ws > 0.f) || !(eb > 0.f)) {   // eb = 0: the edge between two strands
-            if (prec) prec[j] = make_float4(0.f, 0.f, 0.f, 1.f);
-            continue;
-        }
-        float lam = (ell - target) / ws;
-        V3<float> t = ie * e;
-        if (prec) prec[j] = f4(t, target * ie);
-        V3<float> da = (lam * A.w) * t, db = (lam * B.w) * t;
-        D[j] = make_float4(A.x + da.x, A.y + da.y, A.z + da.z, A.w);
-        D[j1] = make_float4(B.x - db.x, B.y - db.y, B.z - db.z, B.w);
-    }
-    g.sync();
-}
+struct ProjEdge {
+    bool on;          // an edge with a length and at least one free end
+    V3<float> r;      // start vector
+    float hi, lo;     // bounds of the length (equal for an inextensible edge)
+    float wa, wb, ws;
+};
 
-template <int NV, bool CONTACT, int TPR>
-__device__ __forceinline__ void inext_color(const RodInfo& R, Smem<NV, CONTACT>& s, const Grp<TPR>& g, int color,
-                                            bool closed, float4* prec = nullptr) {
-    inext_color_arr<TPR>(R, s.X0, s.X, s.ET, g, color, closed, prec);
+// One projection (App. A.1) of the edge between displacements A and B: C = |x_{j+1} - x_j| -
+// target, lambda = C / (w_j + w_{j+1}).  Returns its record (Rec::pbd).
+__device__ __forceinline__ float4 project_edge(const ProjEdge& p, bool inext, V3<float>& A, V3<float>& B) {
+    const V3<float> e = p.r + (B - A);
+    float ell, ie;
+    len_inv(e, ell, ie);
+    const float target = ell > p.hi ? p.hi : p.lo;
+    if (!(p.on && (inext || ell > p.hi || ell < p.lo))) return make_float4(0.f, 0.f, 0.f, 1.f);
+    const float lam = (ell - target) / p.ws;
+    const V3<float> t = ie * e;
+    A += (lam * p.wa) * t;
+    B -= (lam * p.wb) * t;
+    return f4(t, target * ie);
 }
 
 template <int NV, bool CONTACT, int TPR>
@@ -683,16 +663,93 @@ __device__ __forceinline__ void self_friction(const RodInfo& R, Smem<NV, CONTACT
     g.sync();
 }
 
-// The contact sweep and friction as out-of-line calls.  They run only on frames with
+// The N_C projection iterations of a substep on the displacements s.X: the length projections of
+// both colours and, with SWEEPS, a self-contact sweep.  The group has synchronised since s.X was
+// written; on return it has synchronised after the last iteration.
+template <int NV, bool CONTACT, int TPR, bool REC, bool SWEEPS>
+__device__ __forceinline__ void run_projections(const RodInfo& R, Smem<NV, CONTACT>& s, const Grp<TPR>& g, int n_iter, int np,
+                                        const Rec<NV, REC> rec) {
+    const int nv = R.nv, ne = R.ne, i = g.tid;
+    const bool closed = R.flags & ROD_CLOSED, lenc = R.flags & (ROD_INEXT | ROD_SLIMIT), inext = R.flags & ROD_INEXT;
+    const bool ring = closed && (ne & 1);
+    const bool proj = lenc && i < pbd_threads(NV);
+    const int j = 2 * i, j2 = j + 2 >= nv ? 0 : j + 2;   // the edges j (to j + 1) and j + 1 (to j2)
+    const bool last = ring && j == ne - 1;               // edge j is an odd loop's last: ends at vertex 0
+    ProjEdge p0{}, p1{};
+    V3<float> mid = zf3();                               // displacement of vertex j + 1
+    if (proj) {
+        auto edge = [&](int k, int k1) {
+            ProjEdge p;
+            const float len = s.ET[k].w;
+            const float4 xa = s.X0[k], xb = s.X0[k1];
+            p.r = f3(xb) - f3(xa);
+            p.hi = inext ? len : (1.f + R.slim) * len;
+            p.lo = inext ? len : (1.f - R.slim) * len;
+            p.wa = xa.w;
+            p.wb = xb.w;
+            p.ws = xa.w + xb.w;
+            p.on = p.ws > 0.f && len > 0.f;   // length 0: the edge between two strands
+            return p;
+        };
+        if (j < ne) p0 = edge(j, last || j + 1 == nv ? 0 : j + 1);
+        if (j + 1 < ne) p1 = edge(j + 1, j2);
+        if (j + 1 < nv) mid = f3(s.X[j + 1]);
+    }
+    for (int it = 0; it < n_iter; ++it) {
+        if (proj) {
+            auto put = [&](int k, float4 q) {
+                if (REC) rec.pbd(it)[k] = q;
+            };
+            if (j < ne && !last) {
+                const float4 a4 = s.X[j];
+                V3<float> A = f3(a4);
+                put(j, project_edge(p0, inext, A, mid));
+                s.X[j] = f4(A, a4.w);
+            }
+            pbd_sync<NV>(g.bar);
+            if (j + 1 < ne) {
+                const float4 b4 = s.X[j2];
+                V3<float> B = f3(b4);
+                put(j + 1, project_edge(p1, inext, mid, B));
+                s.X[j2] = f4(B, b4.w);
+            }
+            if (SWEEPS || it + 1 == n_iter)
+                if (j + 1 < nv) s.X[j + 1] = f4(mid, p0.wb);
+            if (ring) {
+                pbd_sync<NV>(g.bar);
+                if (last) {
+                    const float4 a4 = s.X[j], b4 = s.X[0];
+                    V3<float> A = f3(a4), B = f3(b4);
+                    put(j, project_edge(p0, inext, A, B));
+                    s.X[j] = f4(A, a4.w);
+                    s.X[0] = f4(B, b4.w);
+                }
+            }
+            if (!SWEEPS) pbd_sync<NV>(g.bar);
+        }
+        if (SWEEPS) {
+            if (lenc) g.sync();
+            // each thread stores its own vertices; the sweep reads s.X and writes only the
+            // accumulators before its own barrier
+            if (REC && i < nv) rec.csnap(it)[i] = s.X[i];
+            contact_sweep<NV, CONTACT, TPR>(R, s, g, np, it == 0);
+            if (proj && j + 1 < nv) mid = f3(s.X[j + 1]);
+        }
+    }
+    if (!SWEEPS) g.sync();
+}
+
+// With contact sweeps, and the friction, as out-of-line calls.  They run only on frames with
 // candidates; kept out of the substep's inlined code they add no registers, and no code, to
 // the path every substep takes.  The rod's shared-memory view is rebuilt from its base
 // inside (a view passed by reference would be read from memory at every use).
-template <int NV, bool CONTACT, int TPR>
-__device__ __noinline__ void contact_sweep_call(const RodInfo* R, float4* base, int gtid, int gbar, int np,
-                                                bool first) {
+template <int NV, bool CONTACT, int TPR, bool REC>
+__device__ __noinline__ void run_projections_call(const RodInfo* Rp, float4* base, int gtid, int gbar, int n_iter, int np,
+                                          float4* rec) {
     Smem<NV, CONTACT> s(base);
     const Grp<TPR> g{gtid, gbar, s.red};
-    contact_sweep<NV, CONTACT, TPR>(*R, s, g, np, first);
+    const RodInfo R = *Rp;
+    run_projections<NV, CONTACT, TPR, REC, true>(R, s, g, n_iter, np, Rec<NV, REC>{rec, n_iter});
 }
 
 template <int NV, bool CONTACT, int TPR>
@@ -891,19 +948,10 @@ __device__ __forceinline__ void substep_body(const SceneDev& sc, const float4* _
     g.sync();
     if (!project) return;
     // --- PBD
-    for (int it = 0; it < sc.n_iter; ++it) {
-        if (lenc) {
-            const int ncol = (closed && (ne & 1)) ? 3 : 2;
-            for (int k = 0; k < ncol; ++k)
-                inext_color<NV, CONTACT, TPR>(R, s, g, k, closed, REC ? rec.pbd(it) : nullptr);
-        }
-        if (CONTACT && np > 0) {
-            // each thread stores its own vertices; the sweep reads s.X and writes only the
-            // accumulators before its own barrier
-            if (REC && vtx) rec.csnap(it)[i] = s.X[i];
-            contact_sweep_call<NV, CONTACT, TPR>(&R, s.X, g.tid, g.bar, np, it == 0);
-        }
-    }
+    if (CONTACT && np > 0)
+        run_projections_call<NV, CONTACT, TPR, REC>(&R, s.X, g.tid, g.bar, sc.n_iter, np, rec.base);
+    else
+        run_projections<NV, CONTACT, TPR, REC, false>(R, s, g, sc.n_iter, 0, rec);
     // --- velocity from the displacement, new positions, friction
     if (vtx) {
         const float4 d = s.X[i];
