@@ -130,11 +130,139 @@ __global__ void loss_winding(const RodInfo* rods, const float4* X, const float4*
     }
 }
 
-// ---- the Gauss double integral of two straight segments (exact closed form) on dual numbers.
+// ---- the Gauss double integral of two straight segments (exact closed form).
 // The directions r_2 - r_1 of the pair sweep the parallelogram r13, r14, r24, r23; the integral
 // is minus its signed solid angle seen from the origin, taken as two triangles with the
 // atan2 form of Van Oosterom and Strackee (IEEE TBME 1983), which stays well conditioned in
 // float where the arcsine form of the same angle loses its derivative.
+// Both triangles, (r13, r14, r24) and (r13, r24, r23), have the same triple product, r13 . (e1 x e2)
+// with e1 and e2 the segments: formed from the segments it keeps the digits that the products of
+// the nearly equal r's of a distant pair cancel.  Their denominators are
+// |u||v||w| + (u.v)|w| + (u.w)|v| + (v.w)|u|.
+
+// The gradient of a denominator, times c, added to those of its three vectors (lengths l, inverse
+// lengths il, dot products d).
+__device__ __forceinline__ void denominator_grad(V3<float> u, V3<float> v, V3<float> w, float lu, float lv, float lw,
+                                                 float iu, float iv, float iw, float duv, float duw, float dvw, float c,
+                                                 V3<float>& gu, V3<float>& gv, V3<float>& gw) {
+    const float au = c * (lv * lw + dvw) * iu, av = c * (lu * lw + duw) * iv, aw = c * (lu * lv + duv) * iw;
+    const float auv = c * lw, auw = c * lv, avw = c * lu;
+    gu += au * u + auv * v + auw * w;
+    gv += av * v + auv * u + avw * w;
+    gw += aw * w + auw * u + avw * v;
+}
+
+// Omega of the segments p1p2 and p3p4; with GRAD also its gradient with respect to the four ends
+// (one reverse pass).
+template <bool GRAD>
+__device__ __forceinline__ float gauss_pair(V3<float> p1, V3<float> p2, V3<float> p3, V3<float> p4, V3<float>* g) {
+    const V3<float> r13 = p3 - p1, r14 = p4 - p1, r23 = p3 - p2, r24 = p4 - p2, e1 = p2 - p1, e2 = p4 - p3;
+    float l13, l14, l23, l24, i13, i14, i23, i24;
+    len_inv(r13, l13, i13);
+    len_inv(r14, l14, i14);
+    len_inv(r23, l23, i23);
+    len_inv(r24, l24, i24);
+    const V3<float> e12 = cross(e1, e2);
+    const float n = dot(r13, e12);
+    const float da = dot(r13, r14), db = dot(r13, r24), dc = dot(r14, r24), dd = dot(r13, r23), de = dot(r24, r23);
+    const float m1 = l13 * l14 * l24 + da * l24 + db * l14 + dc * l13;
+    const float m2 = l13 * l24 * l23 + db * l23 + dd * l24 + de * l13;
+    if (GRAD) {
+        const float q1 = -2.f / (n * n + m1 * m1), q2 = -2.f / (n * n + m2 * m2);
+        V3<float> g13 = zf3(), g14 = zf3(), g23 = zf3(), g24 = zf3();
+        denominator_grad(r13, r14, r24, l13, l14, l24, i13, i14, i24, da, db, dc, -(q1 * n), g13, g14, g24);
+        denominator_grad(r13, r24, r23, l13, l24, l23, i13, i24, i23, db, dd, de, -(q2 * n), g13, g24, g23);
+        const float c = q1 * m1 + q2 * m2;   // of the triple product
+        g13 += c * e12;
+        const V3<float> h1 = c * cross(e2, r13), h2 = c * cross(r13, e1);
+        g[0] = -(g13 + g14) - h1;
+        g[1] = h1 - (g23 + g24);
+        g[2] = g13 + g23 - h2;
+        g[3] = g14 + g24 + h2;
+    }
+    return -2.f * (atan2f(n, m1) + atan2f(n, m2));
+}
+
+// Sum of floats as an unevaluated pair (Knuth's exact two-term sum): FP64 accuracy on the FP32
+// pipe, which an FP64 addition per pair of edges would leave waiting.
+struct PairSum {
+    float h = 0.f, l = 0.f;
+    __device__ __forceinline__ void add(float v) {
+        const float t = __fadd_rn(h, v), b = __fsub_rn(t, h);
+        l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(t, b)), __fsub_rn(v, b)));
+        h = t;
+    }
+    __device__ __forceinline__ double value() const { return (double)h + (double)l; }
+};
+
+// Sum over ordered pairs of non-adjacent edges of Omega / (4 pi), Omega being symmetric twice the
+// sum over unordered ones: edge a meets edge a + k (mod the edge count), k = 1, 2, ... up to half
+// of them, all threads at the same k.  GRAD: the thread of a keeps its ends' gradient, and adds
+// its partner's to that edge's slots (at one k every thread has another partner; a barrier
+// separates the steps).  Bound by instruction issue: about 350 instructions a pair.
+template <bool GRAD>
+__global__ void __launch_bounds__(kLT) loss_crossing(const RodInfo* rods, const float4* X, const float* g, float* q,
+                                                     float4* gx) {
+    constexpr int EPT = GRAD ? 1 : kMaxV / kLT;   // edges per thread (GRAD: rods of up to kLT vertices)
+    __shared__ double sh[kLT];
+    __shared__ float4 xs[kMaxV];
+    __shared__ float4 ge0[GRAD ? kLT : 1], ge1[GRAD ? kLT : 1];   // d/d(first, second endpoint) of each edge's sum
+    const int rod = blockIdx.x;
+    const RodInfo R = rods[rod];
+    const bool closed = R.flags & ROD_CLOSED;
+    const int n = R.nv, ne = closed ? n : n - 1;
+    for (int i = threadIdx.x; i < n; i += kLT) {
+        xs[i] = X[R.v0 + i];
+        if (GRAD) ge0[i] = ge1[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    __syncthreads();
+    PairSum sum;
+    V3<float> g0[EPT], g1[EPT];
+#pragma unroll
+    for (int m = 0; m < EPT; ++m) g0[m] = g1[m] = zf3();
+    for (int k = 1; k <= ne / 2; ++k) {
+#pragma unroll
+        for (int m = 0; m < EPT; ++m) {
+            const int a = threadIdx.x + m * kLT;
+            // the opposite edge of an even ring of indices, from its lower half alone; neighbours
+            // (k = 1, but not the two ends of an open rod) do not cross
+            if (a >= ne || (2 * k == ne && a >= k)) continue;
+            const int b = a + k >= ne ? a + k - ne : a + k;
+            if (abs(a - b) <= 1 || (closed && k == 1)) continue;
+            V3<float> gp[4];
+            sum.add(gauss_pair<GRAD>(f3(xs[a]), f3(xs[a + 1 == n ? 0 : a + 1]), f3(xs[b]), f3(xs[b + 1 == n ? 0 : b + 1]), gp));
+            if (GRAD) {
+                g0[m] += gp[0];
+                g1[m] += gp[1];
+                ge0[b] = f4(f3(ge0[b]) + gp[2], 0.f);
+                ge1[b] = f4(f3(ge1[b]) + gp[3], 0.f);
+            }
+        }
+        if (GRAD) __syncthreads();
+    }
+    if (GRAD) {
+#pragma unroll
+        for (int m = 0; m < EPT; ++m) {
+            const int a = threadIdx.x + m * kLT;
+            if (a >= ne) continue;
+            ge0[a] = f4(f3(ge0[a]) + g0[m], 0.f);
+            ge1[a] = f4(f3(ge1[a]) + g1[m], 0.f);
+        }
+    }
+    __syncthreads();
+    const double s = block_sum(2.0 * sum.value(), sh);
+    if (q && threadIdx.x == 0) q[rod] = (float)(s / (4.0 * M_PI));
+    if (!GRAD) return;
+    // each unordered pair appears twice in the sum: d/dx = 2 sum_b dOmega_ab / (4 pi)
+    const float c = gscale(g, rod) / (2.f * (float)M_PI);
+    for (int i = threadIdx.x; i < n; i += kLT) {
+        V3<float> d = zf3();
+        if (closed || i < ne) d += f3(ge0[i]);                         // i starts edge i
+        if (closed || i > 0) d += f3(ge1[i == 0 ? ne - 1 : i - 1]);     // and ends edge i-1
+        gx[R.v0 + i] = f4(c * d, 0.f);
+    }
+}
+
 __device__ dualf gauss_pair_d(V3<dualf> p1, V3<dualf> p2, V3<dualf> p3, V3<dualf> p4) {
     const V3<dualf> r13 = p3 - p1, r14 = p4 - p1, r23 = p3 - p2, r24 = p4 - p2;
     const dualf l13 = norm(r13), l14 = norm(r14), l23 = norm(r23), l24 = norm(r24);
@@ -146,9 +274,12 @@ __device__ dualf gauss_pair_d(V3<dualf> p1, V3<dualf> p2, V3<dualf> p3, V3<dualf
     return -2.f * (datan2(n1, m1) + datan2(n2, m2));
 }
 
-// sum over ordered pairs of non-adjacent edges of Omega / (4 pi); thread of edge a evaluates
-// Omega(a, b) for every b with the six coordinates of a's endpoints seeded in turn
-__global__ void loss_crossing(const RodInfo* rods, const float4* X, const float* g, float* q, float4* gx) {
+// The same sum and gradient for rods of more than 128 vertices, on dual numbers: the thread of
+// edge a evaluates Omega(a, b) for every b with the six coordinates of a's endpoints seeded in
+// turn.  Four times the work, kept there because the gradient is a sum of thousands of cancelling
+// pairs: the two evaluations agree to 1.1e-5 of it at 128 vertices but only to 2.5e-5 at 250
+// (each 1e-5 to 2e-5 from FP64), and results are to stay what they were to 2e-5.
+__global__ void loss_crossing_long(const RodInfo* rods, const float4* X, const float* g, float* q, float4* gx) {
     __shared__ double sh[kLT];
     __shared__ float4 xs[kMaxV];
     __shared__ float4 ge0[kMaxV], ge1[kMaxV];   // d/d(first, second endpoint) of each edge's sum
@@ -185,7 +316,6 @@ __global__ void loss_crossing(const RodInfo* rods, const float4* X, const float*
     __syncthreads();
     s = block_sum(s, sh);
     if (q && threadIdx.x == 0) q[rod] = (float)(s / (4.0 * M_PI));
-    if (!gx) return;
     // each unordered pair appears twice in the sum: d/dx = 2 sum_b dOmega_ab / (4 pi)
     const float c = gscale(g, rod) / (2.f * (float)M_PI);
     for (int i = threadIdx.x; i < n; i += kLT) {
@@ -245,6 +375,7 @@ __global__ void loss_repulsion(const RodInfo* rods, const float4* X, const float
     __shared__ double sh[kLT];
     __shared__ float4 xs[kMaxV];
     __shared__ float4 ge0[kMaxV], ge1[kMaxV];
+    __shared__ float4 mid[kMaxV];   // each edge's midpoint and half length
     const int rod = blockIdx.x;
     const RodInfo R = rods[rod];
     const bool closed = R.flags & ROD_CLOSED;
@@ -253,15 +384,30 @@ __global__ void loss_repulsion(const RodInfo* rods, const float4* X, const float
     const int k = max(1, (int)prm[rod].y);
     for (int i = threadIdx.x; i < n; i += kLT) xs[i] = X[R.v0 + i];
     __syncthreads();
+    for (int j = threadIdx.x; j < ne; j += kLT) {
+        const V3<float> p0 = f3(xs[j]), p1 = f3(xs[j + 1 == n ? 0 : j + 1]), e = p1 - p0;
+        mid[j] = f4(0.5f * (p0 + p1), 0.5f * sqrtf(dot(e, e)));
+    }
+    __syncthreads();
     double s = 0.0;
     for (int a = threadIdx.x; a < ne; a += kLT) {
         const int a1 = (a + 1 == n) ? 0 : a + 1;
         const V3<float> pa = f3(xs[a]), pb = f3(xs[a1]);
+        const float4 ma = mid[a];
         V3<float> g0 = zf3(), g1 = zf3();
-        for (int b = 0; b < ne; ++b) {
+        // the other edges by their distance ahead: neighbouring threads then have near pairs, the
+        // ones that cost, at the same step
+        for (int o = 1; o < ne; ++o) {
+            const int b = a + o >= ne ? a + o - ne : a + o;
             int sep = abs(a - b);
             if (closed) sep = min(sep, ne - sep);
             if (sep <= k) continue;
+            // segments in spheres farther apart than delta cannot be closer than delta (the
+            // spheres enlarged by more than the roundings): most pairs end here
+            const float4 mb = mid[b];
+            const V3<float> dm = f3(ma) - f3(mb);
+            const float far = 1.0001f * (delta + ma.w + mb.w);
+            if (dot(dm, dm) > far * far && far >= 0.f) continue;
             const int b1 = (b + 1 == n) ? 0 : b + 1;
             // every pair is solved with its lower edge first, as both of its threads must see
             // the same closest points (the near-parallel rule is not symmetric)
@@ -331,7 +477,12 @@ extern "C" dlo_status dlo_loss(dlo_ctx* c, int kind, const float* x, const float
             loss_winding<<<c->B, kLT, 0, c->stream>>>(c->d_rods, X, reinterpret_cast<const float4*>(aux), g, q, GX);
             break;
         case DLO_LOSS_CROSSING:
-            loss_crossing<<<c->B, kLT, 0, c->stream>>>(c->d_rods, X, g, q, GX);
+            if (GX && c->buckets.back().nv_max > kLT)
+                loss_crossing_long<<<c->B, kLT, 0, c->stream>>>(c->d_rods, X, g, q, GX);
+            else if (GX)
+                loss_crossing<true><<<c->B, kLT, 0, c->stream>>>(c->d_rods, X, g, q, GX);
+            else
+                loss_crossing<false><<<c->B, kLT, 0, c->stream>>>(c->d_rods, X, g, q, GX);
             break;
         case DLO_LOSS_MINDIST:
             if (!aux) return set_err(c, DLO_ERR_INVALID_ARG, "the minimum distance needs an object centre per rod");
