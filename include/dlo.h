@@ -178,7 +178,11 @@ dlo_status dlo_get_internal(dlo_ctx* ctx, float* ref, float* tan, float* hinge, 
  * opt.checkpoint_every, or when that is 0 the shortest interval whose ring, action record
  * and backward workspace fit opt.hbm_budget (80 GiB by default).  It also sets how many
  * frames the backward reverses per launch pair: its chunk records may take half of what the
- * ring and the action record leave of the budget (at most 24 GiB).
+ * ring and the action record leave of the budget (at most 24 GiB).  When the records of the
+ * whole rollout fit that share (and 64 frames), dlo_step stores them while it steps, in memory
+ * allocated here, and dlo_backward does not step again; when they do not fit, when that
+ * memory cannot be allocated, or when a step is captured in a graph, dlo_backward recomputes
+ * them from the checkpoints.  The gradients are the same.
  * Defined by: the gradient checkpointing of Sec. 3.3 (checkpoints kept in HBM here).
  * Errors: DLO_ERR_INVALID_ARG for n_frames <= 0; DLO_ERR_OOM when the ring cannot be
  * allocated. */
@@ -218,7 +222,8 @@ dlo_status dlo_backward_plain(dlo_ctx* ctx, const float* dL_dx_T, const float* d
                               float* dL_dx0, float* dL_dv0, float* dL_dtheta0);
 
 /* Differentiate the recorded rollout (the gradient through time of Sec. 3.3, computed by a
- * hand-written adjoint that replays each frame from its checkpoint).  Inputs (device, may be
+ * hand-written adjoint over every substep's records, stored by dlo_step or recomputed by
+ * replaying each frame from its checkpoint).  Inputs (device, may be
  * NULL = zero): dL/dx_T [V][4]
  * (w ignored), dL/dv_T [V][4] (w = dL/d twist rate), dL/dtheta_T [Etot].  Outputs (device,
  * may be NULL = not wanted): dL/dactions [F][B][2][6], dL/dmaterial [B][5] for

@@ -8,6 +8,8 @@
 // chunk's frames from their start state storing every substep's records, then rev_kernel
 // reverses them (dlo_bwd_kernel.cuh).  C is a multiple of K when C >= K, so that every chunk
 // starts at a checkpoint; otherwise the frame-start states of each segment are stored first.
+// When one chunk holds the whole rollout, the forward stores the records itself and rec_kernel
+// does not run.
 #include <algorithm>
 #include <cstring>
 #include <vector>
@@ -250,10 +252,17 @@ void best_shape(int nv, bool contact, bool rec, int& w, int& nb) {
 
 }  // namespace
 
+void backward_shapes(dlo_ctx* c) {
+    for (Bucket& bk : c->buckets) {
+        best_shape(bk.nv_max, bk.contact, true, bk.rec_w, bk.rec_nb);
+        best_shape(bk.nv_max, bk.contact, false, bk.rev_w, bk.rev_nb);
+    }
+}
+
 // Plan of the chunked backward for checkpoint interval K: frames per chunk C (the records of
 // one chunk of every rod within rec_budget, at most 64 frames), per-rod buffer sizes and the
 // workspace of all rods at once.
-dlo_status bwd_plan(dlo_ctx* c, int force, int K, BwdPlan& out, size_t rec_budget) {
+dlo_status bwd_plan(dlo_ctx* c, int force, int K, BwdPlan& out, size_t rec_budget, int frames) {
     const size_t nb_ = c->buckets.size();
     if (!rec_budget) {
         const size_t budget = c->opt.hbm_budget ? c->opt.hbm_budget : ((size_t)80 << 30);
@@ -265,14 +274,13 @@ dlo_status bwd_plan(dlo_ctx* c, int force, int K, BwdPlan& out, size_t rec_budge
     out.l2_rod.assign(nb_, 0);
     out.cs_rod.assign(nb_, 0);
     out.offset.assign(nb_, 0);
+    out.sub_off.assign(nb_, 0);
+    out.rest_off.assign(nb_, 0);
     size_t per_frame = 0;
     for (size_t k = 0; k < nb_; ++k) {
         const Bucket& bk = c->buckets[k];
-        int w, nb;
-        best_shape(bk.nv_max, bk.contact, false, w, nb);
-        if (w < 1) return set_err(c, DLO_ERR_INVALID_ARG, "rod too large for the backward kernel's shared memory");
-        best_shape(bk.nv_max, bk.contact, true, w, nb);
-        if (w < 1) return set_err(c, DLO_ERR_INVALID_ARG, "rod too large for the recompute kernel's shared memory");
+        if (bk.rev_w < 1) return set_err(c, DLO_ERR_INVALID_ARG, "rod too large for the backward kernel's shared memory");
+        if (bk.rec_w < 1) return set_err(c, DLO_ERR_INVALID_ARG, "rod too large for the recompute kernel's shared memory");
         int ns = force;
         if (!ns)
             for (int b = 0; b < c->B; ++b)
@@ -281,8 +289,10 @@ dlo_status bwd_plan(dlo_ctx* c, int force, int K, BwdPlan& out, size_t rec_budge
         per_frame += 16 * (size_t)bk.n * frame_rec_h(bk.nv_max, c->opt.n_iter_pbd, ns);
     }
     int C = (int)std::max<size_t>(1, std::min<size_t>(64, rec_budget / std::max<size_t>(per_frame, 1)));
+    if (frames > 0) C = std::min(C, (frames + K - 1) / K * K);
     if (C >= K) C = (C / K) * K;   // chunks start at checkpoints
-    size_t need = 0;
+    size_t need = 0, sub = 0, rest = 0;
+    auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
     for (size_t k = 0; k < nb_; ++k) {
         const Bucket& bk = c->buckets[k];
         const int NV = bk.nv_max;
@@ -291,15 +301,27 @@ dlo_status bwd_plan(dlo_ctx* c, int force, int K, BwdPlan& out, size_t rec_budge
         out.l2_rod[k] = C < K ? (size_t)K * (5 * (size_t)NV + 6) : 0;
         out.cs_rod[k] = 5 * (size_t)NV + 6;
         out.offset[k] = need;   // each class has its own region: the classes run concurrently
-        need += (16 * (size_t)bk.n * (out.r3_rod[k] + out.l2_rod[k] + out.cs_rod[k]) + 255) & ~(size_t)255;
+        need += up(16 * (size_t)bk.n * (out.r3_rod[k] + out.l2_rod[k] + out.cs_rod[k]));
+        out.sub_off[k] = sub;
+        out.rest_off[k] = rest;
+        sub += up(16 * (size_t)bk.n * out.r3_rod[k]);
+        rest += up(16 * (size_t)bk.n * (out.l2_rod[k] + out.cs_rod[k]));
     }
     out.fixed = (2 * 16 * (size_t)c->Et + 255) & ~(size_t)255;
     out.bytes = out.fixed + need;
+    out.sub_bytes = sub;
+    out.rest_bytes = out.fixed + rest;
     return DLO_OK;
 }
 
+bool records_fit(const dlo_ctx* c, const BwdPlan& plan) {
+    for (int C : plan.C)
+        if (C < c->rec_frames) return false;
+    return plan.sub_bytes <= c->sub_bytes;
+}
+
 dlo_status enqueue_backward_class(dlo_ctx* c, const BwdPlan& plan, size_t k, cudaStream_t st, int item0, int n,
-                                  float4* R3, float4* L2, float4* CS, int C, const BwdParams& common) {
+                                  float4* R3, float4* L2, float4* CS, int C, const BwdParams& common, bool stored) {
     const Bucket& bk = c->buckets[k];
     BwdParams P = common;
     P.order = bk.d_order;
@@ -311,11 +333,9 @@ dlo_status enqueue_backward_class(dlo_ctx* c, const BwdPlan& plan, size_t k, cud
     P.L2 = L2;
     P.CS = CS;
     backward_rod_f4(c, plan, k, C, P.r3_rod, P.l2_rod, P.cs_rod);
-    int rec_w, rec_nb, rev_w, rev_nb;
-    best_shape(bk.nv_max, bk.contact, true, rec_w, rec_nb);
-    best_shape(bk.nv_max, bk.contact, false, rev_w, rev_nb);
-    const int rec_grid = (int)std::min<long long>((long long)rec_nb * c->sm_count, (n + rec_w - 1) / rec_w);
-    const int rev_grid = (int)std::min<long long>((long long)rev_nb * c->sm_count, (n + rev_w - 1) / rev_w);
+    const int rec_w = bk.rec_w, rev_w = bk.rev_w;
+    const int rec_grid = (int)std::min<long long>((long long)bk.rec_nb * c->sm_count, (n + rec_w - 1) / rec_w);
+    const int rev_grid = (int)std::min<long long>((long long)bk.rev_nb * c->sm_count, (n + rev_w - 1) / rev_w);
     const int K = c->ck_every, F = c->rec_frames;
     // the chunks, first to last: from every checkpoint when C >= K (C a multiple of K), else
     // within each segment
@@ -343,13 +363,16 @@ dlo_status enqueue_backward_class(dlo_ctx* c, const BwdPlan& plan, size_t k, cud
         P.mode = 1;
         P.fa = fa;
         P.fb = fb;
-        if (e == cudaSuccess) e = cudaMemsetAsync(P.counter, 0, sizeof(int), st);
-        if (e == cudaSuccess) e = launch_rec(P, bk.nv_max, bk.contact, rec_grid, rec_w, st);
+        if (!stored) {
+            if (e == cudaSuccess) e = cudaMemsetAsync(P.counter, 0, sizeof(int), st);
+            if (e == cudaSuccess) e = launch_rec(P, bk.nv_max, bk.contact, rec_grid, rec_w, st);
+            c->launches++;
+        }
         P.first_chunk = fb == F;
         P.last_chunk = fa == 0;
         if (e == cudaSuccess) e = cudaMemsetAsync(P.counter, 0, sizeof(int), st);
         if (e == cudaSuccess) e = launch_rev(P, bk.nv_max, bk.contact, rev_grid, rev_w, st);
-        c->launches += 2;
+        c->launches++;
         if (e != cudaSuccess) return cuda_err(c, e, "backward launch");
     }
     return DLO_OK;
@@ -363,9 +386,7 @@ void backward_rod_f4(dlo_ctx* c, const BwdPlan& plan, size_t k, int C, size_t& r
 }
 
 int backward_resident_rods(dlo_ctx* c, size_t k) {
-    int w, nb;
-    best_shape(c->buckets[k].nv_max, c->buckets[k].contact, false, w, nb);
-    return w * nb * c->sm_count;
+    return c->buckets[k].rev_w * c->buckets[k].rev_nb * c->sm_count;
 }
 
 // the inputs and outputs shared by every launch of one backward
@@ -413,12 +434,14 @@ extern "C" dlo_status dlo_backward(dlo_ctx* c, const float* dL_dx_T, const float
         return set_err(c, DLO_ERR_INVALID_ARG, "self-contact gradients need at least one projection iteration");
     const int force = c->rec_nsub > 0 ? c->rec_nsub : 0;
     BwdPlan plan;
-    dlo_status pst = bwd_plan(c, force, c->ck_every, plan, c->rec_budget);
+    dlo_status pst = bwd_plan(c, force, c->ck_every, plan, c->rec_budget, c->rec_frames);
     if (pst != DLO_OK) return pst;
-    if (plan.bytes > c->bw_bytes) {
+    const bool stored = c->rec_stored && records_fit(c, plan);
+    const size_t bytes = stored ? plan.rest_bytes : plan.bytes;
+    if (bytes > c->bw_bytes) {
         dev_free(c, c->bw_mem);
-        c->bw_mem = dev_alloc(c, plan.bytes);
-        c->bw_bytes = c->bw_mem ? plan.bytes : 0;
+        c->bw_mem = dev_alloc(c, bytes);
+        c->bw_bytes = c->bw_mem ? bytes : 0;
         if (!c->bw_mem) return set_err(c, DLO_ERR_OOM, "backward workspace allocation failed");
     }
     char* p = reinterpret_cast<char*>(c->bw_mem);
@@ -433,10 +456,12 @@ extern "C" dlo_status dlo_backward(dlo_ctx* c, const float* dL_dx_T, const float
     }
     for (size_t k = 0; k < c->buckets.size(); ++k) {
         const int n = c->buckets[k].n;
-        float4* R3 = reinterpret_cast<float4*>(region + plan.offset[k]);
-        float4* L2 = R3 + (size_t)n * plan.r3_rod[k];
+        float4* R3 = reinterpret_cast<float4*>(stored ? reinterpret_cast<char*>(c->sub_mem) + plan.sub_off[k]
+                                                      : region + plan.offset[k]);
+        float4* L2 = stored ? reinterpret_cast<float4*>(region + plan.rest_off[k]) : R3 + (size_t)n * plan.r3_rod[k];
         float4* CS = L2 + (size_t)n * plan.l2_rod[k];
-        dlo_status st = enqueue_backward_class(c, plan, k, class_stream(c, k), 0, n, R3, L2, CS, plan.C[k], common);
+        dlo_status st = enqueue_backward_class(c, plan, k, class_stream(c, k), 0, n, R3, L2, CS, plan.C[k], common,
+                                               stored);
         if (st != DLO_OK) return st;
     }
     {

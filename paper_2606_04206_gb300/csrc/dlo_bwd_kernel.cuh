@@ -143,19 +143,6 @@ struct RevSmem {
     }
 };
 
-// State snapshot layout in the per-rod scratch: X[NV], V[NV], HG[NV], ED[NV], ET[NV].
-template <int NV, bool C, int TPR>
-__device__ __forceinline__ void save_state(float4* dst, const RodInfo& R, const Grp<TPR>& g, const Smem<NV, C>& s) {
-    for (int i = g.tid; i < R.nv; i += TPR) {
-        dst[i] = s.X0[i];
-        dst[NV + i] = s.V[i];
-        dst[2 * NV + i] = s.HG[i];
-    }
-    for (int j = g.tid; j < R.ne; j += TPR) {
-        dst[3 * NV + j] = s.ED[j];
-        dst[4 * NV + j] = s.ET[j];
-    }
-}
 // row-major 3x3 at o times v
 __device__ __forceinline__ V3<float> mul_rm(const float* o, V3<float> v) {
     return f3(o[0] * v.x + o[1] * v.y + o[2] * v.z, o[3] * v.x + o[4] * v.y + o[5] * v.z,
@@ -696,29 +683,6 @@ __device__ __forceinline__ void reverse_substep(const BwdParams& P, const RodInf
     }
 }
 
-// ------------------------------------------------------------------ record layout
-// Records of one chunk of frames, per rod (float4 units; NV the size class, n the substeps
-// reserved per frame, N the projection iterations):
-//   per frame, kFrameHead + NV:  its start pose (24 floats) and candidate count (int at float 24),
-//                                then its candidate pairs (4 NV uint32)
-//   per substep, sub_rec(NV, N): start state (X0, V, HG, ED, ET; 5 NV), v1 (NV), dfin (NV),
-//                                projection records (N NV), contact snapshots (N NV), first-
-//                                iteration pair data fr0, fr1 (4 NV each)
-// Only what a frame uses is written and read (projection records for length-constrained rods,
-// snapshots and pair data for frames with candidates).
-constexpr int kFrameHead = 8;
-__host__ __device__ constexpr size_t sub_rec(int NV, int n_iter) {
-    return (size_t)(7 + 2 * n_iter + 2 * kPairsPerVertex) * NV;
-}
-__host__ __device__ constexpr size_t frame_rec(int NV, int n_iter, int nsub) {
-    return (size_t)(kFrameHead + NV) + (size_t)nsub * sub_rec(NV, n_iter);
-}
-// frame-start state of one frame of a segment: X0, V, HG, ED, ET and the pose (24 floats)
-__host__ __device__ constexpr size_t seg_state(int NV) { return (size_t)5 * NV + 6; }
-// cotangent state carried from one chunk's reverse to the next: LX, LV, LE, LT, LK, then the
-// material sums (5 doubles) and the frame-start pose cotangents (12 floats)
-__host__ __device__ constexpr size_t cot_state(int NV) { return (size_t)5 * NV + 6; }
-
 // CTAs per SM the reverse kernel is compiled for.  Up to 128 vertices 384 threads per SM (168
 // registers): with 512 (128 registers) 120 registers spill and 4096 ropes x 128 take 12.1 instead
 // of 11.6 ms.  Above, two CTAs: with one (255 registers, no spills) 1024 bands x 200 in contact
@@ -739,7 +703,7 @@ __global__ void __launch_bounds__(kFwdMaxThreads) rec_kernel(BwdParams P) {
     const Grp<TPR> g{(int)(threadIdx.x % TPR), 1 + slot, s.red};
     const SceneDev& sc = P.scene;
     const int n_iter = sc.n_iter;
-    const size_t SR = sub_rec(NV, n_iter), FR = frame_rec(NV, n_iter, P.nsub_max);
+    const size_t FR = frame_rec(NV, n_iter, P.nsub_max);
     if (CONTACT)   // the contact accumulators start at zero; every sweep leaves them at zero
         for (int i = g.tid; i < NV; i += TPR) s.acc[i] = make_int4(0, 0, 0, 0);
     for (;;) {
@@ -809,15 +773,9 @@ __global__ void __launch_bounds__(kFwdMaxThreads) rec_kernel(BwdParams P) {
                 if (g.tid < 12) s.act[g.tid] = P.actions[((size_t)f * P.B + rod) * 12 + g.tid];
                 g.sync();
                 const int np = run_frame<NV, CONTACT, TPR>(sc, P.KIN, R, own, s, g, nsub, h, ovf, [&](int sb) {
-                    float4* e3 = fb + kFrameHead + NV + (size_t)sb * SR;
-                    save_state<NV, CONTACT, TPR>(e3, R, g, s);   // each thread its own vertex and edge
-                    return Rec<NV, true>{e3, n_iter};
+                    return record_substep<NV, CONTACT, TPR>(fb, sb, n_iter, R, g, s);
                 });
-                if (CONTACT) {
-                    uint32_t* pl = reinterpret_cast<uint32_t*>(fb + kFrameHead);
-                    for (int p = g.tid; p < np; p += TPR) pl[p] = s.pairs[p];
-                    if (g.tid == 0) reinterpret_cast<int*>(fb)[24] = np;
-                }
+                if (CONTACT) record_pairs<NV, CONTACT, TPR>(fb, np, g, s);
             }
         }
         g.sync();
@@ -888,7 +846,7 @@ __global__ void __launch_bounds__(NV, rev_min_ctas(NV)) rev_kernel(BwdParams P) 
             }
         }
         // carried sums: the pose cotangents of frame fb's start, positions (2 x 3) then rotations
-        if (i < 12) s.PC[i] = P.first_chunk ? 0.0 : (double)reinterpret_cast<const float*>(CS + 5 * NV + 3)[i];
+        if (i < 12) s.PC[i] = P.first_chunk ? 0.0 : reinterpret_cast<const double*>(CS + 4 * NV)[2 * i + 1];
         for (int m = 0; m < 5; ++m) s.GM[m * NV + i] = make_float2(0.f, 0.f);
         bool touched = true;
         for (int f = P.fb - 1; f >= P.fa; --f) {
@@ -999,7 +957,7 @@ __global__ void __launch_bounds__(NV, rev_min_ctas(NV)) rev_kernel(BwdParams P) 
             if (vtx) {
                 CS[i] = lx;
                 CS[NV + i] = lv;
-                CS[4 * NV + i] = make_float4(c.k0, c.k1, 0.f, 0.f);
+                reinterpret_cast<float2*>(CS + 4 * NV)[2 * i] = make_float2(c.k0, c.k1);
             }
             if (has_e) {
                 CS[2 * NV + i] = f4(c.d1, c.th);
@@ -1010,7 +968,7 @@ __global__ void __launch_bounds__(NV, rev_min_ctas(NV)) rev_kernel(BwdParams P) 
 #pragma unroll
                 for (int m = 0; m < 5; ++m) d[m] = gm[m];
             }
-            if (i < 12) reinterpret_cast<float*>(CS + 5 * NV + 3)[i] = (float)s.PC[i];
+            if (i < 12) reinterpret_cast<double*>(CS + 4 * NV)[2 * i + 1] = s.PC[i];
         }
         g.sync();
         bounds_end<TPR>(g, P.status, rod);

@@ -26,7 +26,8 @@ __device__ __forceinline__ void write_state(const StateRef& D, long long offV, l
         for (int k = 0; k < 24; ++k) D.GP[offB + 24LL * rod + k] = gp[k];
 }
 
-template <int NV, bool CONTACT>
+// REC: every substep's records are stored as well (FwdParams::R3).
+template <int NV, bool CONTACT, bool REC>
 __global__ void __launch_bounds__(kFwdMaxThreads) fwd_kernel(FwdParams P) {
     constexpr int TPR = threads_per_rod(NV);
     extern __shared__ float4 dyn_smem[];
@@ -74,13 +75,25 @@ __global__ void __launch_bounds__(kFwdMaxThreads) fwd_kernel(FwdParams P) {
                 write_state<TPR>(P.ck, c * P.ck_strideV, c * P.ck_strideE, c * P.ck_strideB, R, rod, g, s.X0, s.V,
                                  s.ED, s.ET, s.HG, s.fp);
             }
+            float4* fb = nullptr;
+            if (REC) {
+                fb = P.R3 + (size_t)item * P.r3_rod + (size_t)gf * frame_rec(NV, P.scene.n_iter, P.nsub_max);
+                if (g.tid < 24) reinterpret_cast<float*>(fb)[g.tid] = s.fp[g.tid];
+            }
             if (g.tid < 12) s.act[g.tid] = P.actions ? P.actions[((long long)f * P.B + rod) * 12 + g.tid] : 0.f;
             g.sync();
             bool ovf = false;
             float mv = 0.f;
             const int np = run_frame<NV, CONTACT, TPR>(P.scene, P.KIN, R, own, s, g, nsub, h, ovf,
-                                                       [](int) { return Rec<NV, false>{nullptr, 0}; },
+                                                       [&](int sb) {
+                                                           if constexpr (REC)
+                                                               return record_substep<NV, CONTACT, TPR>(
+                                                                   fb, sb, P.scene.n_iter, R, g, s);
+                                                           else
+                                                               return Rec<NV, false>{nullptr, 0};
+                                                       },
                                                        P.reaction ? P.reaction + 4LL * R.v0 : nullptr, &mv);
+            if (REC && CONTACT) record_pairs<NV, CONTACT, TPR>(fb, np, g, s);
             if (ovf) bad |= 2u;
             np_max = max(np_max, np);
             unsigned fl = 0u;
@@ -132,7 +145,7 @@ __host__ __device__ constexpr int fwd_max_rpc() { return kFwdMaxThreads / thread
 template <int NV, bool C>
 static cudaError_t launch_fwd_t(const FwdParams& P, int grid, int rpc, cudaStream_t st) {
     size_t smem = rod_smem_bytes(NV, C) * rpc;
-    auto k = fwd_kernel<NV, C>;
+    auto k = P.R3 ? fwd_kernel<NV, C, true> : fwd_kernel<NV, C, false>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     k<<<grid, threads_per_rod(NV) * rpc, smem, st>>>(P);
@@ -143,7 +156,7 @@ template <int NV, bool C>
 static int fwd_occ_t(int rpc) {
     if (rpc > fwd_max_rpc<NV>() || rpc < 1) return 0;
     size_t smem = rod_smem_bytes(NV, C) * rpc;
-    auto k = fwd_kernel<NV, C>;
+    auto k = fwd_kernel<NV, C, false>;
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;

@@ -75,6 +75,11 @@ struct FwdParams {
     StateRef ck;
     long long ck_strideV, ck_strideE, ck_strideB;
     int ck_every, ck_count;
+    // substep records for the adjoint, when the whole rollout's fit: [n_order][rollout frames][frame
+    // record], or null (the adjoint recomputes them)
+    float4* R3;
+    size_t r3_rod;
+    int nsub_max;
     unsigned* status;         // [B] bit 1 non-finite, bit 2 pair overflow, bit 4 moved past the margin
     double* residual;         // [B]
     int* npairs;              // [B]

@@ -1186,6 +1186,7 @@ extern "C" dlo_status dlo_step_plain(dlo_ctx* c, const float* actions, int frame
     const float* acts = actions;
     if (rec) {   // the actions are recorded for the backward, as by dlo_step
         c->rec_nsub = substeps;
+        c->rec_stored = false;   // no substep records
         float* dst = c->rec_actions + (size_t)12 * B * c->rec_done;
         cudaError_t e = actions ? cudaMemcpyAsync(dst, actions, sizeof(float) * 12 * B * frames,
                                                   cudaMemcpyDeviceToDevice, c->stream)

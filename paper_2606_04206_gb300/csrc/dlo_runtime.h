@@ -17,9 +17,25 @@ struct Bucket {
     int* d_order = nullptr; // rod ids by decreasing cost (vertices x substeps)
     int warps = 0;          // rods in flight per CTA of the forward kernel
     int grid = 0;           // persistent CTAs
+    // rods per CTA and CTAs per SM of the backward's kernels (0: not possible)
+    int rec_w = 0, rec_nb = 0, rev_w = 0, rev_nb = 0;
 };
 }  // namespace dlo
 
+// launch shapes and workspace of the chunked backward for a checkpoint interval (dlo_adjoint.cu)
+struct BwdPlan {
+    // per size class: substeps reserved per frame, frames per chunk, float4 per rod of the
+    // chunk records (R3), of the segment's frame-start states (L2, empty when chunks start at
+    // checkpoints) and of the carried cotangent state (CS); the class's region in the workspace
+    std::vector<int> nsmax, C;
+    std::vector<size_t> r3_rod, l2_rod, cs_rod, offset;
+    size_t fixed = 0;    // initial-frame cotangents
+    size_t bytes = 0;    // everything, for all rods at once
+    // the same with the chunk records apart (in memory the forward fills): each class's offset
+    // there and their total, and each class's offset and the total of the rest
+    std::vector<size_t> sub_off, rest_off;
+    size_t sub_bytes = 0, rest_bytes = 0;
+};
 struct dlo_ctx {
     int B = 0;
     long long V = 0, Et = 0;
@@ -64,6 +80,11 @@ struct dlo_ctx {
     int rec_frames = 0, rec_done = 0, rec_nsub = 0;
     int ck_every = 0, ck_count = 0;
     size_t rec_budget = 0;   // chunk-record bytes the backward may use (set by dlo_begin_rollout)
+    // substep records of the whole rollout, stored by the forward when they fit the budget
+    bool rec_stored = false;
+    BwdPlan rec_plan;        // the plan they were laid out with
+    void* sub_mem = nullptr;
+    size_t sub_bytes = 0;
     dlo::StateRef ck{};
     void* ck_mem = nullptr;
     size_t ck_bytes = 0;
@@ -80,26 +101,23 @@ struct dlo_ctx {
     size_t sil_bytes = 0;
 };
 
-// launch shapes and workspace of the chunked backward for a checkpoint interval (dlo_adjoint.cu)
-struct BwdPlan {
-    // per size class: substeps reserved per frame, frames per chunk, float4 per rod of the
-    // chunk records (R3), of the segment's frame-start states (L2, empty when chunks start at
-    // checkpoints) and of the carried cotangent state (CS); the class's region in the workspace
-    std::vector<int> nsmax, C;
-    std::vector<size_t> r3_rod, l2_rod, cs_rod, offset;
-    size_t fixed = 0;    // initial-frame cotangents
-    size_t bytes = 0;    // everything, for all rods at once
-};
 // the stream of size class k, and the fork / join around work issued on those streams
 cudaStream_t class_stream(dlo_ctx* c, size_t k);
 cudaError_t fork_classes(dlo_ctx* c);
 cudaError_t join_classes(dlo_ctx* c);
-// rec_budget: bytes allowed for the chunk records of all classes (0 = the default)
-dlo_status bwd_plan(dlo_ctx* c, int force, int K, BwdPlan& out, size_t rec_budget = 0);
+// Bucket::rec_* and rev_*, once at create (occupancy queries take microseconds each).
+void backward_shapes(dlo_ctx* c);
+// rec_budget: bytes allowed for the chunk records of all classes (0 = the default); frames: the
+// rollout's (0 = not known: chunks are not cut to it)
+dlo_status bwd_plan(dlo_ctx* c, int force, int K, BwdPlan& out, size_t rec_budget = 0, int frames = 0);
+// Whether the plan's chunks hold the whole rollout and the memory for its records is there.
+bool records_fit(const dlo_ctx* c, const BwdPlan& plan);
 // Enqueue the backward of size class k for the rods order[item0 .. item0 + n) on stream st,
 // with that class's R3 / L2 / CS buffers sized for n rods; common holds the outputs and inputs.
+// stored: R3 already holds the whole rollout's records.
 dlo_status enqueue_backward_class(dlo_ctx* c, const BwdPlan& plan, size_t k, cudaStream_t st, int item0, int n,
-                                  float4* R3, float4* L2, float4* CS, int C, const dlo::BwdParams& common);
+                                  float4* R3, float4* L2, float4* CS, int C, const dlo::BwdParams& common,
+                                  bool stored = false);
 // the launch inputs and outputs shared by every kernel of one backward
 dlo::BwdParams backward_common(dlo_ctx* c, int force, const float* dL_dx_T, const float* dL_dv_T,
                                const float* dL_dtheta_T, float* dL_dactions, float* dL_dmaterial, float* dL_dx0,

@@ -1010,6 +1010,61 @@ __device__ __forceinline__ void frame_advance(float* F, const float* act, int q)
     for (int k = 0; k < 9; ++k) f[3 + k] = Rn.m[k];
 }
 
+// ------------------------------------------------------------------ record layout
+// Records of a run of frames (a chunk, or the whole rollout), per rod (float4 units; NV the size
+// class, n the substeps reserved per frame, N the projection iterations):
+//   per frame, kFrameHead + NV:  its start pose (24 floats) and candidate count (int at float 24),
+//                                then its candidate pairs (4 NV uint32)
+//   per substep, sub_rec(NV, N): start state (X0, V, HG, ED, ET; 5 NV), v1 (NV), dfin (NV),
+//                                projection records (N NV), contact snapshots (N NV), first-
+//                                iteration pair data fr0, fr1 (4 NV each)
+// Only what a frame uses is written and read (projection records for length-constrained rods,
+// snapshots and pair data for frames with candidates).
+constexpr int kFrameHead = 8;
+__host__ __device__ constexpr size_t sub_rec(int NV, int n_iter) {
+    return (size_t)(7 + 2 * n_iter + 2 * kPairsPerVertex) * NV;
+}
+__host__ __device__ constexpr size_t frame_rec(int NV, int n_iter, int nsub) {
+    return (size_t)(kFrameHead + NV) + (size_t)nsub * sub_rec(NV, n_iter);
+}
+// frame-start state of one frame of a segment: X0, V, HG, ED, ET and the pose (24 floats)
+__host__ __device__ constexpr size_t seg_state(int NV) { return (size_t)5 * NV + 6; }
+// cotangent state carried from one chunk's reverse to the next: LX, LV, LE, LT, LK (two floats,
+// and in the upper half of the first 12 the frame-start pose cotangents, a double each), then
+// the material sums (5 doubles)
+__host__ __device__ constexpr size_t cot_state(int NV) { return (size_t)5 * NV + 6; }
+
+// State snapshot layout in the per-rod scratch: X[NV], V[NV], HG[NV], ED[NV], ET[NV].
+template <int NV, bool C, int TPR>
+__device__ __forceinline__ void save_state(float4* dst, const RodInfo& R, const Grp<TPR>& g, const Smem<NV, C>& s) {
+    for (int i = g.tid; i < R.nv; i += TPR) {
+        dst[i] = s.X0[i];
+        dst[NV + i] = s.V[i];
+        dst[2 * NV + i] = s.HG[i];
+    }
+    for (int j = g.tid; j < R.ne; j += TPR) {
+        dst[3 * NV + j] = s.ED[j];
+        dst[4 * NV + j] = s.ET[j];
+    }
+}
+
+// The records of substep sb of the frame whose record is fb: stores its start state (each thread
+// its own vertex and edge) and returns where the substep stores the rest.
+template <int NV, bool CONTACT, int TPR>
+__device__ __forceinline__ Rec<NV, true> record_substep(float4* fb, int sb, int n_iter, const RodInfo& R,
+                                                        const Grp<TPR>& g, const Smem<NV, CONTACT>& s) {
+    float4* e3 = fb + kFrameHead + NV + (size_t)sb * sub_rec(NV, n_iter);
+    save_state<NV, CONTACT, TPR>(e3, R, g, s);
+    return Rec<NV, true>{e3, n_iter};
+}
+// The frame's candidates, into its record.
+template <int NV, bool CONTACT, int TPR>
+__device__ __forceinline__ void record_pairs(float4* fb, int np, const Grp<TPR>& g, const Smem<NV, CONTACT>& s) {
+    uint32_t* pl = reinterpret_cast<uint32_t*>(fb + kFrameHead);
+    for (int p = g.tid; p < np; p += TPR) pl[p] = s.pairs[p];
+    if (g.tid == 0) reinterpret_cast<int*>(fb)[24] = np;
+}
+
 // One frame of one rod: candidates (if self-contact), nsub substeps, pose update.  The frame's
 // start pose is s.fp and its actions s.act, both set (and synchronised) by the caller; s.fp
 // holds the end pose on return.  pre(sb) runs before substep sb (after a group barrier), e.g.
