@@ -128,6 +128,8 @@ DLO_HD float cross_comp(float p, float q, float r, float s) {   // p q - r s
     return p * q - r * s;
 #endif
 }
+template <class T>
+DLO_HD V3<T> cross_fixed(V3<T> a, V3<T> b) { return cross(a, b); }   // scalars without roundings to fix
 DLO_HD V3<float> cross_fixed(V3<float> a, V3<float> b) {
     return {cross_comp(a.y, b.z, a.z, b.y), cross_comp(a.z, b.x, a.x, b.z), cross_comp(a.x, b.y, a.y, b.x)};
 }
