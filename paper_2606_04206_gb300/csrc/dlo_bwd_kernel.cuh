@@ -107,6 +107,24 @@ __device__ __forceinline__ V3<T> prim_respond(int k, const SceneDev& sc, const R
     return contact_respond(v, sdf, n, vrig, R.radius, R.eps, sc.mu_rigid, sc.restitution, act);
 }
 
+// What the reverse reads of the substep before is copied to shared memory while the present
+// one is reversed: each thread's own state rows, and of the projection records (each
+// projecting thread its own two edges') the last proj_rows(NV) iterations, the rest as they are
+// used up.  Read from memory when needed, the state cost its latency once per substep and the
+// records, fetched one iteration ahead, once per iteration: of 4096 cables x 128 vertices the
+// reverse takes 8.9 instead of 11.1 ms (16 frames).  Fewer rows where more would leave
+// room for fewer CTAs on the SM.
+__host__ __device__ constexpr int proj_rows(int NV) { return NV == 64 || NV == 128 ? 10 : 5; }
+__device__ __forceinline__ void copy16(float4* dst, const float4* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copies_wait() {   // for all but the last N groups of this thread
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
 // Shared memory of one rod of the reverse kernel: what a neighbour (or another vertex of a
 // contact pair) reads, and the frame's gripper data.
 template <int NV, bool CONTACT>
@@ -116,13 +134,16 @@ struct RevSmem {
     float2* GM;                 // [5][NV]: the threads' material sums, each an unevaluated sum of two floats
     float* PA;                  // [24][NV]: the threads' pose terms of the frame: positions (2 x 3),
                                 // rotations (2 x 3), actions (2 x 6)
+    float4* ST;                 // [6][NV]: X0, V, HG, ED, ET, v1 of the substep reversed next
+    float4* PR;                 // [proj_rows][NV]: projection records, iterations in the order of the reverse
+    float4* WB;                 // [NV / 2]: weights of the projecting threads' edges
     uint32_t* pairs;
     float *red, *f0, *act;      // reduction scratch, the frame's start pose (24) and actions (12)
     float *sp, *PM;             // per substep of a batch: gripper blocks (64) and pose maps (72)
     double* PC;                 // the carried pose cotangents (12)
     float* GA;                  // the frame's action cotangents carried from the next frame's pose (12)
     static constexpr size_t kHeader = 64 + 24 + 16 + 64 * kPoseBatch + 72 * kPoseBatch + 2 * 12 + 16;
-    static constexpr size_t kBytes = 16 * (size_t)(5 * NV) + 8 * (size_t)(5 * NV) + 4 * (size_t)(24 * NV) +
+    static constexpr size_t kBytes = 16 * (size_t)((11 + proj_rows(NV)) * NV + NV / 2) + 8 * (size_t)(5 * NV) + 4 * (size_t)(24 * NV) +
                                      (CONTACT ? 4 * (size_t)(kPairsPerVertex * NV) : 0) + 4 * kHeader;
     __device__ explicit RevSmem(float4* b) {
         LD = b;
@@ -130,7 +151,10 @@ struct RevSmem {
         F1 = b + 2 * NV;
         F2 = b + 3 * NV;
         F3 = b + 4 * NV;
-        GM = reinterpret_cast<float2*>(b + 5 * NV);
+        ST = b + 5 * NV;
+        PR = b + 11 * NV;
+        WB = PR + proj_rows(NV) * NV;
+        GM = reinterpret_cast<float2*>(WB + NV / 2);
         PA = reinterpret_cast<float*>(GM + 5 * NV);
         PC = reinterpret_cast<double*>(PA + 24 * NV);
         red = reinterpret_cast<float*>(PC + 12);
@@ -328,7 +352,7 @@ struct Cot {
 struct PbdRev {
     bool e0, e1, ring;         // edge 2t, edge 2t + 1 are projected; edge 2t is an odd loop's last (its own colour)
     int i0, i2;                // vertices 2t and the end of edge 2t + 1
-    float a0, b0, a1, b1;      // w_a / (w_a + w_b), w_b / (w_a + w_b) of both
+    float a0, b0, a1, b1;      // w_a / (w_a + w_b), w_b / (w_a + w_b) of both (RevSmem::WB)
     V3<float> s0, s1;          // sums over the iterations
 };
 
@@ -341,8 +365,41 @@ __device__ __forceinline__ V3<float> project_rev(float4 q, float a, float b, V3<
     return mu - q.w * (mu - dot(mu, t) * t);
 }
 
+// Copies of the substep reversed next (RevSmem::ST, PR); base: its records.
+template <int NV, bool CONTACT>
+__device__ __forceinline__ void fetch_state(const RevSmem<NV, CONTACT>& s, const RodInfo& R, const float4* base, int i) {
+    if (i < R.nv) {
+        copy16(s.ST + i, base + i);
+        copy16(s.ST + NV + i, base + NV + i);
+        copy16(s.ST + 2 * NV + i, base + 2 * NV + i);
+        copy16(s.ST + 5 * NV + i, base + 5 * NV + i);
+    }
+    if (i < R.ne) {
+        copy16(s.ST + 3 * NV + i, base + 3 * NV + i);
+        copy16(s.ST + 4 * NV + i, base + 4 * NV + i);
+    }
+    copies_commit();
+}
+// iteration it's records of the edges 2 i and 2 i + 1 into row `row`
+template <int NV, bool CONTACT>
+__device__ __forceinline__ void fetch_projection(const RevSmem<NV, CONTACT>& s, const RodInfo& R, const float4* base, int it,
+                                                 int row, int i) {
+    const float4* src = base + (size_t)(7 + it) * NV + 2 * i;
+    float4* dst = s.PR + row * NV + 2 * i;
+    if (2 * i < R.ne) copy16(dst, src);
+    if (2 * i + 1 < R.ne) copy16(dst + 1, src + 1);
+}
+template <int NV, bool CONTACT>
+__device__ __forceinline__ void fetch_projections(const RevSmem<NV, CONTACT>& s, const RodInfo& R, const float4* base,
+                                                  int n_iter, int i) {
+#pragma unroll 1
+    for (int k = 0; k < min(n_iter, proj_rows(NV)); ++k) fetch_projection<NV>(s, R, base, n_iter - 1 - k, k, i);
+    copies_commit();
+}
+
 // ------------------------------------------------------------------ reverse of one substep
-// rec: the substep's records.  c holds the cotangents of S_{n+1} on entry and of S_n on exit.
+// rec: the substep's records, of which the state and the first projection rows are in s;
+// before: the records of the substep reversed next (null: none).  c holds the cotangents of S_{n+1} on entry and of S_n on exit.
 // sp, pm: the substep's gripper block and pose maps.  touched: set when the thread adds to its
 // pose terms.
 // Bound by latency: dependent arithmetic of few warps (registers), barriers and record loads.
@@ -350,7 +407,8 @@ __device__ __forceinline__ V3<float> project_rev(float4 q, float a, float b, V3<
 template <int NV, bool CONTACT>
 __device__ __forceinline__ void reverse_substep(const BwdParams& P, const RodInfo& R, const RodInfo* Rp, const Own& own,
                                                 float4 kin, float eb, float eba, RevSmem<NV, CONTACT>& s,
-                                                const Grp<NV>& g, const Rec<NV, true> rec, float h, float c0, float c1,
+                                                const Grp<NV>& g, const Rec<NV, true> rec, const float4* before,
+                                                float h, float c0, float c1,
                                                 int np, const float* sp, const float* pm, Cot& c,
                                                 bool& touched) {
     const SceneDev& sc = P.scene;
@@ -366,21 +424,23 @@ __device__ __forceinline__ void reverse_substep(const BwdParams& P, const RodInf
     const float4* S = rec.base;
     float4 x4 = make_float4(0.f, 0.f, 0.f, 0.f), v4 = x4, xb = x4, hg = x4, ed = x4, et = x4, v1 = x4;
     float tha = 0.f;
+    copies_wait<0>();   // the own copies are there
+    g.sync();   // so are the other threads'; LD of the substep after this one has been read and the
+                // frame's shared data is written
     if (vtx) {
-        x4 = S[i];
-        v4 = S[NV + i];
-        v1 = rec.v1()[i];
+        x4 = s.ST[i];
+        v4 = s.ST[NV + i];
+        v1 = s.ST[5 * NV + i];
     }
     if (has_e) {
-        xb = S[ip];
-        ed = S[3 * NV + i];
-        et = S[4 * NV + i];
+        xb = s.ST[ip];
+        ed = s.ST[3 * NV + i];
+        et = s.ST[4 * NV + i];
     }
     if (has_em) {
-        hg = S[2 * NV + i];
-        tha = S[3 * NV + im].w;
+        hg = s.ST[2 * NV + i];
+        tha = s.ST[3 * NV + im].w;
     }
-    g.sync();   // LD of the substep after this one has been read; its frame's shared data is written
     // ---- positions at the substep end, and the velocity rebuilt from the displacement
     const bool held = own.kind >= 2;
     V3<float> ld = held ? zf3() : c.x, dx = zf3(), lp0 = zf3();
@@ -430,7 +490,7 @@ __device__ __forceinline__ void reverse_substep(const BwdParams& P, const RodInf
         const int ncol = lenc ? ((closed && (ne & 1)) ? 3 : 2) : 0;
         const bool proj = lenc && i < PT;
         PbdRev b{};
-        float4 q0 = make_float4(0.f, 0.f, 0.f, 1.f), q1 = q0;
+        int row = 0;   // of PR: the iteration's
         if (proj) {
             const int j = 2 * i;
             b.e0 = j < ne;
@@ -438,17 +498,12 @@ __device__ __forceinline__ void reverse_substep(const BwdParams& P, const RodInf
             b.ring = ncol == 3 && j == ne - 1;
             b.i0 = min(j, nv - 1);
             b.i2 = j + 2 >= nv ? 0 : j + 2;
-            const float4* W = S;
-            const float w0 = b.e0 ? W[j].w : 0.f, w1 = b.e0 ? W[j + 1 == nv ? 0 : j + 1].w : 0.f,
-                        w2 = b.e1 ? W[b.i2].w : 0.f;
-            b.a0 = w0 + w1 > 0.f ? w0 / (w0 + w1) : 0.f;
-            b.b0 = w0 + w1 > 0.f ? w1 / (w0 + w1) : 0.f;
-            b.a1 = w1 + w2 > 0.f ? w1 / (w1 + w2) : 0.f;
-            b.b1 = w1 + w2 > 0.f ? w2 / (w1 + w2) : 0.f;
+            const float4 w = b.e0 ? s.WB[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+            b.a0 = w.x;
+            b.b0 = w.y;
+            b.a1 = w.z;
+            b.b1 = w.w;
             b.s0 = b.s1 = zf3();
-            const float4* Q = rec.pbd(sc.n_iter - 1);
-            if (b.e0) q0 = Q[j];
-            if (b.e1) q1 = Q[j + 1];
         }
         if (vtx) s.LD[i] = f4(ld, 0.f);
         g.sync();
@@ -487,13 +542,9 @@ __device__ __forceinline__ void reverse_substep(const BwdParams& P, const RodInf
                 g.sync();
             }
             if (proj) {
-                // the records of the iteration before, fetched while this one is reversed
-                const float4 r0 = q0, r1 = q1;
-                if (it > 0) {
-                    const float4* Q = rec.pbd(it - 1);
-                    if (b.e0) q0 = Q[2 * i];
-                    if (b.e1) q1 = Q[2 * i + 1];
-                }
+                if (sc.n_iter - 1 - it >= proj_rows(NV)) copies_wait<proj_rows(NV) - 1>();
+                const float4 none = make_float4(0.f, 0.f, 0.f, 1.f), r0 = b.e0 ? s.PR[row * NV + 2 * i] : none,
+                             r1 = b.e1 ? s.PR[row * NV + 2 * i + 1] : none;
                 if (ncol == 3) {
                     if (b.ring) {
                         const V3<float> la = f3(s.LD[b.i0]), lb = f3(s.LD[0]);
@@ -521,6 +572,11 @@ __device__ __forceinline__ void reverse_substep(const BwdParams& P, const RodInf
                     s.LD[2 * i + 1] = f4(lm + le, 0.f);
                     b.s0 += le;
                 }
+                if (sc.n_iter > proj_rows(NV)) {   // the row just used up takes the iteration proj_rows further on
+                    if (it >= proj_rows(NV)) fetch_projection<NV>(s, R, S, it - proj_rows(NV), row, i);
+                    copies_commit();
+                }
+                row = row + 1 == proj_rows(NV) ? 0 : row + 1;
                 pbd_sync<NV>(g.bar);
             }
             if (CONTACT && np > 0) g.sync();
@@ -528,6 +584,7 @@ __device__ __forceinline__ void reverse_substep(const BwdParams& P, const RodInf
         if (proj) {   // F0: each edge's summed cotangent
             if (b.e0) s.F0[2 * i] = f4(b.s0, 0.f);
             if (b.e1) s.F0[2 * i + 1] = f4(b.s1, 0.f);
+            if (before) fetch_projections<NV>(s, R, before, sc.n_iter, i);
         }
         g.sync();
         if (vtx) {
@@ -572,6 +629,7 @@ __device__ __forceinline__ void reverse_substep(const BwdParams& P, const RodInf
         s.LD[i] = lg;
     }
     g.sync();
+    if (before) fetch_state<NV>(s, R, before, i);   // everyone has read this substep's
     // ---- the own edge's frame as dual numbers in the direction of the force cotangents, the
     // reverse of its stretching
     EdgeF<dualf> E;
@@ -849,6 +907,22 @@ __global__ void __launch_bounds__(NV, rev_min_ctas(NV)) rev_kernel(BwdParams P) 
         if (i < 12) s.PC[i] = P.first_chunk ? 0.0 : reinterpret_cast<const double*>(CS + 4 * NV)[2 * i + 1];
         for (int m = 0; m < 5; ++m) s.GM[m * NV + i] = make_float2(0.f, 0.f);
         bool touched = true;
+        {   // the copies of the last substep, and the projecting threads' weights (the inverse masses
+            // are the same in every record)
+            const float4* last = P.R3 + (size_t)k * P.r3_rod + (size_t)(P.fb - 1 - P.fa) * FR + kFrameHead + NV +
+                                 (size_t)(nsub - 1) * SR;
+            g.sync();   // the rod before has been reversed
+            fetch_state<NV>(s, R, last, i);
+            if ((R.flags & (ROD_INEXT | ROD_SLIMIT)) && i < pbd_threads(NV)) {
+                fetch_projections<NV>(s, R, last, n_iter, i);
+                const int j = 2 * i;
+                const float w0 = j < R.ne ? last[j].w : 0.f, w1 = j < R.ne ? last[j + 1 == R.nv ? 0 : j + 1].w : 0.f,
+                            w2 = j + 1 < R.ne ? last[j + 2 >= R.nv ? 0 : j + 2].w : 0.f;
+                if (j < NV)
+                    s.WB[i] = make_float4(w0 + w1 > 0.f ? w0 / (w0 + w1) : 0.f, w0 + w1 > 0.f ? w1 / (w0 + w1) : 0.f,
+                                          w1 + w2 > 0.f ? w1 / (w1 + w2) : 0.f, w1 + w2 > 0.f ? w2 / (w1 + w2) : 0.f);
+            }
+        }
         for (int f = P.fb - 1; f >= P.fa; --f) {
             const float4* fb = P.R3 + (size_t)k * P.r3_rod + (size_t)(f - P.fa) * FR;
             g.sync();   // the previous frame's reverse has finished reading the frame's shared data
@@ -902,7 +976,10 @@ __global__ void __launch_bounds__(NV, rev_min_ctas(NV)) rev_kernel(BwdParams P) 
                     }
                 }
                 const Rec<NV, true> rec{const_cast<float4*>(fb) + kFrameHead + NV + (size_t)sb * SR, n_iter};
-                reverse_substep<NV, CONTACT>(P, R, Rp, own, kin, eb, eba, s, g, rec, h, (float)sb / (float)nsub,
+                const float4* before = sb > 0     ? rec.base - SR
+                                       : f > P.fa ? fb - FR + kFrameHead + NV + (size_t)(nsub - 1) * SR
+                                                  : nullptr;
+                reverse_substep<NV, CONTACT>(P, R, Rp, own, kin, eb, eba, s, g, rec, before, h, (float)sb / (float)nsub,
                                              (float)(sb + 1) / (float)nsub, np, s.sp + 64 * slot, s.PM + 72 * slot, c,
                                              touched);
             }
