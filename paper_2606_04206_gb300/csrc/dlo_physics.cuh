@@ -137,13 +137,16 @@ DLO_HD V3<dualf> cross_fixed(V3<dualf> a, V3<dualf> b) { return lift(cross_fixed
 
 // The hinge's own part, from its two edges' frames (H.a, H.b: t, d1r, d2r, d1, d2 set).
 template <class T>
-DLO_HD void hinge_core_forward(HingeF<T>& H, T tha, T thb, T mprev) {
+DLO_HD void hinge_bend_forward(HingeF<T>& H) {
     H.cc = 1.f + dot(H.a.t, H.b.t);
     H.X = cross_fixed(H.a.t, H.b.t);
     H.kb = (2.f / H.cc) * H.X;
     H.k0 = 0.5f * dot(H.kb, H.a.d2 + H.b.d2);
     H.k1 = 0.5f * dot(H.kb, H.a.d1 + H.b.d1);
-    // reference twist: angle about t^b from the space-transported d1r^a to d1r^b
+}
+// reference twist: angle about t^b from the space-transported d1r^a to d1r^b
+template <class T>
+DLO_HD void hinge_twist_forward(HingeF<T>& H, T tha, T thb, T mprev) {
     H.u = (H.cc - 1.f) * H.a.d1r + cross(H.X, H.a.d1r) + (dot(H.X, H.a.d1r) / H.cc) * H.X;
     H.y = dot(cross(H.u, H.b.d1r), H.b.t);
     H.xq = dot(H.u, H.b.d1r);
@@ -151,6 +154,11 @@ DLO_HD void hinge_core_forward(HingeF<T>& H, T tha, T thb, T mprev) {
     float wr = rintf((vof(ang) - vof(mprev)) / kTwoPi);
     H.mref = mprev + ((ang - mprev) - kTwoPi * wr);
     H.m = thb - tha + H.mref;
+}
+template <class T>
+DLO_HD void hinge_core_forward(HingeF<T>& H, T tha, T thb, T mprev) {
+    hinge_bend_forward(H);
+    hinge_twist_forward(H, tha, thb, mprev);
 }
 
 template <class T>
@@ -164,10 +172,11 @@ DLO_HD void hinge_forward(HingeF<T>& H, V3<T> xm, V3<T> xi, V3<T> xp, V3<T> tba,
 // Reverse of hinge_core_forward from seeds on kappa (gk0, gk1), on the total twist m (gmt,
 // flows to theta and the reference twist) and on the reference twist alone (gmr): the adjoints
 // of both edges' tangents and reference directors (gta, gd1ra, gtb, gd1rb) and of the two
-// twist angles.
+// twist angles.  Without twist (gmt = gmr = 0, its part of the forward not needed) only the
+// bending part.
 template <class T>
 DLO_HD void hinge_core_reverse(const HingeF<T>& H, T gk0, T gk1, T gmt, T gmr, V3<T>& gta, V3<T>& gd1ra,
-                               V3<T>& gtb_, V3<T>& gd1rb, T& gtha, T& gthb) {
+                               V3<T>& gtb_, V3<T>& gd1rb, T& gtha, T& gthb, bool twist = true) {
     const EdgeF<T>& A = H.a;
     const EdgeF<T>& B = H.b;
     T hk0 = 0.5f * gk0, hk1 = 0.5f * gk1;
@@ -176,21 +185,26 @@ DLO_HD void hinge_core_reverse(const HingeF<T>& H, T gk0, T gk1, T gmt, T gmr, V
     V3<T> gd1 = hk1 * H.kb;
     V3<T> gX = (2.f / H.cc) * gkb;
     T gcc = -dot(gkb, H.kb) / H.cc;
-    // twist
-    T gang = gmt + gmr;
-    gtha = -gmt;
-    gthb = gmt;
-    T r2 = H.y * H.y + H.xq * H.xq;
-    T gy = gang * H.xq / r2;
-    T gxq = -(gang * H.y) / r2;
-    V3<T> gu = gy * cross(B.d1r, B.t) + gxq * B.d1r;
-    gd1rb = gy * cross(B.t, H.u) + gxq * H.u;
-    gtb_ = gy * cross(H.u, B.d1r);
-    T Xd = dot(H.X, A.d1r);
-    T gux = dot(gu, H.X);
-    gcc += dot(gu, A.d1r) - Xd * gux / (H.cc * H.cc);
-    gd1ra = (H.cc - 1.f) * gu + cross(gu, H.X) + (gux / H.cc) * H.X;
-    gX += cross(A.d1r, gu) + (Xd / H.cc) * gu + (gux / H.cc) * A.d1r;
+    if (twist) {
+        T gang = gmt + gmr;
+        gtha = -gmt;
+        gthb = gmt;
+        T r2 = H.y * H.y + H.xq * H.xq;
+        T gy = gang * H.xq / r2;
+        T gxq = -(gang * H.y) / r2;
+        V3<T> gu = gy * cross(B.d1r, B.t) + gxq * B.d1r;
+        gd1rb = gy * cross(B.t, H.u) + gxq * H.u;
+        gtb_ = gy * cross(H.u, B.d1r);
+        T Xd = dot(H.X, A.d1r);
+        T gux = dot(gu, H.X);
+        gcc += dot(gu, A.d1r) - Xd * gux / (H.cc * H.cc);
+        gd1ra = (H.cc - 1.f) * gu + cross(gu, H.X) + (gux / H.cc) * H.X;
+        gX += cross(A.d1r, gu) + (Xd / H.cc) * gu + (gux / H.cc) * A.d1r;
+    } else {
+        const T z = cst<T>(0.f);
+        gtha = gthb = z;
+        gd1ra = gd1rb = gtb_ = V3<T>{z, z, z};
+    }
     gta = gcc * B.t + cross(B.t, gX);
     gtb_ += gcc * A.t + cross(gX, A.t);
     // material frames -> reference frames and twist angles
