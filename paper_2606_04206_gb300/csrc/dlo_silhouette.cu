@@ -56,14 +56,17 @@ __device__ __forceinline__ float4 project(const Cam& c, V3<float> x, float r) {
 
 // signed distance of pixel centre (pu, pv) to the capsule of edge (a, b): distance to the
 // segment minus the edge radius; t is the closest point's parameter, (nu, nv) the unit
-// direction from the closest point to the pixel (zero when they coincide)
+// direction from the closest point to the pixel (zero when they coincide).  The roundings are
+// fixed: at a pixel on the segment's line the direction is decided by them, and both passes
+// should see the same one.
+__device__ __forceinline__ float dot2(float a, float b, float c, float d) { return __fmaf_rn(a, b, __fmul_rn(c, d)); }
 __device__ __forceinline__ float capsule_sd(float pu, float pv, float4 a, float4 b, float rho, float& t, float& nu,
                                             float& nv) {
     const float du = b.x - a.x, dv = b.y - a.y;
-    const float l2 = du * du + dv * dv;
-    t = l2 > 0.f ? fminf(fmaxf(((pu - a.x) * du + (pv - a.y) * dv) / l2, 0.f), 1.f) : 0.f;
-    const float eu = pu - (a.x + t * du), ev = pv - (a.y + t * dv);
-    const float d = sqrtf(eu * eu + ev * ev);
+    const float l2 = dot2(du, du, dv, dv);
+    t = l2 > 0.f ? fminf(fmaxf(dot2(pu - a.x, du, pv - a.y, dv) / l2, 0.f), 1.f) : 0.f;
+    const float eu = pu - __fmaf_rn(t, du, a.x), ev = pv - __fmaf_rn(t, dv, a.y);
+    const float d = sqrtf(dot2(eu, eu, ev, ev));
     nu = d > 0.f ? eu / d : 0.f;
     nv = d > 0.f ? ev / d : 0.f;
     return d - rho;
