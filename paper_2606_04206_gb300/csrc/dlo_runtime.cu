@@ -139,7 +139,17 @@ dlo_status runtime_allocate(dlo_ctx* c, const std::vector<RodInfo>& rods, const 
         c->d_pair_list = reinterpret_cast<uint32_t*>(
             alloc_zero(c, sizeof(uint32_t) * (1 + (size_t)kPairListStride) * c->B, st));
     if (st != DLO_OK) return st;
-    // size classes; rods of a class in decreasing cost so the persistent warps balance
+    // Size classes; rods of a class in decreasing cost, so that the longest do not start last, and
+    // rods of one kind (elastic, with torsion, with length projections) side by side: rods on one SM
+    // that take the same path take it together, and mixed ones keep fetching each other's code.
+    // 4096 rods x 128, a third cables, 16 frames: with the kinds taking turns the forward takes
+    // 4.6 ms and the reverse 8.6 ms, sorted 4.3 and 6.4 ms.  The cost in tenths of an elastic rod's
+    // reverse, from batches of one kind.
+    auto cost = [&](int b) {
+        const RodInfo& R = rods[b];
+        const int kind = 10 + (R.beta != 0.f ? 2 : 0) + (R.flags & (ROD_INEXT | ROD_SLIMIT) ? (6 * c->opt.n_iter_pbd + 9) / 10 : 0);
+        return (long long)R.nv * R.nsub * kind;
+    };
     std::vector<std::vector<int>> cls(kNumSizeClasses);
     for (int b = 0; b < c->B; ++b)
         for (int k = 0; k < kNumSizeClasses; ++k)
@@ -148,7 +158,7 @@ dlo_status runtime_allocate(dlo_ctx* c, const std::vector<RodInfo>& rods, const 
         if (cls[k].empty()) continue;
         std::vector<int>& ids = cls[k];
         std::stable_sort(ids.begin(), ids.end(), [&](int a, int b) {
-            return (long long)rods[a].nv * rods[a].nsub > (long long)rods[b].nv * rods[b].nsub;
+            return cost(a) > cost(b);
         });
         Bucket bk;
         bk.nv_max = size_class_at(k);
