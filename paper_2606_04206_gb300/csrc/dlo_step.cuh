@@ -332,90 +332,122 @@ constexpr int kBpBlock = 8;   // edges per block of the broad phase's first leve
 //   - each edge's segment lies in the sphere around its midpoint with its half length.
 // A segment distance below contact_d implies both sphere distances are below contact_d plus
 // the radii.  Level 1 tests every pair of blocks (one pair per thread) and lists the near
-// ones; level 2 spreads the edge pairs of the listed block pairs over the group, one edge
-// pair per thread, and runs the edge-sphere test, the exclusion window and the exact
-// distance.  Found pairs are appended with a shared-memory atomic (rare), so their order
+// ones; level 2 takes an edge of a listed pair's first block per thread against the eight of its
+// second and runs the edge-sphere test and the exclusion window on the eight side by side; level
+// 3 the exact distance, on the pairs that passed.  (One edge pair per thread, one after the other, and
+// a block's sphere by one thread took 9400 cycles for a loose rope of 128 vertices, a sixth
+// of its frame, most of them the latency of dependent loads; this takes 3800.)  Found pairs are
+// appended with a shared-memory atomic (rare), so their order
 // varies; every use of the list (the Jacobi projection and friction, summed in fixed point,
 // the records of the backward's recompute, the pair-list query) is independent of it.
 template <int NV, bool CONTACT, int TPR>
 __device__ int broad_phase(const RodInfo& R, Smem<NV, CONTACT>& s, const Grp<TPR>& g, bool closed, bool& overflow) {
     float4* mid = s.HB0;                          // midpoint, half length of each edge (-1: a break edge)
-    int* cnt = reinterpret_cast<int*>(s.HB1);     // [0] pairs found, [1] near block pairs
+    int* cnt = reinterpret_cast<int*>(s.HB1);     // [0] pairs found, [1] near block pairs, [2] listed edge pairs
+    constexpr int kList = 4 * kPairsPerVertex * NV;
+    uint32_t* list = reinterpret_cast<uint32_t*>(s.fr0);   // free between substeps
     uint32_t* nearb = reinterpret_cast<uint32_t*>(s.HB1) + 4;   // near block pairs kA | kB << 16, kA <= kB
     float4* blk = s.HB2;                          // centre, radius of each block of edges
     static_assert((NV / kBpBlock + 1) * (NV / kBpBlock + 2) / 2 + 4 <= 4 * NV, "block pairs fit in HB1");
     const int ne = R.ne, nv = R.nv;
     const bool strands = R.flags & ROD_STRANDS;
-    for (int j = g.tid; j < ne; j += TPR) {
-        const int j1 = (j + 1 == nv) ? 0 : j + 1;
-        const V3<float> p0 = f3(s.X0[j]), p1 = f3(s.X0[j1]);
-        const V3<float> e = p1 - p0;
-        mid[j] = (strands && !(s.ET[j].w > 0.f)) ? make_float4(0.f, 0.f, 0.f, -1.f)
-                                                 : f4(0.5f * (p0 + p1), 0.5f * sqrtf(dot(e, e)));
-    }
     const int nblk = (ne + kBpBlock - 1) / kBpBlock;
-    for (int k = g.tid; k < nblk; k += TPR) {
-        // the vertices of edges k*B .. min(ne, (k+1)*B) - 1 (a loop's last edge ends at vertex 0)
-        const int v0 = k * kBpBlock, v1 = min(ne, v0 + kBpBlock);
-        V3<float> lo = f3(s.X0[v0]), hi = lo;
-        for (int v = v0 + 1; v <= v1; ++v) {
-            const V3<float> x = f3(s.X0[v == nv ? 0 : v]);
-            lo = f3(fminf(lo.x, x.x), fminf(lo.y, x.y), fminf(lo.z, x.z));
-            hi = f3(fmaxf(hi.x, x.x), fmaxf(hi.y, x.y), fmaxf(hi.z, x.z));
+    {   // thread j's edge; its block's box and sphere over the block's kBpBlock neighbouring lanes
+        static_assert(TPR >= NV && kBpBlock == 8, "one thread per edge, blocks of eight lanes");
+        const int j = g.tid;
+        const float inf = __int_as_float(0x7f800000);
+        V3<float> p0 = f3(inf, inf, inf), p1 = p0, lo = p0, hi = f3(-inf, -inf, -inf);
+        if (j < ne) {
+            p0 = f3(s.X0[j]);
+            p1 = f3(s.X0[j + 1 == nv ? 0 : j + 1]);
+            const V3<float> e = p1 - p0;
+            mid[j] = (strands && !(s.ET[j].w > 0.f)) ? make_float4(0.f, 0.f, 0.f, -1.f)
+                                                     : f4(0.5f * (p0 + p1), 0.5f * sqrtf(dot(e, e)));
+            lo = f3(fminf(p0.x, p1.x), fminf(p0.y, p1.y), fminf(p0.z, p1.z));
+            hi = f3(fmaxf(p0.x, p1.x), fmaxf(p0.y, p1.y), fmaxf(p0.z, p1.z));
         }
-        const V3<float> c = 0.5f * (lo + hi);
-        float r2 = 0.f;
-        for (int v = v0; v <= v1; ++v) {
-            const V3<float> d = f3(s.X0[v == nv ? 0 : v]) - c;
-            r2 = fmaxf(r2, dot(d, d));
+#pragma unroll
+        for (int o = 1; o < kBpBlock; o *= 2) {
+            auto other = [&](float v) { return __shfl_xor_sync(0xffffffffu, v, o); };
+            lo = f3(fminf(lo.x, other(lo.x)), fminf(lo.y, other(lo.y)), fminf(lo.z, other(lo.z)));
+            hi = f3(fmaxf(hi.x, other(hi.x)), fmaxf(hi.y, other(hi.y)), fmaxf(hi.z, other(hi.z)));
         }
-        blk[k] = f4(c, sqrtf(r2));
+        const V3<float> c = 0.5f * (lo + hi), d0 = p0 - c, d1 = p1 - c;
+        float r2 = j < ne ? fmaxf(dot(d0, d0), dot(d1, d1)) : 0.f;
+#pragma unroll
+        for (int o = 1; o < kBpBlock; o *= 2) r2 = fmaxf(r2, __shfl_xor_sync(0xffffffffu, r2, o));
+        if (j % kBpBlock == 0 && j < ne) blk[j / kBpBlock] = f4(c, sqrtf(r2));
     }
     if (g.tid == 0) {
         cnt[0] = 0;
         cnt[1] = 0;
+        cnt[2] = 0;
     }
     g.sync();
     const float cd = R.contact_d;
     // level 1: pairs of blocks
-    for (int q = g.tid; q < nblk * nblk; q += TPR) {
-        const int ka = q / nblk, kb = q - ka * nblk;
-        if (kb < ka) continue;
+    constexpr int NB = NV <= 32 ? 4 : NV <= 64 ? 8 : NV <= 128 ? 16 : 32;   // blocks, as a power of two
+    for (int q = g.tid; q < nblk * NB; q += TPR) {
+        const int ka = q / NB, kb = q % NB;
+        if (kb < ka || kb >= nblk) continue;
         const float4 A = blk[ka], B = blk[kb];
         const float dx = A.x - B.x, dy = A.y - B.y, dz = A.z - B.z;
         const float rr = (cd + A.w + B.w) * 1.0001f;
         if (dx * dx + dy * dy + dz * dz < rr * rr) nearb[atomicAdd(&cnt[1], 1)] = (uint32_t)ka | ((uint32_t)kb << 16);
     }
     g.sync();
-    // level 2: the edge pairs of the near block pairs
-    const int nn = cnt[1], cap = R.pair_cap;
+    // level 2: an edge of the first block of a near pair against the second block's eight, whose
+    // spheres are tested side by side.  Those that pass are listed and measured one per thread
+    // (level 3), beyond the list's room at once.
+    const int nn = cnt[1], cap = R.pair_cap, excl = R.excl;   // not read again after each store
     bool ovf = false;
-    constexpr int BB = kBpBlock * kBpBlock;
-    for (int t = g.tid; t < nn * BB; t += TPR) {
-        const uint32_t bp = nearb[t / BB];
-        const int a = (int)(bp & 0xffffu) * kBpBlock + (t % BB) / kBpBlock;
-        const int b = (int)(bp >> 16) * kBpBlock + t % kBpBlock;
-        if (b <= a || b >= ne) continue;
-        const float4 ma = mid[a], mb = mid[b];
-        if (!(ma.w >= 0.f && mb.w >= 0.f)) continue;
-        const float dx = ma.x - mb.x, dy = ma.y - mb.y, dz = ma.z - mb.z;
-        const float rr = (cd + ma.w + mb.w) * 1.00001f;
-        if (!(dx * dx + dy * dy + dz * dz < rr * rr)) continue;
+    auto measure = [&](uint32_t pr) {
+        const int a = (int)(pr & 0xffffu), b = (int)(pr >> 16);
         int sep = b - a;
         if (closed) sep = min(sep, ne - sep);
-        if (!(sep > R.excl || (strands && break_between(s.ET, a, b)))) continue;
+        if (!(sep > excl || (strands && break_between(s.ET, a, b)))) return;
         const int a1 = (a + 1 == nv) ? 0 : a + 1, b1 = (b + 1 == nv) ? 0 : b + 1;
         const V3<float> pa0 = f3(s.X0[a]), pa1 = f3(s.X0[a1]), pb0 = f3(s.X0[b]), pb1 = f3(s.X0[b1]);
         float su, uu;
         closest_params(pa0, pa1, pb0, pb1, su, uu);
         const V3<float> dd = (pa0 + su * (pa1 - pa0)) - (pb0 + uu * (pb1 - pb0));
-        if (!(sqrtf(dot(dd, dd)) < cd)) continue;
+        if (!(sqrtf(dot(dd, dd)) < cd)) return;
         const int idx = atomicAdd(&cnt[0], 1);
         if (idx < cap)
-            s.pairs[idx] = (uint32_t)a | ((uint32_t)b << 16);
+            s.pairs[idx] = pr;
         else
             ovf = true;
+    };
+    for (int t = g.tid; t < nn * kBpBlock; t += TPR) {
+        const uint32_t bp = nearb[t / kBpBlock];
+        const int a = (int)(bp & 0xffffu) * kBpBlock + t % kBpBlock, b0 = (int)(bp >> 16) * kBpBlock;
+        const float4 ma = mid[min(a, ne - 1)];
+        unsigned hits = 0;
+#pragma unroll
+        for (int m = 0; m < kBpBlock; ++m) {
+            const int b = b0 + m;
+            const float4 mb = mid[min(b, ne - 1)];
+            const float dx = ma.x - mb.x, dy = ma.y - mb.y, dz = ma.z - mb.z, rr = (cd + ma.w + mb.w) * 1.00001f;
+            int sep = b - a;
+            if (closed) sep = min(sep, ne - sep);
+            const bool near = b > a && b < ne && ma.w >= 0.f && mb.w >= 0.f && (sep > excl || strands) &&
+                              dx * dx + dy * dy + dz * dz < rr * rr;
+            hits |= near ? 1u << m : 0u;
+        }
+        if (hits) {
+            int at = atomicAdd(&cnt[2], __popc(hits));
+            for (; hits; hits &= hits - 1, ++at) {
+                const uint32_t pr = (uint32_t)a | (uint32_t)(b0 + __ffs(hits) - 1) << 16;
+                if (at < kList)
+                    list[at] = pr;
+                else
+                    measure(pr);
+            }
+        }
     }
+    g.sync();
+    // level 3
+    for (int t = g.tid; t < min(cnt[2], kList); t += TPR) measure(list[t]);
     g.sync();
     overflow = grp_any<TPR>(ovf, g);
     const int np = cnt[0];
