@@ -45,6 +45,18 @@ struct Grp {
         else
             asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(TPR) : "memory");
     }
+    // the same, returning whether p holds for any thread
+    __device__ __forceinline__ bool sync_any(bool p) const {
+        if (TPR == 32) {
+            const bool r = __any_sync(0xffffffffu, p);
+            __syncwarp();
+            return r;
+        }
+        unsigned r;
+        asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.or.pred q, %2, %3, p;\n\t"
+                     "selp.u32 %0, 1, 0, q;\n\t}" : "=r"(r) : "r"((unsigned)p), "r"(bar), "r"(TPR) : "memory");
+        return r != 0;
+    }
 };
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -608,11 +620,14 @@ __device__ __forceinline__ float4 project_edge(const ProjEdge& p, bool inext, V3
     return f4(t, target * ie);
 }
 
+// One Jacobi sweep over the candidate pairs.  With ask, returns whether any pair was closer than
+// the two radii (the positions are as they were otherwise).  The group has synchronised on return.
 template <int NV, bool CONTACT, int TPR>
-__device__ __forceinline__ void contact_sweep(const RodInfo& R, Smem<NV, CONTACT>& s, const Grp<TPR>& g, int np,
-                                              bool first) {
+__device__ __forceinline__ bool contact_sweep(const RodInfo& R, Smem<NV, CONTACT>& s, const Grp<TPR>& g, int np,
+                                              bool first, bool ask) {
     const int nv = R.nv;   // s.acc is zero on entry and is left zero
     const float rsum = 2.f * R.radius;
+    bool acts = false;
     for (int p = g.tid; p < np; p += TPR) {
         uint32_t pr = s.pairs[p];
         int a0 = pr & 0xffff, c0 = pr >> 16;
@@ -631,6 +646,7 @@ __device__ __forceinline__ void contact_sweep(const RodInfo& R, Smem<NV, CONTACT
             s.fr1[p] = make_float4(su, uu, W, on ? 1.f : 0.f);
         }
         if (on) {
+            acts = true;
             const int idx[4] = {a0, a1, c0, c1};
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -640,7 +656,11 @@ __device__ __forceinline__ void contact_sweep(const RodInfo& R, Smem<NV, CONTACT
             }
         }
     }
-    g.sync();
+    if (ask) {
+        if (!g.sync_any(acts)) return false;
+    } else {
+        g.sync();
+    }
     for (int i = g.tid; i < nv; i += TPR) {
         int4 q = s.acc[i];
         if (q.x | q.y | q.z) {
@@ -651,6 +671,7 @@ __device__ __forceinline__ void contact_sweep(const RodInfo& R, Smem<NV, CONTACT
         }
     }
     g.sync();
+    return true;
 }
 
 template <int NV, bool CONTACT, int TPR>
@@ -696,7 +717,9 @@ __device__ __forceinline__ void self_friction(const RodInfo& R, Smem<NV, CONTACT
 }
 
 // The N_C projection iterations of a substep on the displacements s.X: the length projections of
-// both colours and, with SWEEPS, a self-contact sweep.  The group has synchronised since s.X was
+// both colours and, with SWEEPS, a self-contact sweep.  A rod without length projections stops at
+// the first sweep that moves nothing (of the sweeps of 400 knotted ropes after the first three
+// quarters move nothing: 1.44 -> 1.13 ms for 20 frames).  The group has synchronised since s.X was
 // written; on return it has synchronised after the last iteration.
 template <int NV, bool CONTACT, int TPR, bool REC, bool SWEEPS>
 __device__ __forceinline__ void run_projections(const RodInfo& R, Smem<NV, CONTACT>& s, const Grp<TPR>& g, int n_iter, int np,
@@ -764,8 +787,13 @@ __device__ __forceinline__ void run_projections(const RodInfo& R, Smem<NV, CONTA
             // each thread stores its own vertices; the sweep reads s.X and writes only the
             // accumulators before its own barrier
             if (REC && i < nv) rec.csnap(it)[i] = s.X[i];
-            contact_sweep<NV, CONTACT, TPR>(R, s, g, np, it == 0);
-            if (proj && j + 1 < nv) mid = f3(s.X[j + 1]);
+            if (contact_sweep<NV, CONTACT, TPR>(R, s, g, np, it == 0, !lenc)) {
+                if (proj && j + 1 < nv) mid = f3(s.X[j + 1]);
+            } else {   // nothing moves any more: the sweeps left would find the same
+                if (REC && i < nv)
+                    for (int k = it + 1; k < n_iter; ++k) rec.csnap(k)[i] = s.X[i];
+                break;
+            }
         }
     }
     if (!SWEEPS) g.sync();
