@@ -947,10 +947,10 @@ __device__ __forceinline__ void substep_body(const SceneDev& sc, const float4* _
     const bool project = lenc || (CONTACT && np > 0);
     const float ih = 1.f / h;
     // new position (the absolute target for a held vertex) and velocity from the displacement d
-    auto finish = [&](float4 x0, V3<float> d, float om) {
+    const bool held = own.kind >= 2 && in_bounds(own.kind - 2 < R.ngrip, s.red);
+    auto finish = [&](float4 x0, V3<float> d, float om, V3<float> target) {
         float4 x = make_float4(x0.x + d.x, x0.y + d.y, x0.z + d.z, x0.w);
-        if (own.kind >= 2 && in_bounds(own.kind - 2 < R.ngrip, s.red))
-            x = f4(grasp_target(sp, own.kind, KIN[R.v0 + i]), x0.w);
+        if (held) x = f4(target, x0.w);
         if (mv) {
             const float dx = x.x - x0.x, dy = x.y - x0.y, dz = x.z - x0.z;
             *mv += sqrtf(dx * dx + dy * dy + dz * dz);
@@ -975,7 +975,7 @@ __device__ __forceinline__ void substep_body(const SceneDev& sc, const float4* _
         const float4 vi = s.V[i];
         // displacement d of this substep (positions are only formed at its end, so the rebuilt
         // velocity d/h carries no cancellation error from |x| >> |h v|)
-        V3<float> d = zf3();
+        V3<float> d = zf3(), target = zf3();
         if (own.kind == 0) {
             V3<float> grav = f3(0.f, 0.f, -sc.gravity);
             V3<float> acc = (-xi4.w) * gr + grav - R.cd * f3(vi);
@@ -983,8 +983,9 @@ __device__ __forceinline__ void substep_body(const SceneDev& sc, const float4* _
             if (REC) rec.v1()[i] = f4(v1, 0.f);
             const V3<float> v2 = rigid_contact(sc, R, xi, v1, sp, imp ? imp + 4 * i : nullptr, 1.f / xi4.w);
             d = h * v2;
-        } else if (own.kind >= 2 && in_bounds(own.kind - 2 < R.ngrip, s.red)) {
-            d = grasp_target(sp, own.kind, KIN[R.v0 + i]) - xi;   // a held vertex sits at its target
+        } else if (held) {   // a held vertex sits at its target
+            target = grasp_target(sp, own.kind, KIN[R.v0 + i]);
+            d = target - xi;
         }
         float om1 = vi.w;
         if (has_e) {
@@ -1002,7 +1003,7 @@ __device__ __forceinline__ void substep_body(const SceneDev& sc, const float4* _
             s.V[i].w = om1;
         } else {
             if (REC) rec.dfin()[i] = f4(d, xi4.w);
-            finish(xi4, d, om1);
+            finish(xi4, d, om1, target);
         }
     }
     g.sync();
@@ -1016,7 +1017,7 @@ __device__ __forceinline__ void substep_body(const SceneDev& sc, const float4* _
     if (vtx) {
         const float4 d = s.X[i];
         if (REC) rec.dfin()[i] = d;
-        finish(s.X0[i], f3(d), s.V[i].w);
+        finish(s.X0[i], f3(d), s.V[i].w, held ? grasp_target(sp, own.kind, KIN[R.v0 + i]) : zf3());
     }
     if (CONTACT && REC)
         for (int p = g.tid; p < np; p += TPR) {
