@@ -454,7 +454,7 @@ extern "C" dlo_status dlo_backward(dlo_ctx* c, const float* dL_dx_T, const float
         cudaError_t fe = fork_classes(c);
         if (fe != cudaSuccess) return cuda_err(c, fe, "fork");
     }
-    for (size_t k = 0; k < c->buckets.size(); ++k) {
+    for (size_t k = c->buckets.size(); k-- > 0;) {   // the longest rods first, as in the forward
         const int n = c->buckets[k].n;
         float4* R3 = reinterpret_cast<float4*>(stored ? reinterpret_cast<char*>(c->sub_mem) + plan.sub_off[k]
                                                       : region + plan.offset[k]);

