@@ -213,9 +213,7 @@ __device__ __forceinline__ void material_frame(EdgeF<dualf>& E) {
     opaque(E.d1r.z);
     opaque(E.c);
     opaque(E.s);
-    E.d2r = cross(E.t, E.d1r);
-    E.d1 = E.c * E.d1r + E.s * E.d2r;
-    E.d2 = E.c * E.d2r - E.s * E.d1r;
+    material_directors(E);
 }
 
 // Reverse of an active gripper contact: the cotangents of the vertex position (to add) and of

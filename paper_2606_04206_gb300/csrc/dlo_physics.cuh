@@ -61,12 +61,57 @@ DLO_HD float edge_strain(V3<float> e, float eb) {
 #endif
 }
 
+// a x b with the roundings of its values fixed: each component one rounded product and one fused
+// multiply-add.  A hinge on its yield surface branches on the last bits of its curvature, and the
+// compiler may fuse either product, differently in the forward and in the backward's
+// recomputation, unless it is told which.
+DLO_HD float cross_comp(float p, float q, float r, float s) {   // p q - r s
+#ifdef __CUDA_ARCH__
+    return __fmaf_rn(p, q, -__fmul_rn(r, s));
+#else
+    return p * q - r * s;
+#endif
+}
+template <class T>
+DLO_HD V3<T> cross_fixed(V3<T> a, V3<T> b) { return cross(a, b); }   // scalars without roundings to fix
+DLO_HD V3<float> cross_fixed(V3<float> a, V3<float> b) {
+    return {cross_comp(a.y, b.z, a.z, b.y), cross_comp(a.z, b.x, a.x, b.z), cross_comp(a.x, b.y, a.y, b.x)};
+}
+DLO_HD V3<dualf> cross_fixed(V3<dualf> a, V3<dualf> b) { return lift(cross_fixed(vals(a), vals(b)), ders(cross(a, b))); }
+// The same for a . b (x and y first) and for p a + q b (the first product fused).
+template <class T>
+DLO_HD T dot_fixed(V3<T> a, V3<T> b) { return dot(a, b); }
+DLO_HD float dot_fixed(V3<float> a, V3<float> b) {
+#ifdef __CUDA_ARCH__
+    return __fmaf_rn(a.z, b.z, __fmaf_rn(a.x, b.x, __fmul_rn(a.y, b.y)));
+#else
+    return dot(a, b);
+#endif
+}
+DLO_HD dualf dot_fixed(V3<dualf> a, V3<dualf> b) { return mkd(dot_fixed(vals(a), vals(b)), dot(a, b).d); }
+template <class T>
+DLO_HD V3<T> comb_fixed(T p, V3<T> a, T q, V3<T> b) { return p * a + q * b; }
+DLO_HD V3<float> comb_fixed(float p, V3<float> a, float q, V3<float> b) {
+    return {cross_comp(p, a.x, -q, b.x), cross_comp(p, a.y, -q, b.y), cross_comp(p, a.z, -q, b.z)};
+}
+DLO_HD V3<dualf> comb_fixed(dualf p, V3<dualf> a, dualf q, V3<dualf> b) {
+    return lift(comb_fixed(p.v, vals(a), q.v, vals(b)), ders(p * a + q * b));
+}
+
 // ------------------------------------------------------------------ edge frames
 template <class T>
 struct EdgeF {
     V3<T> t, w0, d1r, d2r, d1, d2;
     T ell, n1, c, s;
 };
+
+// d2r and the material directors from t, d1r and the twist angle's cosine and sine
+template <class T>
+DLO_HD void material_directors(EdgeF<T>& E) {
+    E.d2r = cross_fixed(E.t, E.d1r);
+    E.d1 = comb_fixed(E.c, E.d1r, E.s, E.d2r);
+    E.d2 = comb_fixed(E.c, E.d2r, -E.s, E.d1r);
+}
 
 template <class T>
 DLO_HD void edge_forward(EdgeF<T>& E, V3<T> xa, V3<T> xb, V3<T> tb, V3<T> d1b, T th) {
@@ -77,11 +122,9 @@ DLO_HD void edge_forward(EdgeF<T>& E, V3<T> xa, V3<T> xb, V3<T> tb, V3<T> d1b, T
     V3<T> w1 = E.w0 - dot(E.w0, E.t) * E.t;
     E.n1 = norm(w1);
     E.d1r = w1 / E.n1;
-    E.d2r = cross(E.t, E.d1r);
     E.c = dcos(th);
     E.s = dsin(th);
-    E.d1 = E.c * E.d1r + E.s * E.d2r;
-    E.d2 = E.c * E.d2r - E.s * E.d1r;
+    material_directors(E);
 }
 
 // Reverse of edge_forward: given adjoints of t and d1r (and of |e|), the adjoint of the edge
@@ -117,32 +160,14 @@ struct HingeF {
     T cc, y, xq, mref, m, k0, k1;
 };
 
-// a x b with the roundings of its values fixed: each component one rounded product and one fused
-// multiply-add.  A hinge on its yield surface branches on the last bits of its curvature, and the
-// compiler may fuse either product, differently in the forward and in the backward's
-// recomputation, unless it is told which.
-DLO_HD float cross_comp(float p, float q, float r, float s) {   // p q - r s
-#ifdef __CUDA_ARCH__
-    return __fmaf_rn(p, q, -__fmul_rn(r, s));
-#else
-    return p * q - r * s;
-#endif
-}
-template <class T>
-DLO_HD V3<T> cross_fixed(V3<T> a, V3<T> b) { return cross(a, b); }   // scalars without roundings to fix
-DLO_HD V3<float> cross_fixed(V3<float> a, V3<float> b) {
-    return {cross_comp(a.y, b.z, a.z, b.y), cross_comp(a.z, b.x, a.x, b.z), cross_comp(a.x, b.y, a.y, b.x)};
-}
-DLO_HD V3<dualf> cross_fixed(V3<dualf> a, V3<dualf> b) { return lift(cross_fixed(vals(a), vals(b)), ders(cross(a, b))); }
-
 // The hinge's own part, from its two edges' frames (H.a, H.b: t, d1r, d2r, d1, d2 set).
 template <class T>
 DLO_HD void hinge_bend_forward(HingeF<T>& H) {
-    H.cc = 1.f + dot(H.a.t, H.b.t);
+    H.cc = 1.f + dot_fixed(H.a.t, H.b.t);
     H.X = cross_fixed(H.a.t, H.b.t);
     H.kb = (2.f / H.cc) * H.X;
-    H.k0 = 0.5f * dot(H.kb, H.a.d2 + H.b.d2);
-    H.k1 = 0.5f * dot(H.kb, H.a.d1 + H.b.d1);
+    H.k0 = 0.5f * dot_fixed(H.kb, H.a.d2 + H.b.d2);
+    H.k1 = 0.5f * dot_fixed(H.kb, H.a.d1 + H.b.d1);
 }
 // reference twist: angle about t^b from the space-transported d1r^a to d1r^b
 template <class T>

@@ -827,9 +827,7 @@ __device__ __forceinline__ void load_frame(EdgeF<float>& E, float4 ta, float4 rc
     E.d1r = f3(rc);
     E.c = rc.w;
     E.s = sn;
-    E.d2r = cross(E.t, E.d1r);
-    E.d1 = E.c * E.d1r + E.s * E.d2r;
-    E.d2 = E.c * E.d2r - E.s * E.d1r;
+    material_directors(E);
 }
 
 // ------------------------------------------------------------------ one substep

@@ -75,3 +75,25 @@ def test_a_captured_step_stores_no_records():
         stream.synchronize()
     for k in ref:
         assert torch.equal(got[k], ref[k]), k
+
+
+@pytest.mark.parametrize("n", [128, 192, 224, 256])
+def test_recording_changes_neither_state_nor_gradient(n):
+    """Yielding wires of each size class: a hinge on its yield surface branches on the last bit of
+    its curvature, so the three kernels that step a rod have to round alike."""
+    p = inputs.batching(60, 1, 5, vmin=n - 31, vmax=n)
+    p.E[:], p.K[:], p.G[:] = (inputs.f32(np.full(60, v)) for v in (1e5, 1e5, 4e4))
+    sim = sim_for(p)
+    states = []
+    for record in (False, True):
+        sim.reset()
+        if record:
+            sim.begin_rollout(1)
+        sim.step(actions_dev(p), 1)
+        states.append(sim.full_state_numpy())
+    for k in states[0]:
+        assert np.array_equal(states[0][k], states[1][k]), k
+    ref, _ = gradients(p, 1, hbm_budget=1 << 20)
+    got, _ = gradients(p, 1)
+    for k in ref:
+        assert torch.equal(got[k], ref[k]), k
