@@ -325,7 +325,7 @@ extern "C" dlo_status dlo_begin_rollout(dlo_ctx* c, int n_frames) {
     // them as it steps and the backward does not step again to get them.  Without the memory, or
     // beside a workspace that an earlier, longer rollout's backward left, the backward
     // recomputes them.  4096 rods x 128 vertices, 16 frames (19 GB of records), forward and
-    // backward: 18.0 ms recomputed, 14.5 ms stored; one rod x 128: 1.42 ms and 1.13 ms.
+    // backward: 14.0 ms recomputed, 10.9 ms stored; one rod x 128, 10 frames: 1.54 and 1.07 ms.
     BwdPlan& plan = c->rec_plan;
     const size_t used = c->ck_bytes + c->rec_bytes;
     bool fits = bwd_plan(c, 0, K, plan, c->rec_budget, n_frames) == DLO_OK && plan.C[0] >= n_frames &&
