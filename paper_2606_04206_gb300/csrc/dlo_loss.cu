@@ -139,6 +139,11 @@ __global__ void loss_winding(const RodInfo* rods, const float4* X, const float4*
 // with e1 and e2 the segments: formed from the segments it keeps the digits that the products of
 // the nearly equal r's of a distant pair cancel.  Their denominators are
 // |u||v||w| + (u.v)|w| + (u.w)|v| + (v.w)|u|.
+// Two vertices much closer to each other than the segments are long turn this round: the product of
+// the segments is then off by 1e-7 |e1||e2||r13|, the denominators of the triangles that hold the
+// short r shrink with it, and at zero the angle is atan2(rounding, 0).  With an r below a quarter of
+// the rod's longest edge each triangle takes the product of its own three vectors, which vanishes with
+// its shortest, and the lengths are square roots (zero at zero, where s rsqrt(s) is not a number).
 
 // The gradient of a denominator, times c, added to those of its three vectors (lengths l, inverse
 // lengths il, dot products d).
@@ -153,9 +158,10 @@ __device__ __forceinline__ void denominator_grad(V3<float> u, V3<float> v, V3<fl
 }
 
 // Omega of the segments p1p2 and p3p4; with GRAD also its gradient with respect to the four ends
-// (one reverse pass).
+// (one reverse pass).  near2: the squared distance below which two vertices count as close.
 template <bool GRAD>
-__device__ __forceinline__ float gauss_pair(V3<float> p1, V3<float> p2, V3<float> p3, V3<float> p4, V3<float>* g) {
+__device__ __forceinline__ float gauss_pair(V3<float> p1, V3<float> p2, V3<float> p3, V3<float> p4, float near2,
+                                            V3<float>* g) {
     const V3<float> r13 = p3 - p1, r14 = p4 - p1, r23 = p3 - p2, r24 = p4 - p2, e1 = p2 - p1, e2 = p4 - p3;
     float l13, l14, l23, l24, i13, i14, i23, i24;
     len_inv(r13, l13, i13);
@@ -163,15 +169,28 @@ __device__ __forceinline__ float gauss_pair(V3<float> p1, V3<float> p2, V3<float
     len_inv(r23, l23, i23);
     len_inv(r24, l24, i24);
     const V3<float> e12 = cross(e1, e2);
-    const float n = dot(r13, e12);
+    float n1 = dot(r13, e12), n2 = n1;
+    const float s13 = dot(r13, r13), s14 = dot(r14, r14), s23 = dot(r23, r23), s24 = dot(r24, r24);
+    if (fminf(fminf(s13, s14), fminf(s23, s24)) <= near2) {
+        n1 = dot(r13, cross(r14, r24));
+        n2 = dot(r13, cross(r24, r23));
+        auto root = [](float s, float& l, float& i) {
+            l = sqrtf(s);
+            i = l > 0.f ? 1.f / l : 0.f;
+        };
+        root(s13, l13, i13);
+        root(s14, l14, i14);
+        root(s23, l23, i23);
+        root(s24, l24, i24);
+    }
     const float da = dot(r13, r14), db = dot(r13, r24), dc = dot(r14, r24), dd = dot(r13, r23), de = dot(r24, r23);
     const float m1 = l13 * l14 * l24 + da * l24 + db * l14 + dc * l13;
     const float m2 = l13 * l24 * l23 + db * l23 + dd * l24 + de * l13;
     if (GRAD) {
-        const float q1 = -2.f / (n * n + m1 * m1), q2 = -2.f / (n * n + m2 * m2);
+        const float q1 = -2.f / (n1 * n1 + m1 * m1), q2 = -2.f / (n2 * n2 + m2 * m2);
         V3<float> g13 = zf3(), g14 = zf3(), g23 = zf3(), g24 = zf3();
-        denominator_grad(r13, r14, r24, l13, l14, l24, i13, i14, i24, da, db, dc, -(q1 * n), g13, g14, g24);
-        denominator_grad(r13, r24, r23, l13, l24, l23, i13, i24, i23, db, dd, de, -(q2 * n), g13, g24, g23);
+        denominator_grad(r13, r14, r24, l13, l14, l24, i13, i14, i24, da, db, dc, -(q1 * n1), g13, g14, g24);
+        denominator_grad(r13, r24, r23, l13, l24, l23, i13, i24, i23, db, dd, de, -(q2 * n2), g13, g24, g23);
         const float c = q1 * m1 + q2 * m2;   // of the triple product
         g13 += c * e12;
         const V3<float> h1 = c * cross(e2, r13), h2 = c * cross(r13, e1);
@@ -180,7 +199,7 @@ __device__ __forceinline__ float gauss_pair(V3<float> p1, V3<float> p2, V3<float
         g[2] = g13 + g23 - h2;
         g[3] = g14 + g24 + h2;
     }
-    return -2.f * (atan2f(n, m1) + atan2f(n, m2));
+    return -2.f * (atan2f(n1, m1) + atan2f(n2, m2));
 }
 
 // Sum of floats as an unevaluated pair (Knuth's exact two-term sum): FP64 accuracy on the FP32
@@ -207,6 +226,7 @@ __global__ void __launch_bounds__(kLT) loss_crossing(const RodInfo* rods, const 
     __shared__ double sh[kLT];
     __shared__ float4 xs[kMaxV];
     __shared__ float4 ge0[GRAD ? kLT : 1], ge1[GRAD ? kLT : 1];   // d/d(first, second endpoint) of each edge's sum
+    __shared__ unsigned longest;   // the longest edge squared (non-negative floats order like their bits)
     const int rod = blockIdx.x;
     const RodInfo R = rods[rod];
     const bool closed = R.flags & ROD_CLOSED;
@@ -215,7 +235,17 @@ __global__ void __launch_bounds__(kLT) loss_crossing(const RodInfo* rods, const 
         xs[i] = X[R.v0 + i];
         if (GRAD) ge0[i] = ge1[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
+    if (threadIdx.x == 0) longest = 0u;
     __syncthreads();
+    unsigned far = 0u;
+    for (int j = threadIdx.x; j < ne; j += kLT) {
+        const V3<float> e = f3(xs[j + 1 == n ? 0 : j + 1]) - f3(xs[j]);
+        far = max(far, __float_as_uint(dot(e, e)));
+    }
+    far = __reduce_max_sync(0xffffffffu, far);
+    if (threadIdx.x % 32 == 0) atomicMax(&longest, far);
+    __syncthreads();
+    const float near2 = 0.0625f * __uint_as_float(longest);
     PairSum sum;
     V3<float> g0[EPT], g1[EPT];
 #pragma unroll
@@ -230,7 +260,8 @@ __global__ void __launch_bounds__(kLT) loss_crossing(const RodInfo* rods, const 
             const int b = a + k >= ne ? a + k - ne : a + k;
             if (abs(a - b) <= 1 || (closed && k == 1)) continue;
             V3<float> gp[4];
-            sum.add(gauss_pair<GRAD>(f3(xs[a]), f3(xs[a + 1 == n ? 0 : a + 1]), f3(xs[b]), f3(xs[b + 1 == n ? 0 : b + 1]), gp));
+            sum.add(gauss_pair<GRAD>(f3(xs[a]), f3(xs[a + 1 == n ? 0 : a + 1]), f3(xs[b]), f3(xs[b + 1 == n ? 0 : b + 1]),
+                                         near2, gp));
             if (GRAD) {
                 g0[m] += gp[0];
                 g1[m] += gp[1];
