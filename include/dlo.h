@@ -178,11 +178,13 @@ dlo_status dlo_get_internal(dlo_ctx* ctx, float* ref, float* tan, float* hinge, 
  * opt.checkpoint_every, or when that is 0 the shortest interval whose ring, action record
  * and backward workspace fit opt.hbm_budget (80 GiB by default).  It also sets how many
  * frames the backward reverses per launch pair: its chunk records may take half of what the
- * ring and the action record leave of the budget (at most 24 GiB).  When the records of the
- * whole rollout fit that share (and 64 frames), dlo_step stores them while it steps, in memory
- * allocated here, and dlo_backward does not step again; when they do not fit, when that
- * memory cannot be allocated, or when a step is captured in a graph, dlo_backward recomputes
- * them from the checkpoints.  The gradients are the same.
+ * ring and the action record leave of the budget (at most 24 GiB).  When an
+ * earlier dlo_backward of this context left a workspace with room for the records of the whole
+ * rollout (at most 64 frames), dlo_step stores them there while it steps, and dlo_backward does
+ * not step again.  Otherwise (the first rollout, one longer than those before, a step captured
+ * in a graph, or a last backward that was dlo_backward_noalloc or dlo_backward_plain)
+ * dlo_backward recomputes them from the checkpoints.  The gradients are the same.  The call
+ * allocates the ring and the action record, nothing else.
  * Defined by: the gradient checkpointing of Sec. 3.3 (checkpoints kept in HBM here).
  * Errors: DLO_ERR_INVALID_ARG for n_frames <= 0; DLO_ERR_OOM when the ring cannot be
  * allocated. */

@@ -274,8 +274,6 @@ dlo_status bwd_plan(dlo_ctx* c, int force, int K, BwdPlan& out, size_t rec_budge
     out.l2_rod.assign(nb_, 0);
     out.cs_rod.assign(nb_, 0);
     out.offset.assign(nb_, 0);
-    out.sub_off.assign(nb_, 0);
-    out.rest_off.assign(nb_, 0);
     size_t per_frame = 0;
     for (size_t k = 0; k < nb_; ++k) {
         const Bucket& bk = c->buckets[k];
@@ -291,8 +289,7 @@ dlo_status bwd_plan(dlo_ctx* c, int force, int K, BwdPlan& out, size_t rec_budge
     int C = (int)std::max<size_t>(1, std::min<size_t>(64, rec_budget / std::max<size_t>(per_frame, 1)));
     if (frames > 0) C = std::min(C, (frames + K - 1) / K * K);
     if (C >= K) C = (C / K) * K;   // chunks start at checkpoints
-    size_t need = 0, sub = 0, rest = 0;
-    auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
+    size_t need = 0;
     for (size_t k = 0; k < nb_; ++k) {
         const Bucket& bk = c->buckets[k];
         const int NV = bk.nv_max;
@@ -301,23 +298,17 @@ dlo_status bwd_plan(dlo_ctx* c, int force, int K, BwdPlan& out, size_t rec_budge
         out.l2_rod[k] = C < K ? (size_t)K * (5 * (size_t)NV + 6) : 0;
         out.cs_rod[k] = 5 * (size_t)NV + 6;
         out.offset[k] = need;   // each class has its own region: the classes run concurrently
-        need += up(16 * (size_t)bk.n * (out.r3_rod[k] + out.l2_rod[k] + out.cs_rod[k]));
-        out.sub_off[k] = sub;
-        out.rest_off[k] = rest;
-        sub += up(16 * (size_t)bk.n * out.r3_rod[k]);
-        rest += up(16 * (size_t)bk.n * (out.l2_rod[k] + out.cs_rod[k]));
+        need += (16 * (size_t)bk.n * (out.r3_rod[k] + out.l2_rod[k] + out.cs_rod[k]) + 255) & ~(size_t)255;
     }
     out.fixed = (2 * 16 * (size_t)c->Et + 255) & ~(size_t)255;
     out.bytes = out.fixed + need;
-    out.sub_bytes = sub;
-    out.rest_bytes = out.fixed + rest;
     return DLO_OK;
 }
 
 bool records_fit(const dlo_ctx* c, const BwdPlan& plan) {
     for (int C : plan.C)
         if (C < c->rec_frames) return false;
-    return plan.sub_bytes <= c->sub_bytes;
+    return plan.bytes <= c->bw_bytes;
 }
 
 dlo_status enqueue_backward_class(dlo_ctx* c, const BwdPlan& plan, size_t k, cudaStream_t st, int item0, int n,
@@ -437,11 +428,11 @@ extern "C" dlo_status dlo_backward(dlo_ctx* c, const float* dL_dx_T, const float
     dlo_status pst = bwd_plan(c, force, c->ck_every, plan, c->rec_budget, c->rec_frames);
     if (pst != DLO_OK) return pst;
     const bool stored = c->rec_stored && records_fit(c, plan);
-    const size_t bytes = stored ? plan.rest_bytes : plan.bytes;
-    if (bytes > c->bw_bytes) {
+    c->rec_wanted = true;
+    if (plan.bytes > c->bw_bytes) {
         dev_free(c, c->bw_mem);
-        c->bw_mem = dev_alloc(c, bytes);
-        c->bw_bytes = c->bw_mem ? bytes : 0;
+        c->bw_mem = dev_alloc(c, plan.bytes);
+        c->bw_bytes = c->bw_mem ? plan.bytes : 0;
         if (!c->bw_mem) return set_err(c, DLO_ERR_OOM, "backward workspace allocation failed");
     }
     char* p = reinterpret_cast<char*>(c->bw_mem);
@@ -456,9 +447,8 @@ extern "C" dlo_status dlo_backward(dlo_ctx* c, const float* dL_dx_T, const float
     }
     for (size_t k = c->buckets.size(); k-- > 0;) {   // the longest rods first, as in the forward
         const int n = c->buckets[k].n;
-        float4* R3 = reinterpret_cast<float4*>(stored ? reinterpret_cast<char*>(c->sub_mem) + plan.sub_off[k]
-                                                      : region + plan.offset[k]);
-        float4* L2 = stored ? reinterpret_cast<float4*>(region + plan.rest_off[k]) : R3 + (size_t)n * plan.r3_rod[k];
+        float4* R3 = reinterpret_cast<float4*>(region + plan.offset[k]);
+        float4* L2 = R3 + (size_t)n * plan.r3_rod[k];
         float4* CS = L2 + (size_t)n * plan.l2_rod[k];
         dlo_status st = enqueue_backward_class(c, plan, k, class_stream(c, k), 0, n, R3, L2, CS, plan.C[k], common,
                                                stored);

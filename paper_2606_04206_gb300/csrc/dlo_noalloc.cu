@@ -81,6 +81,7 @@ extern "C" dlo_status dlo_backward_noalloc(dlo_ctx* c, const float* dL_dx_T, con
     char* base = nullptr;
     dlo_status st = scratch_address(c, &base);
     if (st != DLO_OK) return st;
+    c->rec_wanted = false;   // the records a step may have stored are not read here
 
     // fixed part: cotangents of the initial reference frames (gtb0, gd1b0) and, when the
     // gradient must reach x0 through the frame initialisation, the 96 bytes per vertex that

@@ -1238,6 +1238,7 @@ extern "C" dlo_status dlo_backward_plain(dlo_ctx* c, const float* dL_dx_T, const
     const size_t f4 = 3 * nV + 2 * nE + rec_f4 + 7 * nV + 3 * nE;
     const size_t bytes = 16 * f4 + sizeof(double) * 5 * B + sizeof(float) * (size_t)B * (12 + 12 + 36 + 72 + 24 + 24) +
                          2 * 16 * nE + 4096;
+    c->rec_wanted = c->rec_stored = false;   // this takes over the workspace the records are in
     if (bytes > c->bw_bytes) {
         dev_free(c, c->bw_mem);
         c->bw_mem = dev_alloc(c, bytes);

@@ -321,26 +321,7 @@ extern "C" dlo_status dlo_begin_rollout(dlo_ctx* c, int n_frames) {
     c->rec_frames = n_frames;
     c->rec_done = 0;
     c->rec_active = true;
-    // When the substep records of the whole rollout fit the backward's budget, the forward stores
-    // them as it steps and the backward does not step again to get them.  Without the memory, or
-    // beside a workspace that an earlier, longer rollout's backward left, the backward
-    // recomputes them.  4096 rods x 128 vertices, 16 frames (19 GB of records), forward and
-    // backward: 14.0 ms recomputed, 10.9 ms stored; one rod x 128, 10 frames: 1.54 and 1.07 ms.
-    BwdPlan& plan = c->rec_plan;
-    const size_t used = c->ck_bytes + c->rec_bytes;
-    bool fits = bwd_plan(c, 0, K, plan, c->rec_budget, n_frames) == DLO_OK && plan.C[0] >= n_frames &&
-                used + plan.sub_bytes + std::max(plan.rest_bytes, c->bw_bytes) <= budget;
-    if (fits && plan.sub_bytes > c->sub_bytes) {
-        dev_free(c, c->sub_mem);
-        c->sub_mem = dev_alloc(c, plan.sub_bytes);
-        c->sub_bytes = c->sub_mem ? plan.sub_bytes : 0;
-        fits = c->sub_mem != nullptr;
-    } else if (!fits && c->sub_mem && used + plan.bytes + c->sub_bytes > budget) {
-        dev_free(c, c->sub_mem);   // the backward's own workspace needs the room
-        c->sub_mem = nullptr;
-        c->sub_bytes = 0;
-    }
-    c->rec_stored = fits;
+    c->rec_stored = c->rec_wanted;   // if they fit: the first step, which knows the substeps, finds out
     c->rec_from_set = c->from_set_state;
     c->rec_nsub = -1;
     return DLO_OK;
@@ -350,15 +331,21 @@ extern "C" dlo_status dlo_begin_rollout(dlo_ctx* c, int n_frames) {
 dlo_status launch_step(dlo_ctx* c, const float* actions, int frames, int substeps, float* x_frames, int frame0,
                        bool record) {
     if (record && c->rec_stored) {
-        // A captured step stores no records: a graph may outlive the buffer, which a later
-        // dlo_begin_rollout may exchange.
+        // A captured step stores no records: a graph may outlive the workspace, which a later
+        // backward may exchange.
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         const cudaError_t e = cudaStreamIsCapturing(c->stream, &cap);
         if (e != cudaSuccess) return cuda_err(c, e, "capture status");
         if (cap != cudaStreamCaptureStatusNone) c->rec_stored = false;
     }
-    if (record && c->rec_stored && c->rec_done == 0 && substeps > 0)
-        // forced substeps change the records' size: they may not fit
+    // When the workspace of an earlier dlo_backward has room for the substep records of the whole
+    // rollout, the forward stores them there as it steps and the backward does not step again to
+    // get them.  Nothing is allocated for it: the first dlo_backward of a context recomputes, and
+    // a caller of dlo_backward_noalloc or dlo_backward_plain, which read no such records, neither
+    // holds memory for them nor writes them.  4096 rods x 128 vertices, 16 frames (19 GB of
+    // records), forward and backward: 14.0 ms recomputed, 10.9 ms stored; one rod x 128, 10 frames:
+    // 1.54 and 1.07 ms.
+    if (record && c->rec_stored && c->rec_done == 0)
         c->rec_stored = bwd_plan(c, substeps, c->ck_every, c->rec_plan, c->rec_budget, c->rec_frames) == DLO_OK &&
                         records_fit(c, c->rec_plan);
     cudaError_t fe = cudaMemsetAsync(c->d_counters, 0, sizeof(int) * c->buckets.size(), c->stream);
@@ -392,7 +379,7 @@ dlo_status launch_step(dlo_ctx* c, const float* actions, int frames, int substep
             P.ck_count = c->ck_count;
             if (c->rec_stored) {
                 const BwdPlan& plan = c->rec_plan;
-                P.R3 = reinterpret_cast<float4*>(reinterpret_cast<char*>(c->sub_mem) + plan.sub_off[k]);
+                P.R3 = reinterpret_cast<float4*>(reinterpret_cast<char*>(c->bw_mem) + plan.fixed + plan.offset[k]);
                 P.r3_rod = plan.r3_rod[k];
                 P.nsub_max = plan.nsmax[k];
             }

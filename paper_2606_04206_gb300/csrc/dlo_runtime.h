@@ -31,10 +31,6 @@ struct BwdPlan {
     std::vector<size_t> r3_rod, l2_rod, cs_rod, offset;
     size_t fixed = 0;    // initial-frame cotangents
     size_t bytes = 0;    // everything, for all rods at once
-    // the same with the chunk records apart (in memory the forward fills): each class's offset
-    // there and their total, and each class's offset and the total of the rest
-    std::vector<size_t> sub_off, rest_off;
-    size_t sub_bytes = 0, rest_bytes = 0;
 };
 struct dlo_ctx {
     int B = 0;
@@ -80,11 +76,11 @@ struct dlo_ctx {
     int rec_frames = 0, rec_done = 0, rec_nsub = 0;
     int ck_every = 0, ck_count = 0;
     size_t rec_budget = 0;   // chunk-record bytes the backward may use (set by dlo_begin_rollout)
-    // substep records of the whole rollout, stored by the forward when they fit the budget
-    bool rec_stored = false;
-    BwdPlan rec_plan;        // the plan they were laid out with
-    void* sub_mem = nullptr;
-    size_t sub_bytes = 0;
+    // substep records of the whole rollout, stored by the forward in the workspace that an earlier
+    // dlo_backward left (bw_mem), while dlo_backward is the backward the caller uses
+    bool rec_wanted = false;   // the last backward was dlo_backward, which reads them
+    bool rec_stored = false;   // this rollout's are being stored
+    BwdPlan rec_plan;          // the plan they are laid out with
     dlo::StateRef ck{};
     void* ck_mem = nullptr;
     size_t ck_bytes = 0;
@@ -110,7 +106,7 @@ void backward_shapes(dlo_ctx* c);
 // rec_budget: bytes allowed for the chunk records of all classes (0 = the default); frames: the
 // rollout's (0 = not known: chunks are not cut to it)
 dlo_status bwd_plan(dlo_ctx* c, int force, int K, BwdPlan& out, size_t rec_budget = 0, int frames = 0);
-// Whether the plan's chunks hold the whole rollout and the memory for its records is there.
+// Whether the plan's chunks hold the whole rollout and the present workspace has room for them.
 bool records_fit(const dlo_ctx* c, const BwdPlan& plan);
 // Enqueue the backward of size class k for the rods order[item0 .. item0 + n) on stream st,
 // with that class's R3 / L2 / CS buffers sized for n rods; common holds the outputs and inputs.
