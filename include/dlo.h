@@ -181,8 +181,9 @@ dlo_status dlo_get_internal(dlo_ctx* ctx, float* ref, float* tan, float* hinge, 
  * ring and the action record leave of the budget (at most 24 GiB).  When an
  * earlier dlo_backward of this context left a workspace with room for the records of the whole
  * rollout (at most 64 frames), dlo_step stores them there while it steps, and dlo_backward does
- * not step again.  Otherwise (the first rollout, one longer than those before, a step captured
- * in a graph, or a last backward that was dlo_backward_noalloc or dlo_backward_plain)
+ * not step again.  Otherwise (the first rollout, one longer than those before, a last backward
+ * that was dlo_backward_noalloc or dlo_backward_plain, or any rollout once a recorded step of
+ * this context has been captured in a graph, whose replays write the checkpoints unseen)
  * dlo_backward recomputes them from the checkpoints.  The gradients are the same.  The call
  * allocates the ring and the action record, nothing else.
  * Defined by: the gradient checkpointing of Sec. 3.3 (checkpoints kept in HBM here).

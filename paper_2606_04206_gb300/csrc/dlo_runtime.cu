@@ -321,23 +321,28 @@ extern "C" dlo_status dlo_begin_rollout(dlo_ctx* c, int n_frames) {
     c->rec_frames = n_frames;
     c->rec_done = 0;
     c->rec_active = true;
-    c->rec_stored = c->rec_wanted;   // if they fit: the first step, which knows the substeps, finds out
+    // if they fit: the first step, which knows the substeps, finds out
+    c->rec_stored = c->rec_wanted && !c->rec_captured;
     c->rec_from_set = c->from_set_state;
     c->rec_nsub = -1;
     return DLO_OK;
 }
 
 // ------------------------------------------------------------------ step
+dlo_status note_capture(dlo_ctx* c) {
+    if (c->rec_captured) return DLO_OK;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const cudaError_t e = cudaStreamIsCapturing(c->stream, &cap);
+    if (e != cudaSuccess) return cuda_err(c, e, "capture status");
+    if (cap != cudaStreamCaptureStatusNone) {
+        c->rec_captured = true;
+        c->rec_stored = false;
+    }
+    return DLO_OK;
+}
+
 dlo_status launch_step(dlo_ctx* c, const float* actions, int frames, int substeps, float* x_frames, int frame0,
                        bool record) {
-    if (record && c->rec_stored) {
-        // A captured step stores no records: a graph may outlive the workspace, which a later
-        // backward may exchange.
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        const cudaError_t e = cudaStreamIsCapturing(c->stream, &cap);
-        if (e != cudaSuccess) return cuda_err(c, e, "capture status");
-        if (cap != cudaStreamCaptureStatusNone) c->rec_stored = false;
-    }
     // When the workspace of an earlier dlo_backward has room for the substep records of the whole
     // rollout, the forward stores them there as it steps and the backward does not step again to
     // get them.  Nothing is allocated for it: the first dlo_backward of a context recomputes, and
@@ -413,6 +418,8 @@ extern "C" dlo_status dlo_step(dlo_ctx* c, const float* actions, int frames, int
             return set_err(c, DLO_ERR_STATE, "step runs past the frames armed by dlo_begin_rollout");
         if (c->rec_nsub >= 0 && c->rec_nsub != substeps)
             return set_err(c, DLO_ERR_STATE, "substeps changed inside a recorded rollout");
+        dlo_status cs = note_capture(c);
+        if (cs != DLO_OK) return cs;
         c->rec_nsub = substeps;
         float* dst = c->rec_actions + (size_t)12 * c->B * c->rec_done;
         cudaError_t e = actions ? cudaMemcpyAsync(dst, actions, sizeof(float) * 12 * c->B * frames,

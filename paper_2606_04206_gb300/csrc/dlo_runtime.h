@@ -79,6 +79,7 @@ struct dlo_ctx {
     // substep records of the whole rollout, stored by the forward in the workspace that an earlier
     // dlo_backward left (bw_mem), while dlo_backward is the backward the caller uses
     bool rec_wanted = false;   // the last backward was dlo_backward, which reads them
+    bool rec_captured = false; // a recorded step is in a graph somewhere: nothing is stored any more
     bool rec_stored = false;   // this rollout's are being stored
     BwdPlan rec_plan;          // the plan they are laid out with
     dlo::StateRef ck{};
@@ -106,6 +107,11 @@ void backward_shapes(dlo_ctx* c);
 // rec_budget: bytes allowed for the chunk records of all classes (0 = the default); frames: the
 // rollout's (0 = not known: chunks are not cut to it)
 dlo_status bwd_plan(dlo_ctx* c, int force, int K, BwdPlan& out, size_t rec_budget = 0, int frames = 0);
+// Called by every recorded dlo_step (dlo_step_plain cannot be captured).  A graph that holds one writes the checkpoints and the actions anew
+// each time it is replayed, of which the context learns nothing: records that a later step stored
+// beside it would be of another rollout than the checkpoints, and the graph may outlive the
+// workspace.  So from the first captured recorded step on the backward recomputes.
+dlo_status note_capture(dlo_ctx* c);
 // Whether the plan's chunks hold the whole rollout and the present workspace has room for them.
 bool records_fit(const dlo_ctx* c, const BwdPlan& plan);
 // Enqueue the backward of size class k for the rods order[item0 .. item0 + n) on stream st,
