@@ -324,8 +324,8 @@ dlo_status dlo_loss(dlo_ctx* ctx, int kind, const float* x, const float* aux, in
  *   tau     edge softness in pixels (> 0)
  *   g, q, dL_dx as for dlo_loss (L = sum_b g_b Q_b)
  *   render  [B][n_cams][height][width] device floats: the soft silhouettes o (NULL = not wanted)
- * Grows a context workspace of B * height * width floats (one camera at a time), a few percent
- * of that for sums, and 48 bytes per vertex and camera.  Enqueued on the context's stream,
+ * Grows a context workspace to 5 bytes per rod and pixel (one camera at a time) and 208 bytes per
+ * vertex, whatever the number of cameras and whether or not the gradient is asked for.  Enqueued on the context's stream,
  * deterministic.  Errors: DLO_ERR_INVALID_ARG for a missing or unaligned array, no camera,
  * more than 2^24 pixels, tau <= 0, rods of more than 256 vertices or a context with strands
  * (dlo_scene.strand_start); DLO_ERR_OOM when the workspace cannot grow. */

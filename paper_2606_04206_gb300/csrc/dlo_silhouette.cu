@@ -9,8 +9,8 @@
 // edges whose reach box meets the tile are listed once (in order), then each thread composites
 // its pixel over the list and stores dL/d(occupancy) * prod_e (1 - sigma_e), the factor every
 // edge's gradient at that pixel shares.  Pass 2, a warp per edge: the lanes walk the pixels of the
-// edge's reach box and their sums give its endpoints' gradient.  A last launch adds up each
-// rod's tiles and, per vertex, its edges over the cameras.  Nothing is accumulated with atomics:
+// edge's reach box and their sums give its endpoints' gradient.  A last launch (one per group of four
+// cameras) adds up each rod's tiles and, per vertex, its edges over the cameras.  Nothing is accumulated with atomics:
 // the result is deterministic.  Bound by instruction issue: the exponentials and logarithms of
 // the pixels near a rope (at 256 x 256 a rope is near 1 pixel in 25).  One CTA per rod testing
 // every pixel against every edge took 2.87 ms for 64 rods of 64 vertices and 2 cameras of
@@ -28,6 +28,7 @@ constexpr int kTileW = 32, kTileH = 8;   // pixels per CTA of pass 1, one per th
 constexpr int kSilT = kTileW * kTileH;
 constexpr int kSilMaxV = 256;            // vertices per rod
 constexpr int kEdgesPerCta = 8;          // warps of pass 2
+constexpr int kCamsPerGroup = 4;         // cameras whose vertices and edge gradients are held at once
 // an edge is skipped at pixels farther than rho_e + kReach tau from it: sigma < 1.4e-11 there
 constexpr float kReach = 25.f;
 constexpr float kNear = 1e-3f;  // edges with an endpoint this close to the camera plane or behind it are not drawn
@@ -75,6 +76,7 @@ __device__ __forceinline__ float capsule_sd(float pu, float pv, float4 a, float4
 struct SilParams {
     const RodInfo* rods;
     int B, C, H, W, tiles_x, tiles, edge_ctas;
+    int c0, nc;                 // the group's first camera and their number
     float tau;
     const float4* X;
     const float* cams;
@@ -82,7 +84,8 @@ struct SilParams {
     const float* g;
     float *q, *render, *wbuf;   // wbuf: the current camera's pixel factors [B][H][W]
     float4* gx;
-    float4 *pv, *ge;            // projected vertices [C][V]; edge gradients [C][V][2] (an edge at its first vertex)
+    float4 *pv, *ge;            // projected vertices [nc][V]; edge gradients [nc][V][2] (an edge at its first vertex)
+    float4* acc;                // [V] the vertices' gradient over the groups before
     double* part;               // [B][tiles] sums of squared differences
     long long V;
 };
@@ -99,12 +102,12 @@ __device__ __forceinline__ float4 reach_box(float4 a, float4 b, float tau) {
     return make_float4(fminf(a.x, b.x) - m, fmaxf(a.x, b.x) + m, fminf(a.y, b.y) - m, fmaxf(a.y, b.y) + m);
 }
 
-// every vertex in every camera; one CTA per rod and camera
+// every vertex in the group's cameras; one CTA per rod and camera (c: the camera within the group)
 __global__ void __launch_bounds__(kSilMaxV) sil_project(SilParams P) {
     __shared__ Cam cm;
     const int c = blockIdx.y, i = threadIdx.x;
     const RodInfo R = P.rods[blockIdx.x];
-    load_cam(P, c, cm);
+    load_cam(P, P.c0 + c, cm);
     if (i < R.nv) P.pv[c * P.V + R.v0 + i] = project(cm, f3(P.X[R.v0 + i]), R.radius);
 }
 
@@ -157,7 +160,7 @@ __global__ void __launch_bounds__(kSilT) sil_pixels(SilParams P, int c) {
             const float sd = capsule_sd(px, py, a, b, 0.5f * (a.z + b.z), t, nu, nv);
             S -= softplus(-sd * inv_tau);
         }
-        const size_t HW = (size_t)P.H * P.W, p = (size_t)j * P.W + i, im = ((size_t)rod * P.C + c) * HW + p;
+        const size_t HW = (size_t)P.H * P.W, p = (size_t)j * P.W + i, im = ((size_t)rod * P.C + P.c0 + c) * HW + p;
         const float o = -expm1f(S);
         const float d = o - (P.masks[im] ? 1.f : 0.f);
         sq = (double)d * d;
@@ -170,7 +173,7 @@ __global__ void __launch_bounds__(kSilT) sil_pixels(SilParams P, int c) {
     if (lane == 0) red[w] = sq;
     __syncthreads();
     if (threadIdx.x == 0) {
-        double t = c ? P.part[blockIdx.x] : 0.0;   // the cameras follow one another on the stream
+        double t = P.c0 + c ? P.part[blockIdx.x] : 0.0;   // the cameras follow one another on the stream
         for (int k = 0; k < kSilT / 32; ++k) t += red[k];
         P.part[blockIdx.x] = t;
     }
@@ -181,7 +184,7 @@ __global__ void __launch_bounds__(32 * kEdgesPerCta) sil_edges(SilParams P, int 
     const int rod = blockIdx.x / P.edge_ctas, lane = threadIdx.x & 31;
     const int e = blockIdx.x % P.edge_ctas * kEdgesPerCta + (threadIdx.x >> 5);
     const RodInfo R = P.rods[rod];
-    load_cam(P, c, cm);
+    load_cam(P, P.c0 + c, cm);
     if (e >= R.ne) return;
     const float4* pv = P.pv + c * P.V + R.v0;
     const float4 a = pv[e], b = pv[e + 1 == R.nv ? 0 : e + 1], bx = reach_box(a, b, P.tau);
@@ -232,7 +235,8 @@ __global__ void __launch_bounds__(32 * kEdgesPerCta) sil_edges(SilParams P, int 
             lane == 0 ? to_world(a, gau, gav, 0.5f * gr) : to_world(b, gbu, gbv, 0.5f * gr);
 }
 
-// each rod's loss, and its vertices' gradient over the cameras
+// each rod's loss, and its vertices' gradient over the cameras (kept in acc until the last group, so
+// that the gradient may go where the positions are)
 __global__ void __launch_bounds__(kSilMaxV) sil_gather(SilParams P) {
     __shared__ double red[kSilMaxV];
     const int rod = blockIdx.x, i = threadIdx.x;
@@ -240,8 +244,8 @@ __global__ void __launch_bounds__(kSilMaxV) sil_gather(SilParams P) {
     const bool closed = R.flags & ROD_CLOSED;
     const int n = R.nv, ne = R.ne;
     if (P.gx && i < n) {
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int c = 0; c < P.C; ++c) {
+        float4 acc = P.c0 ? P.acc[R.v0 + i] : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int c = 0; c < P.nc; ++c) {
             const float4* ge = P.ge + 2 * (c * P.V + R.v0);
             if (closed || i < ne) {   // the edge that starts here
                 const float4 o = ge[2 * i];
@@ -252,9 +256,9 @@ __global__ void __launch_bounds__(kSilMaxV) sil_gather(SilParams P) {
                 acc = make_float4(acc.x + o.x, acc.y + o.y, acc.z + o.z, 0.f);
             }
         }
-        P.gx[R.v0 + i] = acc;
+        (P.c0 + P.nc < P.C ? P.acc : P.gx)[R.v0 + i] = acc;
     }
-    if (!P.q) return;
+    if (!P.q || P.c0 + P.nc < P.C) return;
     double t = 0.0;
     for (int k = i; k < P.tiles; k += kSilMaxV) t += P.part[(size_t)rod * P.tiles + k];
     red[i] = t;
@@ -303,11 +307,15 @@ extern "C" dlo_status dlo_loss_silhouette(dlo_ctx* c, const float* x, const floa
     P.render = render;
     P.gx = reinterpret_cast<float4*>(dL_dx);
     P.V = c->V;
-    // workspace: projected vertices, edge gradients, tile sums, one camera's pixel factors
-    const size_t nproj = (size_t)n_cams * c->V, ntile = (size_t)c->B * P.tiles;
-    const size_t pv_bytes = 16 * nproj, ge_bytes = P.gx ? 32 * nproj : 0, part_bytes = (8 * ntile + 15) & ~(size_t)15;
-    const size_t w_bytes = P.gx ? sizeof(float) * (size_t)c->B * height * width : 0;
-    const size_t need = pv_bytes + ge_bytes + part_bytes + w_bytes;
+    // Workspace: projected vertices and edge gradients of one group of cameras, the vertices'
+    // gradient, tile sums, one camera's pixel factors.  Its size follows from the rods and the
+    // number of pixels alone (no image has more tiles than an eighth of its pixels): a graph that
+    // holds a call keeps its workspace when a later call asks for the gradient as well, for
+    // other cameras or for another shape of as many pixels.
+    const size_t nproj = (size_t)kCamsPerGroup * c->V, ntile = (size_t)c->B * P.tiles, pixels = (size_t)height * width;
+    const size_t pv_bytes = 16 * nproj, ge_bytes = 32 * nproj, acc_bytes = 16 * (size_t)c->V;
+    const size_t part_bytes = (8 * (size_t)c->B * ((pixels + 7) / 8) + 15) & ~(size_t)15;
+    const size_t need = pv_bytes + ge_bytes + acc_bytes + part_bytes + sizeof(float) * (size_t)c->B * pixels;
     if (ntile >= ((size_t)1 << 31) || (size_t)c->B * P.edge_ctas >= ((size_t)1 << 31))
         return set_err(c, DLO_ERR_OOM, "too many rods and pixels for one silhouette call");
     if (need > c->sil_bytes) {
@@ -319,30 +327,29 @@ extern "C" dlo_status dlo_loss_silhouette(dlo_ctx* c, const float* x, const floa
     char* m = reinterpret_cast<char*>(c->sil_mem);
     P.pv = reinterpret_cast<float4*>(m);
     P.ge = reinterpret_cast<float4*>(m + pv_bytes);
-    P.part = reinterpret_cast<double*>(m + pv_bytes + ge_bytes);
-    P.wbuf = reinterpret_cast<float*>(m + pv_bytes + ge_bytes + part_bytes);
+    P.acc = reinterpret_cast<float4*>(m + pv_bytes + ge_bytes);
+    P.part = reinterpret_cast<double*>(m + pv_bytes + ge_bytes + acc_bytes);
+    P.wbuf = reinterpret_cast<float*>(m + pv_bytes + ge_bytes + acc_bytes + part_bytes);
     cudaError_t e = cudaSuccess;
-    for (int c0 = 0; c0 < n_cams && e == cudaSuccess; c0 += 65535) {   // the grid's second dimension
-        SilParams Q = P;
-        Q.cams += 16 * (size_t)c0;
-        Q.pv += (size_t)c0 * c->V;
-        sil_project<<<dim3(c->B, std::min(n_cams - c0, 65535)), kSilMaxV, 0, c->stream>>>(Q);
+    for (P.c0 = 0; P.c0 < n_cams && e == cudaSuccess; P.c0 += kCamsPerGroup) {
+        P.nc = std::min(n_cams - P.c0, kCamsPerGroup);
+        sil_project<<<dim3(c->B, P.nc), kSilMaxV, 0, c->stream>>>(P);
+        c->launches++;
         e = cudaGetLastError();
-        c->launches++;
-    }
-    for (int k = 0; k < n_cams && e == cudaSuccess; ++k) {
-        sil_pixels<<<(unsigned)ntile, kSilT, 0, c->stream>>>(P, k);
-        c->launches++;
-        if (P.gx) {
-            sil_edges<<<c->B * P.edge_ctas, 32 * kEdgesPerCta, 0, c->stream>>>(P, k);
+        for (int k = 0; k < P.nc && e == cudaSuccess; ++k) {
+            sil_pixels<<<(unsigned)ntile, kSilT, 0, c->stream>>>(P, k);
             c->launches++;
+            if (P.gx) {
+                sil_edges<<<c->B * P.edge_ctas, 32 * kEdgesPerCta, 0, c->stream>>>(P, k);
+                c->launches++;
+            }
+            e = cudaGetLastError();
         }
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) {
-        sil_gather<<<c->B, kSilMaxV, 0, c->stream>>>(P);
-        c->launches++;
-        e = cudaGetLastError();
+        if (e == cudaSuccess && (P.gx || P.c0 + P.nc == n_cams)) {
+            sil_gather<<<c->B, kSilMaxV, 0, c->stream>>>(P);
+            c->launches++;
+            e = cudaGetLastError();
+        }
     }
     return cuda_err(c, e, "silhouette launch");
 }
