@@ -229,6 +229,7 @@ __global__ void __launch_bounds__(kLT) loss_crossing(const RodInfo* rods, const 
     __shared__ unsigned longest;   // the longest edge squared (non-negative floats order like their bits)
     const int rod = blockIdx.x;
     const RodInfo R = rods[rod];
+    if (GRAD && R.nv > kLT) return;   // loss_crossing_long's
     const bool closed = R.flags & ROD_CLOSED;
     const int n = R.nv, ne = closed ? n : n - 1;
     for (int i = threadIdx.x; i < n; i += kLT) {
@@ -307,15 +308,17 @@ __device__ dualf gauss_pair_d(V3<dualf> p1, V3<dualf> p2, V3<dualf> p3, V3<dualf
 
 // The same sum and gradient for rods of more than 128 vertices, on dual numbers: the thread of
 // edge a evaluates Omega(a, b) for every b with the six coordinates of a's endpoints seeded in
-// turn.  Four times the work, kept there because the gradient is a sum of thousands of cancelling
-// pairs: the two evaluations agree to 1.1e-5 of it at 128 vertices but only to 2.5e-5 at 250
-// (each 1e-5 to 2e-5 from FP64), and results are to stay what they were to 2e-5.
+// turn.  Four times the work of the closed form, which holds one edge's gradient per thread.  (The
+// gradient is a sum of thousands of cancelling pairs: the two evaluations agree to 1.1e-5 of it at
+// 128 vertices and to 2.5e-5 at 250, each 1e-5 to 2e-5 from FP64.)  A rod's kernel follows from its own
+// size, so that its result does not depend on the batch it is in.
 __global__ void loss_crossing_long(const RodInfo* rods, const float4* X, const float* g, float* q, float4* gx) {
     __shared__ double sh[kLT];
     __shared__ float4 xs[kMaxV];
     __shared__ float4 ge0[kMaxV], ge1[kMaxV];   // d/d(first, second endpoint) of each edge's sum
     const int rod = blockIdx.x;
     const RodInfo R = rods[rod];
+    if (R.nv <= kLT) return;   // loss_crossing's
     const bool closed = R.flags & ROD_CLOSED;
     const int n = R.nv, ne = closed ? n : n - 1;
     for (int i = threadIdx.x; i < n; i += kLT) xs[i] = X[R.v0 + i];
@@ -508,12 +511,16 @@ extern "C" dlo_status dlo_loss(dlo_ctx* c, int kind, const float* x, const float
             loss_winding<<<c->B, kLT, 0, c->stream>>>(c->d_rods, X, reinterpret_cast<const float4*>(aux), g, q, GX);
             break;
         case DLO_LOSS_CROSSING:
-            if (GX && c->buckets.back().nv_max > kLT)
-                loss_crossing_long<<<c->B, kLT, 0, c->stream>>>(c->d_rods, X, g, q, GX);
-            else if (GX)
-                loss_crossing<true><<<c->B, kLT, 0, c->stream>>>(c->d_rods, X, g, q, GX);
-            else
+            if (!GX) {
                 loss_crossing<false><<<c->B, kLT, 0, c->stream>>>(c->d_rods, X, g, q, GX);
+                break;
+            }
+            if (c->buckets.front().nv_max <= kLT)
+                loss_crossing<true><<<c->B, kLT, 0, c->stream>>>(c->d_rods, X, g, q, GX);
+            if (c->buckets.back().nv_max > kLT) {
+                if (c->buckets.front().nv_max <= kLT) c->launches++;   // beside the one counted below
+                loss_crossing_long<<<c->B, kLT, 0, c->stream>>>(c->d_rods, X, g, q, GX);
+            }
             break;
         case DLO_LOSS_MINDIST:
             if (!aux) return set_err(c, DLO_ERR_INVALID_ARG, "the minimum distance needs an object centre per rod");
