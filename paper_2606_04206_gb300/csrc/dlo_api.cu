@@ -379,8 +379,7 @@ extern "C" dlo_status dlo_set_state(dlo_ctx* c, const float* x, const float* v, 
     P.S = c->S;
     P.GP0 = c->d_gp0;
     P.rest_mode = 0;
-    dlo_status st = cuda_err(c, launch_init(P, c->buckets.back().nv_max, c->stream), "init kernel");
-    c->launches++;
+    dlo_status st = cuda_err(c, init_rods(c, P), "init kernel");
     if (st != DLO_OK) return st;
     st = cuda_err(c, cudaMemsetAsync(c->d_status, 0, sizeof(unsigned) * c->B, c->stream), "status reset");
     c->from_set_state = true;

@@ -97,6 +97,10 @@ struct InitParams {
     StateRef S;
     const float* GP0;        // [B][2][12] initial gripper poses
     int rest_mode;           // 1: compute the rest twist from xin into rest[].z only
+    // the rods of up to 32 vertices (nv_small at most), when they take the kernel that packs several
+    // into a warp (n_small > 0)
+    const int* small;
+    int n_small, nv_small;
 };
 // nv_max: the largest size class of the batch (threads per block)
 cudaError_t launch_init(const InitParams& P, int nv_max, cudaStream_t st);

@@ -114,6 +114,22 @@ static dlo_status autotune_rods_per_cta(dlo_ctx* c) {
     return st;
 }
 
+// From this many rods of up to 32 vertices on they are packed into warps, when that saves warps: if none
+// has more than 16 vertices, or if longer rods in the batch would give each a longer rod's block.
+// dlo_set_state, a block per rod and packed: 1024 rods x 4 14.5 and 10.8 us, 65536 x 4 486 and
+// 64 us, 65536 x 16 484 and 240 us, 65536 x 32 483 and 482 us.
+static constexpr int kPackRods = 1024;
+
+cudaError_t init_rods(dlo_ctx* c, InitParams& P) {
+    const Bucket& bk = c->buckets.front();
+    const bool pack = bk.nv_max <= 32 && bk.n >= kPackRods && (bk.nv_top <= 16 || bk.n < c->B);
+    P.small = bk.d_order;
+    P.n_small = pack ? bk.n : 0;
+    P.nv_small = bk.nv_top;
+    c->launches += pack && bk.n < c->B ? 2 : 1;
+    return launch_init(P, c->buckets.back().nv_max, c->stream);
+}
+
 dlo_status runtime_allocate(dlo_ctx* c, const std::vector<RodInfo>& rods, const std::vector<float4>& kin,
                             const std::vector<float2>& mass, const std::vector<float2>& es,
                             const std::vector<float4>& rest, const std::vector<float>& gp0,
@@ -164,6 +180,7 @@ dlo_status runtime_allocate(dlo_ctx* c, const std::vector<RodInfo>& rods, const 
         bk.nv_max = size_class_at(k);
         bk.contact = c->opt.self_contact != 0;
         bk.n = (int)ids.size();
+        for (int b : ids) bk.nv_top = std::max(bk.nv_top, rods[b].nv);
         bk.d_order = alloc_up(c, ids, st);
         if (st != DLO_OK) return st;
         // rods per CTA: the count (within the thread budget) that keeps the most rods resident;
@@ -209,11 +226,10 @@ dlo_status runtime_allocate(dlo_ctx* c, const std::vector<RodInfo>& rods, const 
     P.S = c->S;
     P.GP0 = c->d_gp0;
     P.rest_mode = 1;
-    st = cuda_err(c, launch_init(P, c->buckets.back().nv_max, c->stream), "rest init");
+    st = cuda_err(c, init_rods(c, P), "rest init");
     if (st != DLO_OK) return st;
     P.rest_mode = 0;
-    st = cuda_err(c, launch_init(P, c->buckets.back().nv_max, c->stream), "state init");
-    c->launches += 2;
+    st = cuda_err(c, init_rods(c, P), "state init");
     if (st == DLO_OK && c->opt.warps_per_cta == 0) {
         // measured autotune of rods per CTA; then the rest state is set again (positions
         // re-uploaded, frames, velocities and poses re-initialised, status cleared)
@@ -223,8 +239,7 @@ dlo_status runtime_allocate(dlo_ctx* c, const std::vector<RodInfo>& rods, const 
                                              c->stream), "rest positions");
         if (st == DLO_OK)
             st = cuda_err(c, cudaMemsetAsync(c->d_status, 0, sizeof(unsigned) * c->B, c->stream), "status reset");
-        if (st == DLO_OK) st = cuda_err(c, launch_init(P, c->buckets.back().nv_max, c->stream), "state init");
-        c->launches++;
+        if (st == DLO_OK) st = cuda_err(c, init_rods(c, P), "state init");
     }
     c->from_set_state = true;
     if (st == DLO_OK) st = cuda_err(c, cudaStreamSynchronize(c->stream), "create");

@@ -7,6 +7,7 @@
 #include "dlo_internal.h"
 
 namespace dlo {
+struct InitParams;
 constexpr int kMaxVerts = 256;
 
 // Rods of one shared-memory size class, launched together by the persistent kernels.
@@ -17,6 +18,7 @@ struct Bucket {
     int* d_order = nullptr; // rod ids by decreasing cost (vertices x substeps)
     int warps = 0;          // rods in flight per CTA of the forward kernel
     int grid = 0;           // persistent CTAs
+    int nv_top = 0;         // the largest rod of the class
     // rods per CTA and CTAs per SM of the backward's kernels (0: not possible)
     int rec_w = 0, rec_nb = 0, rev_w = 0, rev_nb = 0;
 };
@@ -107,6 +109,8 @@ void backward_shapes(dlo_ctx* c);
 // rec_budget: bytes allowed for the chunk records of all classes (0 = the default); frames: the
 // rollout's (0 = not known: chunks are not cut to it)
 dlo_status bwd_plan(dlo_ctx* c, int force, int K, BwdPlan& out, size_t rec_budget = 0, int frames = 0);
+// launch_init over the context's rods
+cudaError_t init_rods(dlo_ctx* c, dlo::InitParams& P);
 // Called by every recorded dlo_step (dlo_step_plain cannot be captured).  A graph that holds one writes the checkpoints and the actions anew
 // each time it is replayed, of which the context learns nothing: records that a later step stored
 // beside it would be of another rollout than the checkpoints, and the graph may outlive the
