@@ -8,8 +8,8 @@
 // chunk's frames from their start state storing every substep's records, then rev_kernel
 // reverses them (dlo_bwd_kernel.cuh).  C is a multiple of K when C >= K, so that every chunk
 // starts at a checkpoint; otherwise the frame-start states of each segment are stored first.
-// When one chunk holds the whole rollout, the forward stores the records itself and rec_kernel
-// does not run.
+// When one chunk holds the whole rollout and an earlier call left a workspace with room for it, the
+// forward stores the records there and rec_kernel does not run.
 #include <algorithm>
 #include <cstring>
 #include <vector>

@@ -4,8 +4,9 @@
 // for each segment in reverse, re-running the forward simulation before back-propagating.
 // Here the checkpoints live in HBM (written by the forward kernel every K frames) and the
 // rollout is reversed in chunks of frames, last first, by two persistent kernels per chunk:
-//   rec_kernel   forward-like (several rods per CTA): re-runs the chunk's frames from their
-//                start state and stores every substep's records in HBM: its start state, the
+//   rec_kernel   forward-like (a rod per CTA, see best_shape; not run when the forward stored the
+//                records): re-runs the chunk's frames from their start state and stores every
+//                substep's records in HBM: its start state, the
 //                velocity before rigid contact, the displacement before friction, one record
 //                per edge and projection iteration (direction and target / length), the
 //                displacements before each contact sweep and the first iteration's pair data;
@@ -760,6 +761,9 @@ __device__ __forceinline__ void reverse_substep(const BwdParams& P, const RodInf
 // of 11.6 ms.  Above, two CTAs: with one (255 registers, no spills) 1024 bands x 200 in contact
 // take 5.8 instead of 4.8 ms.
 __host__ __device__ constexpr int rev_min_ctas(int NV) { return NV <= 128 ? 384 / NV : 2; }
+static_assert(rev_min_ctas(256) * (RevSmem<256, true>::kBytes + 1024) <= 228 * 1024 &&
+                  rev_min_ctas(128) * (RevSmem<128, true>::kBytes + 1024) <= 228 * 1024,
+              "as many rods as registers allow fit the SM's shared memory (1 KB of it reserved per CTA)");
 
 // ------------------------------------------------------------------ the recompute kernel
 // Persistent, forward-like (a group of threads per rod, state in shared memory).  RECORD false:

@@ -75,8 +75,8 @@ struct FwdParams {
     StateRef ck;
     long long ck_strideV, ck_strideE, ck_strideB;
     int ck_every, ck_count;
-    // substep records for the adjoint, when the whole rollout's fit: [n_order][rollout frames][frame
-    // record], or null (the adjoint recomputes them)
+    // substep records for the adjoint, in its workspace when that holds the whole rollout's:
+    // [n_order][rollout frames][frame record], or null (the adjoint recomputes them)
     float4* R3;
     size_t r3_rod;
     int nsub_max;

@@ -63,14 +63,16 @@ int rev_blocks_per_sm(int nv_max, bool contact, int warps);
 // Substeps whose gripper blocks (256 B each) are formed together.
 constexpr int kPoseBatch = 8;
 // Shared memory of one rod: the arrays above, 256 B of group-reduction scratch, and the gripper
-// blocks, two poses and the actions (240 B), in whole 256 B.
+// blocks, the pose and the actions (144 B), in whole 256 B.
 __host__ __device__ constexpr size_t rod_smem_bytes(int NV, bool contact) {
     return warp_smem_bytes(NV, contact) + 512 + 256 * kPoseBatch;
 }
 
 // Rod size classes: a rod of nv vertices runs in the kernels instantiated for the smallest
-// class that holds it (shared memory is sized per class; 192 and 224 let two rods of up to
-// 224 vertices share an SM in the backward, where a 256-vertex rod needs 124 KB).
+// class that holds it: threads, shared memory, records and candidate slots are sized per class.  In the
+// reverse two rods of any class above 128 share an SM; 192 and 224 leave a thread more registers
+// and move fewer record bytes than 256 does.  608 ropes, 2 frames with their gradient: x 150
+// 0.55 ms (0.64 in class 256), x 180 0.98 (1.09), x 200 1.09 (1.11), x 224 1.16 (1.18).
 constexpr int kNumSizeClasses = 6;
 __host__ __device__ constexpr int size_class_at(int k) {
     return k == 0 ? 32 : k == 1 ? 64 : k == 2 ? 128 : k == 3 ? 192 : k == 4 ? 224 : 256;

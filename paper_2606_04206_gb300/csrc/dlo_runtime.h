@@ -15,7 +15,7 @@ struct Bucket {
     int nv_max = 0;
     bool contact = false;
     int n = 0;              // rods in the bucket
-    int* d_order = nullptr; // rod ids by decreasing cost (vertices x substeps)
+    int* d_order = nullptr; // rod ids by decreasing cost (vertices x substeps x kind)
     int warps = 0;          // rods in flight per CTA of the forward kernel
     int grid = 0;           // persistent CTAs
     int nv_top = 0;         // the largest rod of the class

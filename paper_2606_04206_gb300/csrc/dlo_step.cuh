@@ -298,16 +298,14 @@ struct Smem {
     float* red;
     // gripper block (read by every thread of the rod with broadcasts):
     //   fp  [24] pose at the start of the frame being stepped, per gripper p (3), R (9) row major
-    //   f0  [24] a second frame-start pose (the frame the backward reverses)
     //   sp  [kPoseBatch][64] per substep and gripper (32): p0 (3), p1 (3), R0 (9), R1 (9), vp (3), w (3),
     //       grip_bound (1)
     //   act [12] the frame's actions
-    float *fp, *f0, *sp, *act;
+    float *fp, *sp, *act;
     __device__ Smem(float4* base) {
         red = reinterpret_cast<float*>(base + warp_smem_bytes(NV, CONTACT) / 16);
         fp = red + 64;
-        f0 = fp + 24;
-        sp = f0 + 24;
+        sp = fp + 24;
         act = sp + 64 * kPoseBatch;
         X = base;
         X0 = base + NV;
