@@ -305,6 +305,18 @@ dlo_status bwd_plan(dlo_ctx* c, int force, int K, BwdPlan& out, size_t rec_budge
     return DLO_OK;
 }
 
+dlo_status grow_workspace(dlo_ctx* c, size_t bytes, const char* what) {
+    if (bytes <= c->bw_bytes) return DLO_OK;
+    if (c->bw_mem) {
+        const cudaError_t e = cudaStreamSynchronize(c->stream);
+        if (e != cudaSuccess) return cuda_err(c, e, "stream");
+        dev_free(c, c->bw_mem);
+    }
+    c->bw_mem = dev_alloc(c, bytes);
+    c->bw_bytes = c->bw_mem ? bytes : 0;
+    return c->bw_mem ? DLO_OK : set_err(c, DLO_ERR_OOM, what);
+}
+
 bool records_fit(const dlo_ctx* c, const BwdPlan& plan) {
     for (int C : plan.C)
         if (C < c->rec_frames) return false;
@@ -429,12 +441,8 @@ extern "C" dlo_status dlo_backward(dlo_ctx* c, const float* dL_dx_T, const float
     if (pst != DLO_OK) return pst;
     const bool stored = c->rec_stored && records_fit(c, plan);
     c->rec_wanted = true;
-    if (plan.bytes > c->bw_bytes) {
-        dev_free(c, c->bw_mem);
-        c->bw_mem = dev_alloc(c, plan.bytes);
-        c->bw_bytes = c->bw_mem ? plan.bytes : 0;
-        if (!c->bw_mem) return set_err(c, DLO_ERR_OOM, "backward workspace allocation failed");
-    }
+    pst = grow_workspace(c, plan.bytes, "backward workspace allocation failed");
+    if (pst != DLO_OK) return pst;
     char* p = reinterpret_cast<char*>(c->bw_mem);
     float4* gtb0 = reinterpret_cast<float4*>(p);
     float4* gd1b0 = gtb0 + c->Et;

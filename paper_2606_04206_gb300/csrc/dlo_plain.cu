@@ -1239,12 +1239,8 @@ extern "C" dlo_status dlo_backward_plain(dlo_ctx* c, const float* dL_dx_T, const
     const size_t bytes = 16 * f4 + sizeof(double) * 5 * B + sizeof(float) * (size_t)B * (12 + 12 + 36 + 72 + 24 + 24) +
                          2 * 16 * nE + 4096;
     c->rec_wanted = c->rec_stored = false;   // this takes over the workspace the records are in
-    if (bytes > c->bw_bytes) {
-        dev_free(c, c->bw_mem);
-        c->bw_mem = dev_alloc(c, bytes);
-        c->bw_bytes = c->bw_mem ? bytes : 0;
-        if (!c->bw_mem) return set_err(c, DLO_ERR_OOM, "plain backward workspace allocation failed");
-    }
+    st = grow_workspace(c, bytes, "plain backward workspace allocation failed");
+    if (st != DLO_OK) return st;
     char* m = reinterpret_cast<char*>(c->bw_mem);
     auto take4 = [&](size_t n) {
         float4* q = reinterpret_cast<float4*>(m);

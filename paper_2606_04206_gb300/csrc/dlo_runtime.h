@@ -116,6 +116,10 @@ cudaError_t init_rods(dlo_ctx* c, dlo::InitParams& P);
 // beside it would be of another rollout than the checkpoints, and the graph may outlive the
 // workspace.  So from the first captured recorded step on the backward recomputes.
 dlo_status note_capture(dlo_ctx* c);
+// bw_mem of at least `bytes` (its contents are lost when it grows; what: the error's text).  A step
+// may still be storing records in the old one, and the caller's allocator may hand it to another
+// stream at once: it is given back after the context's stream has finished.
+dlo_status grow_workspace(dlo_ctx* c, size_t bytes, const char* what);
 // Whether the plan's chunks hold the whole rollout and the present workspace has room for them.
 bool records_fit(const dlo_ctx* c, const BwdPlan& plan);
 // Enqueue the backward of size class k for the rods order[item0 .. item0 + n) on stream st,

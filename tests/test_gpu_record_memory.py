@@ -17,7 +17,7 @@ class Counting:
     """Allocations through torch, with the bytes that are out."""
 
     def __init__(self):
-        self.size, self.live = {}, 0
+        self.size, self.live, self.on_free = {}, 0, None
 
     def alloc(self, nbytes):
         ptr = torch.cuda.caching_allocator_alloc(nbytes, torch.cuda.current_device(), torch.cuda.current_stream())
@@ -26,6 +26,8 @@ class Counting:
         return ptr
 
     def free(self, ptr):
+        if self.on_free:
+            self.on_free()
         self.live -= self.size.pop(ptr)
         torch.cuda.caching_allocator_delete(ptr)
 
@@ -163,3 +165,21 @@ def test_other_backwards_hold_and_write_no_records(how):
     for k in out:
         rel, cos = grad_agreement(out[k].double().cpu().numpy(), ref[k].double().cpu().numpy())
         assert rel <= 1e-3 and cos >= 0.999, k
+
+
+def test_the_workspace_is_given_back_when_nothing_writes_it():
+    """A rollout that stores its records and is abandoned, then a longer one whose backward needs a
+    larger workspace: the old one goes back to the caller's allocator after the steps have ended."""
+    p = inputs.small_case("diff", n_rods=1500, n=60, frames=8)
+    r = Rollouts(p)
+    r.forward(4)
+    r.backward(recomputes=True)
+    r.sim.begin_rollout(4)
+    r.sim.step(actions_dev(p, 0, 4), 4)
+    r.sim.begin_rollout(8)
+    acts, busy = actions_dev(p), []
+    r.mem.on_free = lambda: busy.append(not torch.cuda.current_stream().query())
+    r.sim.step(acts, 8)
+    r.sim.backward(*r.w)
+    r.mem.on_free = None
+    assert busy == [False]
